@@ -1,10 +1,8 @@
 // Particle-side kernels of the PM step:
 //   * cell-count scans of the cell-ordered codec (Sec. 2.4): count byte with
 //     the 255 escape, CSR offsets, escape-list compaction;
-//   * decompress / compress of one species (Sec. 2.4);
-//   * CIC deposit (Sec. 2.3 density_interpolation; Sec. 2.1 footnote: both
-//     species, their own masses, one mesh), float32 or int64 fixed point;
-//   * CIC force interpolation, kick and drift;
+//   * compress of one species (Sec. 2.4; decompress and the kernels over
+//     float particles are in plain.cu);
 //   * the fused step passes that read the codes directly: decode + deposit
 //     (binned in shared memory per block of compression cells), and decode +
 //     interpolate + kick + drift + recompress (count pass, then scatter pass
@@ -12,6 +10,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "cic.cuh"
 #include "particles.cuh"
 
 namespace pm {
@@ -308,217 +307,6 @@ cudaError_t scan_counts2(const uint32_t* counts0, const uint32_t* counts1, int64
 // Partials of one species; the two-species scans use twice this.
 size_t scan_partial_bytes(int64_t ncell) { return sizeof(V2) * (size_t)(scan_blocks(ncell) + 1); }
 
-// ------------------------------------------------- plain per-particle -----
-
-// Cell of stream index p: the last c with off[c] <= p (binary search over all cells).
-__device__ __forceinline__ int64_t find_cell(const int64_t* off, int64_t ncell, int64_t p) {
-  int64_t lo = 0, hi = ncell - 1;
-  while (lo < hi) {
-    int64_t mid = (lo + hi + 1) >> 1;
-    if (off[mid] <= p) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
-
-__global__ void k_decompress(PCodes in, const int64_t* off, Geo g, float* x, float* v) {
-  const float pscale = (float)g.rcmp / 256.0f;
-  const float vm = *in.vmax;
-  const int half = in.vel16 ? 32768 : 128;
-  const float step = __fmul_rn(vm, 1.0f / (float)half);
-  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < in.n; p += (int64_t)gridDim.x * blockDim.x) {
-    int64_t c = find_cell(off, g.ncell, p);
-    int cx = (int)(c % g.ncmp), cy = (int)((c / g.ncmp) % g.ncmp), cz = (int)(c / ((int64_t)g.ncmp * g.ncmp));
-    int q[3], qv[3];
-    unpack_pos(in.pos[p], q);
-    load_vel(in.vel, in.vel16, p, qv);
-    x[3 * p + 0] = decode_pos(cx, q[0], pscale);
-    x[3 * p + 1] = decode_pos(cy, q[1], pscale);
-    x[3 * p + 2] = decode_pos(cz, q[2], pscale);
-#pragma unroll
-    for (int d = 0; d < 3; ++d) v[3 * p + d] = decode_vel(qv[d], half, step);
-  }
-}
-
-// Float32 CIC deposit into global meshes with atomics.
-__device__ __forceinline__ void cic_axis(float x, int n, int& i0, int& i1, float& w0, float& w1) {
-  float f = floorf(x);
-  w1 = __fsub_rn(x, f);
-  w0 = __fsub_rn(1.0f, w1);
-  i0 = (int)f;
-  if (i0 >= n) i0 -= n;
-  if (i0 < 0) i0 += n;
-  i1 = (i0 + 1 == n) ? 0 : i0 + 1;
-}
-
-__global__ void k_deposit_global(const float* x, int64_t n, float m, Geo g, float* rho_c, float* rho_f) {
-  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
-    float px = x[3 * p], py = x[3 * p + 1], pz = x[3 * p + 2];
-    int ix[2], iy[2], iz[2];
-    float wx[2], wy[2], wz[2];
-    cic_axis(px, g.nf, ix[0], ix[1], wx[0], wx[1]);
-    cic_axis(py, g.nf, iy[0], iy[1], wy[0], wy[1]);
-    cic_axis(pz, g.nf, iz[0], iz[1], wz[0], wz[1]);
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      int dx = c & 1, dy = (c >> 1) & 1, dz = c >> 2;
-      float w = __fmul_rn(__fmul_rn(wx[dx], wy[dy]), wz[dz]);
-      atomicAdd(&rho_f[((int64_t)iz[dz] * g.nf + iy[dy]) * g.nf + ix[dx]], __fmul_rn(m, w));
-    }
-    if (rho_c) {
-      float s = 1.0f / (float)g.rc;
-      cic_axis(__fmul_rn(px, s), g.nc, ix[0], ix[1], wx[0], wx[1]);
-      cic_axis(__fmul_rn(py, s), g.nc, iy[0], iy[1], wy[0], wy[1]);
-      cic_axis(__fmul_rn(pz, s), g.nc, iz[0], iz[1], wz[0], wz[1]);
-#pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        int dx = c & 1, dy = (c >> 1) & 1, dz = c >> 2;
-        float w = __fmul_rn(__fmul_rn(wx[dx], wy[dy]), wz[dz]);
-        atomicAdd(&rho_c[((int64_t)iz[dz] * g.nc + iy[dy]) * g.nc + ix[dx]], __fmul_rn(m, w));
-      }
-    }
-  }
-}
-
-// Periodic CIC deposit of nw per-particle weights (w[p nw + c], c < nw <= 4)
-// onto nw fine meshes out[c][nf^3] (float32, the mesh convention of the
-// deposit above): number and momentum densities for the power spectra of
-// the compression study.
-__global__ void k_deposit_weights(const float* x, int64_t n, const float* w, int nw, Geo g, float* out) {
-  const int64_t nf3 = (int64_t)g.nf * g.nf * g.nf;
-  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
-    int ix[2], iy[2], iz[2];
-    float wx[2], wy[2], wz[2];
-    cic_axis(x[3 * p], g.nf, ix[0], ix[1], wx[0], wx[1]);
-    cic_axis(x[3 * p + 1], g.nf, iy[0], iy[1], wy[0], wy[1]);
-    cic_axis(x[3 * p + 2], g.nf, iz[0], iz[1], wz[0], wz[1]);
-    float q[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int c = 0; c < nw; ++c) q[c] = w[p * nw + c];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const int dx = k & 1, dy = (k >> 1) & 1, dz = k >> 2;
-      const float wt = __fmul_rn(__fmul_rn(wx[dx], wy[dy]), wz[dz]);
-      float* cell = out + ((int64_t)iz[dz] * g.nf + iy[dy]) * g.nf + ix[dx];
-      for (int c = 0; c < nw; ++c) atomicAdd(cell + c * nf3, __fmul_rn(q[c], wt));
-    }
-  }
-}
-
-// Fixed point: weights a1 = floor(f 2^20), mass split hi = (M a1 + 2^19) >> 20, lo = M - hi.
-__device__ __forceinline__ void fixed_axis(float x, int n, int& i0, int& i1, long long& a1) {
-  float f = floorf(x);
-  float fr = __fsub_rn(x, f);
-  a1 = (long long)__fmul_rn(fr, 1048576.0f);
-  i0 = (int)f;
-  if (i0 >= n) i0 -= n;
-  if (i0 < 0) i0 += n;
-  i1 = (i0 + 1 == n) ? 0 : i0 + 1;
-}
-__device__ __forceinline__ void fixed_split(long long M, long long a1, long long& lo, long long& hi) {
-  hi = (M * a1 + (1LL << 19)) >> 20;
-  lo = M - hi;
-}
-__device__ __forceinline__ void fixed_corners(long long M, const long long a[3], long long out[8]) {
-  long long mx[2], my[2], mz[2];
-  fixed_split(M, a[0], mx[0], mx[1]);
-#pragma unroll
-  for (int dx = 0; dx < 2; ++dx) {
-    fixed_split(mx[dx], a[1], my[0], my[1]);
-#pragma unroll
-    for (int dy = 0; dy < 2; ++dy) {
-      fixed_split(my[dy], a[2], mz[0], mz[1]);
-      out[dx + 2 * dy + 0] = mz[0];
-      out[dx + 2 * dy + 4] = mz[1];
-    }
-  }
-}
-
-__global__ void k_deposit_fixed_global(const float* x, int64_t n, long long M, Geo g, long long* rho_c,
-                                       long long* rho_f) {
-  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
-    float pp[3] = {x[3 * p], x[3 * p + 1], x[3 * p + 2]};
-    for (int level = 0; level < 2; ++level) {
-      long long* rho = level == 0 ? rho_f : rho_c;
-      if (!rho) continue;
-      int nn = level == 0 ? g.nf : g.nc;
-      float s = level == 0 ? 1.0f : 1.0f / (float)g.rc;
-      int i0[3], i1[3];
-      long long a1[3];
-#pragma unroll
-      for (int d = 0; d < 3; ++d) fixed_axis(__fmul_rn(pp[d], s), nn, i0[d], i1[d], a1[d]);
-      long long terms[8];
-      fixed_corners(M, a1, terms);
-#pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        int dx = c & 1, dy = (c >> 1) & 1, dz = c >> 2;
-        int gx = dx ? i1[0] : i0[0], gy = dy ? i1[1] : i0[1], gz = dz ? i1[2] : i0[2];
-        atomicAdd(reinterpret_cast<unsigned long long*>(&rho[((int64_t)gz * nn + gy) * nn + gx]),
-                  (unsigned long long)terms[c]);
-      }
-    }
-  }
-}
-
-// CIC gather of a [3][n^3] field; fixed operation order so recomputation is bit-identical.
-__device__ __forceinline__ void gather(const float* __restrict__ F, int n, float px, float py, float pz, float a[3]) {
-  int ix[2], iy[2], iz[2];
-  float wx[2], wy[2], wz[2];
-  cic_axis(px, n, ix[0], ix[1], wx[0], wx[1]);
-  cic_axis(py, n, iy[0], iy[1], wy[0], wy[1]);
-  cic_axis(pz, n, iz[0], iz[1], wz[0], wz[1]);
-  const int64_t n3 = (int64_t)n * n * n;
-  float s0 = 0.f, s1 = 0.f, s2 = 0.f;
-#pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    int dx = c & 1, dy = (c >> 1) & 1, dz = c >> 2;
-    float w = __fmul_rn(__fmul_rn(wx[dx], wy[dy]), wz[dz]);
-    int64_t idx = ((int64_t)iz[dz] * n + iy[dy]) * n + ix[dx];
-    s0 = __fmaf_rn(w, __ldg(F + idx), s0);
-    s1 = __fmaf_rn(w, __ldg(F + n3 + idx), s1);
-    s2 = __fmaf_rn(w, __ldg(F + 2 * n3 + idx), s2);
-  }
-  a[0] = s0;
-  a[1] = s1;
-  a[2] = s2;
-}
-
-__device__ __forceinline__ void accel_at(const Geo& g, const float* acc_c, const float* acc_f, float px, float py,
-                                         float pz, float a[3]) {
-  gather(acc_f, g.nf, px, py, pz, a);
-  if (g.two) {
-    float s = 1.0f / (float)g.rc;
-    float b[3];
-    gather(acc_c, g.nc, __fmul_rn(px, s), __fmul_rn(py, s), __fmul_rn(pz, s), b);
-    a[0] = __fadd_rn(b[0], a[0]);
-    a[1] = __fadd_rn(b[1], a[1]);
-    a[2] = __fadd_rn(b[2], a[2]);
-  }
-}
-
-// The same CIC gather from a shared-memory copy S[3][fz][fy][fx] of the mesh
-// region whose cell (0,0,0) is the global cell (ox, oy, oz); identical
-// arithmetic and order to gather(), so both give the same bits.
-__device__ __forceinline__ void gather_local(const float* S, int fx, int fy, int fz, int ox, int oy, int oz, float px,
-                                             float py, float pz, float a[3]) {
-  float fl[3] = {floorf(px), floorf(py), floorf(pz)};
-  float w1[3] = {__fsub_rn(px, fl[0]), __fsub_rn(py, fl[1]), __fsub_rn(pz, fl[2])};
-  float w0[3] = {__fsub_rn(1.0f, w1[0]), __fsub_rn(1.0f, w1[1]), __fsub_rn(1.0f, w1[2])};
-  const int lx = (int)fl[0] - ox, ly = (int)fl[1] - oy, lz = (int)fl[2] - oz;
-  const int plane = fx * fy * fz;
-  float s0 = 0.f, s1 = 0.f, s2 = 0.f;
-#pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    int dx = c & 1, dy = (c >> 1) & 1, dz = c >> 2;
-    float w = __fmul_rn(__fmul_rn(dx ? w1[0] : w0[0], dy ? w1[1] : w0[1]), dz ? w1[2] : w0[2]);
-    int idx = ((lz + dz) * fy + (ly + dy)) * fx + (lx + dx);
-    s0 = __fmaf_rn(w, S[idx], s0);
-    s1 = __fmaf_rn(w, S[plane + idx], s1);
-    s2 = __fmaf_rn(w, S[2 * plane + idx], s2);
-  }
-  a[0] = s0;
-  a[1] = s1;
-  a[2] = s2;
-}
-
 // The same CIC gather when the lower corner's local index (lx, ly, lz) and the
 // upper weights w1 are already known; same weights and order as gather().
 __device__ __forceinline__ void gather_idx(const float* S, int fx, int fy, int fz, int lx, int ly, int lz,
@@ -578,51 +366,6 @@ __device__ __forceinline__ void gather_strided(const float* S, RegionStrides st,
   a[0] = s0;
   a[1] = s1;
   a[2] = s2;
-}
-
-__device__ __forceinline__ float wrap_pos(float x, float nf) {
-  if (x < 0.f) x = __fadd_rn(x, nf);
-  if (x >= nf) x = __fsub_rn(x, nf);
-  if (!(x >= 0.f && x < nf)) {      // moved more than one box length, or rounding onto nf
-    x = __fsub_rn(x, __fmul_rn(nf, floorf(__fdiv_rn(x, nf))));
-    if (!(x >= 0.f && x < nf)) x = 0.f;
-  }
-  return x;
-}
-
-// v' = v + c_k a ; x' = wrap(x + c_d v')
-__device__ __forceinline__ void kick_drift(float x[3], float v[3], const float a[3], float ck, float cd, float nf) {
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    v[d] = __fmaf_rn(ck, a[d], v[d]);
-    x[d] = wrap_pos(__fmaf_rn(cd, v[d], x[d]), nf);
-  }
-}
-
-__global__ void k_interpolate(const float* x, int64_t n, Geo g, const float* acc_c, const float* acc_f, float* a) {
-  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
-    float r[3];
-    accel_at(g, acc_c, acc_f, x[3 * p], x[3 * p + 1], x[3 * p + 2], r);
-    a[3 * p] = r[0];
-    a[3 * p + 1] = r[1];
-    a[3 * p + 2] = r[2];
-  }
-}
-
-__global__ void k_kick_drift(float* x, float* v, int64_t n, Geo g, const float* acc_c, const float* acc_f, float ck,
-                             float cd) {
-  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
-    float xx[3] = {x[3 * p], x[3 * p + 1], x[3 * p + 2]};
-    float vv[3] = {v[3 * p], v[3 * p + 1], v[3 * p + 2]};
-    float a[3];
-    accel_at(g, acc_c, acc_f, xx[0], xx[1], xx[2], a);
-    kick_drift(xx, vv, a, ck, cd, (float)g.nf);
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      x[3 * p + d] = xx[d];
-      v[3 * p + d] = vv[d];
-    }
-  }
 }
 
 // ------------------------------------------------ recompress passes ------
@@ -846,30 +589,6 @@ __device__ __forceinline__ void smem_acc(float* a, float v) { atomicAdd(a, v); }
 __device__ __forceinline__ void global_add(float* a, float v) { atomicAdd(a, v); }
 __device__ __forceinline__ void global_add(long long* a, long long v) {
   atomicAdd(reinterpret_cast<unsigned long long*>(a), (unsigned long long)v);
-}
-
-// Sums v[] over runs of consecutive lanes holding the same key (the particle
-// stream is cell ordered, so a warp's particles form few runs); returns true
-// on the last lane of each run, which then holds the run's totals.
-template <int K, typename T>
-__device__ __forceinline__ bool run_reduce(unsigned key, T (&v)[K]) {
-  const unsigned FULL = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
-  const unsigned prev = __shfl_up_sync(FULL, key, 1);
-  const unsigned next = __shfl_down_sync(FULL, key, 1);
-  const bool head = lane == 0 || prev != key;
-  const bool tail = lane == 31 || next != key;
-  const unsigned heads = __ballot_sync(FULL, head);
-  const int start = 31 - __clz(heads & (FULL >> (31 - lane)));
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      T u = __shfl_up_sync(FULL, v[k], o);
-      if (lane - start >= o) v[k] += u;
-    }
-  }
-  return tail;
 }
 
 // Compile-time cell-block shape: RX_ > 0 fixes RX, RY, RZ and the fine cells per
@@ -1617,52 +1336,6 @@ static int grid_for(int64_t n, int threads) {
   int64_t b = (n + threads - 1) / threads;
   if (b > 152 * 32) b = 152 * 32;
   return (int)(b < 1 ? 1 : b);
-}
-
-cudaError_t launch_decompress(const PCodes& in, const int64_t* off, const Geo& g, float* x, float* v, cudaStream_t st) {
-  if (in.n == 0) return cudaSuccess;
-  k_decompress<<<grid_for(in.n, 256), 256, 0, st>>>(in, off, g, x, v);
-  note_launches(1);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_deposit(const float* x, int64_t n, float m, const Geo& g, float* rho_c, float* rho_f, cudaStream_t st) {
-  if (n == 0) return cudaSuccess;
-  k_deposit_global<<<grid_for(n, 256), 256, 0, st>>>(x, n, m, g, rho_c, rho_f);
-  note_launches(1);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_deposit_weights(const float* x, int64_t n, const float* w, int nw, const Geo& g, float* out,
-                                  cudaStream_t st) {
-  if (n == 0) return cudaSuccess;
-  k_deposit_weights<<<grid_for(n, 256), 256, 0, st>>>(x, n, w, nw, g, out);
-  note_launches(1);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_deposit_fixed(const float* x, int64_t n, long long M, const Geo& g, long long* rho_c,
-                                 long long* rho_f, cudaStream_t st) {
-  if (n == 0) return cudaSuccess;
-  k_deposit_fixed_global<<<grid_for(n, 256), 256, 0, st>>>(x, n, M, g, rho_c, rho_f);
-  note_launches(1);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_interpolate(const float* x, int64_t n, const Geo& g, const float* acc_c, const float* acc_f,
-                               float* a, cudaStream_t st) {
-  if (n == 0) return cudaSuccess;
-  k_interpolate<<<grid_for(n, 256), 256, 0, st>>>(x, n, g, acc_c, acc_f, a);
-  note_launches(1);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_kick_drift(float* x, float* v, int64_t n, const Geo& g, const float* acc_c, const float* acc_f,
-                              float ck, float cd, cudaStream_t st) {
-  if (n == 0) return cudaSuccess;
-  k_kick_drift<<<grid_for(n, 256), 256, 0, st>>>(x, v, n, g, acc_c, acc_f, ck, cd);
-  note_launches(1);
-  return cudaGetLastError();
 }
 
 cudaError_t launch_compress(const float* x, const float* v, int64_t n, const Geo& g, uint32_t* counts,

@@ -1,0 +1,61 @@
+"""Deposits of float particles: orders whose warps fall into small boxes, across
+mesh faces or anywhere, group remainders and both group sizes, against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import mesh
+from synth.generators import FOUR_PI_G_ONE
+from tests.helpers import rel_rms
+
+pytestmark = pytest.mark.gpu
+
+N = 64
+DENSITY_TOL = 1e-5   # float32 deposit vs float64, relative RMS (as tests/test_gpu_mesh.py)
+
+
+def _positions(n, order, seed=3):
+    rng = np.random.default_rng(seed)
+    x = (rng.random((n, 3)) * N).astype(np.float32)
+    if order == "corner":                      # one cell at the far corner: every upper node wraps
+        x = (N - rng.random((n, 3))).astype(np.float32)
+    x[x >= N] = 0.0
+    if order == "cell":
+        c = (x // 4).astype(np.int64)
+        x = x[np.argsort(c[:, 0] + 16 * (c[:, 1] + 16 * c[:, 2]), kind="stable")]
+    return np.ascontiguousarray(x)
+
+
+def _pm(mass):
+    from paper_1611_01545_gb300 import PM
+    return PM(dict(n_fine=N, coarse_ratio=4, tile=16, buffer=8, cmp_ratio=4, vel_bits=16, G=FOUR_PI_G_ONE,
+                   mass=mass, count=(0, 0), r_split=6.0 / 4.5, r_cut=6.0))
+
+
+# 1 .. 65: remainders of a group; 2,490,401: the wide groups (from 152 * 32 * 512 particles)
+@pytest.mark.parametrize("order", ["cell", "random", "corner"])
+@pytest.mark.parametrize("n", [1, 31, 65, 70001, 2490401])
+def test_deposits_of_float_particles(n, order):
+    mass = (8.0, 100.0)       # 100 x 2^32 exceeds the int64 bins: corners go to the mesh directly
+    pm = _pm(mass)
+    x = _positions(n, order)
+    xd = torch.from_numpy(x).cuda()
+    for s in range(2):
+        rc, rf = pm.zeros_meshes()
+        pm.deposit(s, xd, rc, rf)
+        assert rel_rms(rf.cpu().numpy(), mesh.cic_deposit(x, mass[s], N)) < DENSITY_TOL
+        assert rel_rms(rc.cpu().numpy(), mesh.cic_deposit(x / 4.0, mass[s], N // 4)) < DENSITY_TOL
+        rc, rf = pm.zeros_meshes(fixed=True)
+        pm.deposit_fixed(s, xd, rc, rf)
+        M = mesh.fixed_mass(mass[s])
+        np.testing.assert_array_equal(rf.cpu().numpy(), mesh.cic_deposit_fixed(x, M, N))
+        np.testing.assert_array_equal(rc.cpu().numpy(),
+                                      mesh.cic_deposit_fixed((x / np.float32(4)).astype(np.float32), M, N // 4))
+    w = np.random.default_rng(4).standard_normal((n, 2)).astype(np.float32)
+    w[:, 0] = 1.0
+    f = pm.deposit_weights(xd, torch.from_numpy(w).cuda()).cpu().numpy()
+    pm.check()
+    for q in range(2):
+        ref = mesh.cic_deposit(x, w[:, q].astype(np.float64), N)
+        scale = np.sqrt(np.mean(mesh.cic_deposit(x, np.abs(w[:, q]).astype(np.float64), N) ** 2))
+        assert np.sqrt(np.mean((f[q] - ref) ** 2)) < DENSITY_TOL * scale
