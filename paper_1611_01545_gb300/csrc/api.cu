@@ -35,10 +35,10 @@ struct pm_handle {
   int64_t* off[2] = {nullptr, nullptr};
   int64_t* newoff[2] = {nullptr, nullptr};
   uint32_t* counts[2] = {nullptr, nullptr};
-  uint32_t* vmax_bits = nullptr;  // [2]
+  uint32_t* vmax_bits = nullptr;  // [2]; one allocation with amax and work, cleared together by a step's first scan
   uint32_t* amax = nullptr;       // [3] max |a| over the coarse / fine force meshes and the PP accelerations (float bits)
   float4* app = nullptr;          // per particle PP acceleration (pp = 1), stream order, species 0 first
-  void* partial = nullptr;
+  void* scan_state = nullptr;     // look-back state of the scans, both species (zero between launches)
   int* status = nullptr;
   Blk blk_dep{}, blk_ikd{};
   bool persist_dep = false, persist_ikd = false;   // persistent launches of the particle passes
@@ -288,10 +288,8 @@ Blk ikd_blk(const pm_handle* h, int pass) {
   b.brick = block_brick(b);
   return b;
 }
-cudaError_t zero_work(const pm_handle* h, cudaStream_t st) {
-  if (!h->persist_dep && !h->persist_ikd) return cudaSuccess;
-  return cudaMemsetAsync(h->work, 0, 4 * sizeof(int), st);
-}
+// Words of vmax_bits [4], amax [4] and work [4].
+constexpr int kSmallWords = 12;
 
 PCodes view(const pm_codes_t& c, bool vel16) {
   return PCodes{reinterpret_cast<const uint32_t*>(c.pos), c.vel, c.vmax, c.n, vel16};
@@ -437,15 +435,14 @@ int pm_init(const pm_config_t* cfg, pm_handle_t** out) {
     if (e != cudaSuccess) rc = fail(h, PM_ERR_CUDA, std::string("cudaMalloc: ") + cudaGetErrorString(e));
   };
   const size_t nf3 = (size_t)g.nfine3(), nc3 = (size_t)g.ncoarse3();
-  A(&h->rho_f, nf3 * 4);
+  // the coarse density follows the fine one, so that a step clears both at once
+  A(&h->rho_f, (nf3 + nc3) * 4);
   A(&h->acc_f, 3 * nf3 * 4);
-  if (g.two) {
-    A(&h->rho_c, nc3 * 4);
-    A(&h->acc_c, 3 * nc3 * 4);
-  }
-  if (fixed) {
-    A(&h->rho_f_fix, nf3 * 8);
-    if (g.two) A(&h->rho_c_fix, nc3 * 8);
+  if (g.two) A(&h->acc_c, 3 * nc3 * 4);
+  if (fixed) A(&h->rho_f_fix, (nf3 + nc3) * 8);
+  if (g.two && rc == PM_OK) {
+    h->rho_c = h->rho_f + nf3;
+    if (fixed) h->rho_c_fix = h->rho_f_fix + nf3;
   }
   const size_t ncell = (size_t)g.ncell();
   for (int s = 0; s < 2; ++s) {
@@ -453,14 +450,16 @@ int pm_init(const pm_config_t* cfg, pm_handle_t** out) {
     A(&h->newoff[s], (ncell + 1) * 8);
     A(&h->counts[s], ncell * 4);
   }
-  A(&h->vmax_bits, 2 * 4);
-  A(&h->amax, 3 * 4);
+  A(&h->vmax_bits, kSmallWords * 4);
+  if (rc == PM_OK) {
+    h->amax = h->vmax_bits + 4;
+    h->work = reinterpret_cast<int*>(h->vmax_bits + 8);
+  }
   if (c.pp) A(&h->app, (size_t)(c.count[0] + c.count[1]) * sizeof(float4));
-  A(&h->work, 4 * 4);
   h->scratch_n = c.count[0] + c.count[1];
   A(&h->tkey, (size_t)h->scratch_n * 4);
   A(&h->tpv, (size_t)h->scratch_n * 16);
-  A(&h->partial, 2 * scan_partial_bytes((int64_t)ncell));
+  A(&h->scan_state, 2 * scan_state_bytes((int64_t)ncell));
   A(&h->status, 4);
   // plans and tables
   auto make_plan = [&](SolvePlan& p, int N, int nts, int t, int b, int src_n, int batch, const std::vector<float>& kern) {
@@ -498,6 +497,7 @@ int pm_init(const pm_config_t* cfg, pm_handle_t** out) {
     for (int s = 0; s < 2; ++s)
       if (cudaMemset(h->counts[s], 0, ncell * 4) != cudaSuccess) rc = fail(h, PM_ERR_CUDA, "memset");
     if (cudaMemset(h->status, 0, 4) != cudaSuccess) rc = fail(h, PM_ERR_CUDA, "memset");
+    if (cudaMemset(h->scan_state, 0, 2 * scan_state_bytes((int64_t)ncell)) != cudaSuccess) rc = fail(h, PM_ERR_CUDA, "memset");
     if (cudaDeviceSynchronize() != cudaSuccess) rc = fail(h, PM_ERR_CUDA, "init sync");
   }
   if (!g.two) {
@@ -560,7 +560,7 @@ int pm_decompress(pm_handle_t* h, int species, const pm_codes_t* in, float* x, f
   if (int r = check_species(h, species)) return r;
   cudaStream_t st = (cudaStream_t)stream;
   const bool vel16 = h->cfg.vel_bits == 16;
-  CK(h, scan_codes(*in, h->gm.ncell(), h->off[species], h->partial, h->status, st));
+  CK(h, scan_codes(*in, h->gm.ncell(), h->off[species], h->scan_state, h->status, st));
   CK(h, launch_decompress(view(*in, vel16), h->off[species], h->geo, x, v, st));
   return PM_OK;
 }
@@ -574,7 +574,7 @@ int pm_compress(pm_handle_t* h, int species, const float* x, const float* v, con
   cudaStream_t st = (cudaStream_t)stream;
   CK(h, cudaMemsetAsync(h->counts[species], 0, (size_t)h->gm.ncell() * 4, st));
   CK(h, launch_compress(x, v, out->n, h->geo, h->counts[species], h->vmax_bits + species, vmax_in,
-                        h->newoff[species], *out, h->cfg.vel_bits == 16, h->partial, h->status, st));
+                        h->newoff[species], *out, h->cfg.vel_bits == 16, h->scan_state, h->status, st));
   return PM_OK;
 }
 
@@ -613,9 +613,9 @@ int pm_deposit_codes(pm_handle_t* h, const pm_codes_t in[2], void* rho_coarse, v
   cudaStream_t st = (cudaStream_t)stream;
   const bool fixed = h->cfg.deposit_mode == 1;
   const bool vel16 = h->cfg.vel_bits == 16;
-  CK(h, scan_codes2(in, h->gm.ncell(), h->off[0], h->off[1], h->partial, h->status, st));
+  const ScanClear clear{{nullptr, nullptr}, h->vmax_bits, kSmallWords};
+  CK(h, scan_codes2(in, h->gm.ncell(), h->off[0], h->off[1], h->scan_state, h->status, &clear, st));
   long long M0 = llrint(h->cfg.mass[0] * 4294967296.0), M1 = llrint(h->cfg.mass[1] * 4294967296.0);
-  CK(h, zero_work(h, st));
   CK(h, launch_deposit_codes(view(in[0], vel16), view(in[1], vel16), h->off[0], h->off[1], h->geo, dep_blk(h),
                              (float)h->cfg.mass[0], (float)h->cfg.mass[1], M0, M1, h->gm.two ? rho_coarse : nullptr,
                              rho_fine, fixed, st));
@@ -632,7 +632,7 @@ int pm_pp_accel(pm_handle_t* h, const pm_codes_t in[2], float* acc, void* stream
   if (!(h->cfg.r_soft >= 0.0 && h->cfg.r_soft < 1.0)) return fail(h, PM_ERR_ARG, "r_soft must lie in [0, 1)");
   cudaStream_t st = (cudaStream_t)stream;
   const bool vel16 = h->cfg.vel_bits == 16;
-  CK(h, scan_codes2(in, h->gm.ncell(), h->off[0], h->off[1], h->partial, h->status, st));
+  CK(h, scan_codes2(in, h->gm.ncell(), h->off[0], h->off[1], h->scan_state, h->status, nullptr, st));
   CK(h, launch_pp(view(in[0], vel16), view(in[1], vel16), h->off[0], h->off[1], h->geo, (float)h->cfg.mass[0],
                   (float)h->cfg.mass[1], (float)h->cfg.G, (float)h->cfg.r_soft, reinterpret_cast<float4*>(acc), nullptr,
                   st));
@@ -1024,7 +1024,8 @@ int step_launch(pm_handle_t* h, const pm_codes_t in[2], pm_codes_t out[2], doubl
   const int64_t ncell = g.ncell();
   {
     TimedScope ts(tm, "scan_in", st);
-    CK(h, scan_codes2(in, ncell, h->off[0], h->off[1], h->partial, h->status, st));
+    const ScanClear clear{{h->counts[0], h->counts[1]}, h->vmax_bits, kSmallWords};
+    CK(h, scan_codes2(in, ncell, h->off[0], h->off[1], h->scan_state, h->status, &clear, st));
   }
   void* rc = fixed ? (void*)h->rho_c_fix : (void*)h->rho_c;
   void* rf = fixed ? (void*)h->rho_f_fix : (void*)h->rho_f;
@@ -1036,10 +1037,8 @@ int step_launch(pm_handle_t* h, const pm_codes_t in[2], pm_codes_t out[2], doubl
   const bool via_fine = g.two && !fixed;
   {
     TimedScope ts(tm, "deposit", st);
-    CK(h, cudaMemsetAsync(rf, 0, (size_t)g.nfine3() * (fixed ? 8 : 4), st));
-    if (g.two) CK(h, cudaMemsetAsync(rc, 0, (size_t)g.ncoarse3() * (fixed ? 8 : 4), st));
+    CK(h, cudaMemsetAsync(rf, 0, (size_t)(g.nfine3() + g.ncoarse3()) * (fixed ? 8 : 4), st));   // and rc after it
     long long M0 = llrint(h->cfg.mass[0] * 4294967296.0), M1 = llrint(h->cfg.mass[1] * 4294967296.0);
-    CK(h, zero_work(h, st));
     // (float: the coarse density is restricted from each block's fine tile as it flushes)
     CK(h, launch_deposit_codes(view(in[0], vel16), view(in[1], vel16), h->off[0], h->off[1], h->geo, dep_blk(h),
                                (float)h->cfg.mass[0], (float)h->cfg.mass[1], M0, M1, g.two ? rc : nullptr, rf, fixed,
@@ -1047,7 +1046,6 @@ int step_launch(pm_handle_t* h, const pm_codes_t in[2], pm_codes_t out[2], doubl
   }
   const bool bound = h->cfg.vmax_mode == 1;
   const float ck = (float)c_kick, cd = (float)c_drift;
-  if (bound) CK(h, cudaMemsetAsync(h->amax, 0, 12, st));
   if (int r = solve_impl(h, rc, rf, fixed, h->acc_c, h->acc_f, st, bound ? h->amax : nullptr, via_fine)) return r;
   if (h->cfg.pp) {
     TimedScope ts(tm, "pp", st);
@@ -1061,8 +1059,6 @@ int step_launch(pm_handle_t* h, const pm_codes_t in[2], pm_codes_t out[2], doubl
   if (bound) CK(h, launch_vmax_bound(in[0].vmax, in[1].vmax, h->amax, ck, out[0].vmax, out[1].vmax, st));
   {
     TimedScope ts(tm, "ikd_count", st);
-    if (!bound) CK(h, cudaMemsetAsync(h->vmax_bits, 0, 8, st));
-    for (int s = 0; s < 2; ++s) CK(h, cudaMemsetAsync(h->counts[s], 0, (size_t)ncell * 4, st));
     CK(h, launch_ikd_count(view(in[0], vel16), view(in[1], vel16), h->off[0], h->off[1], h->geo, ikd_blk(h, 0),
                            h->acc_c, h->acc_f, ck, cd, h->counts[0], h->counts[1], h->vmax_bits, h->tkey, h->tpv,
                            bound ? out[0].vmax : nullptr, bound ? out[1].vmax : nullptr, h->cfg.pp ? h->app : nullptr,
@@ -1071,10 +1067,9 @@ int step_launch(pm_handle_t* h, const pm_codes_t in[2], pm_codes_t out[2], doubl
   if (h->post_count_record) CK(h, cudaEventRecord(h->post_count_record, st));
   {
     TimedScope ts(tm, "scan_out", st);
-    if (!bound) CK(h, launch_set_vmax2(h->vmax_bits, out[0].vmax, out[1].vmax, st));
     const int64_t expect[2] = {in[0].n, in[1].n};
-    CK(h, scan_counts2(h->counts[0], h->counts[1], ncell, expect, h->newoff[0], h->newoff[1], out, h->partial,
-                       h->status, st));
+    CK(h, scan_counts2(h->counts[0], h->counts[1], ncell, expect, h->newoff[0], h->newoff[1], out,
+                       bound ? nullptr : h->vmax_bits, h->scan_state, h->status, st));
   }
   {
     TimedScope ts(tm, "ikd_scatter", st);

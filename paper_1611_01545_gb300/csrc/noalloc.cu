@@ -21,7 +21,7 @@ namespace {
 constexpr int64_t kMaxCells = (int64_t)64 * 64 * 64;   // n_cmp <= 64
 constexpr size_t kOffBytes = (size_t)(kMaxCells + 1) * sizeof(int64_t);
 constexpr size_t kPartialOffset = (kOffBytes + 255) / 256 * 256;
-constexpr size_t kPartialBytes = 4096;                  // >= pm::scan_partial_bytes(kMaxCells)
+constexpr size_t kPartialBytes = 4096;                  // >= pm::scan_state_bytes(kMaxCells); zero at load, and again after each scan
 constexpr size_t kStatusOffset = kPartialOffset + kPartialBytes;
 constexpr size_t kScratchBytes = kStatusOffset + 256;
 
@@ -60,7 +60,7 @@ extern "C" int pm_decompress_noalloc(int32_t n_fine, int32_t cmp_ratio, int32_t 
   if (n_fine <= 0 || cmp_ratio <= 0 || (cmp_ratio & (cmp_ratio - 1)) || n_fine % cmp_ratio) return PM_ERR_ARG;
   const int ncmp = n_fine / cmp_ratio;
   const int64_t ncell = (int64_t)ncmp * ncmp * ncmp;
-  if (ncell > kMaxCells || pm::scan_partial_bytes(ncell) > kPartialBytes) return PM_ERR_ARG;
+  if (ncell > kMaxCells || pm::scan_state_bytes(ncell) > kPartialBytes) return PM_ERR_ARG;
   unsigned char* base = nullptr;
   if (scratch_address(&base) != cudaSuccess) return PM_ERR_CUDA;
   int64_t* off = reinterpret_cast<int64_t*>(base);

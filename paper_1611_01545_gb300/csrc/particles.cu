@@ -1,6 +1,4 @@
 // Particle-side kernels of the PM step:
-//   * cell-count scans of the cell-ordered codec (Sec. 2.4): count byte with
-//     the 255 escape, CSR offsets, escape-list compaction;
 //   * compress of one species (Sec. 2.4; decompress and the kernels over
 //     float particles are in plain.cu);
 //   * the fused step passes that read the codes directly: decode + deposit
@@ -14,298 +12,6 @@
 #include "particles.cuh"
 
 namespace pm {
-
-// ------------------------------------------------------------ scan -------
-
-struct V2 {
-  long long a;
-  int b;
-};
-__device__ __forceinline__ V2 v2add(V2 x, V2 y) { return V2{x.a + y.a, x.b + y.b}; }
-
-constexpr int SCAN_THREADS = 256;
-constexpr int SCAN_ITEMS = 8;
-constexpr int SCAN_TILE = SCAN_THREADS * SCAN_ITEMS;
-
-__device__ __forceinline__ V2 warp_incl(V2 v) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    long long a = __shfl_up_sync(0xffffffffu, v.a, o);
-    int b = __shfl_up_sync(0xffffffffu, v.b, o);
-    if (lane >= o) { v.a += a; v.b += b; }
-  }
-  return v;
-}
-
-// Exclusive block scan of one V2 per thread; returns the exclusive prefix and the block total.
-__device__ V2 block_excl(V2 v, V2* total) {
-  __shared__ V2 warp_sums[32];
-  __shared__ V2 block_total;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  V2 inc = warp_incl(v);
-  if (lane == 31) warp_sums[wid] = inc;
-  __syncthreads();
-  if (wid == 0) {
-    int nw = blockDim.x >> 5;
-    V2 w = lane < nw ? warp_sums[lane] : V2{0, 0};
-    V2 wi = warp_incl(w);
-    if (lane < nw) warp_sums[lane] = V2{wi.a - w.a, wi.b - w.b};
-    if (lane == nw - 1) block_total = wi;
-  }
-  __syncthreads();
-  V2 res = v2add(warp_sums[wid], V2{inc.a - v.a, inc.b - v.b});
-  *total = block_total;
-  __syncthreads();
-  return res;
-}
-
-// Count of compression cell c from the count byte and the escape list.
-struct CodesCount {
-  const uint8_t* cnt;
-  const uint32_t* esc;
-  const uint32_t* n_esc;
-  int64_t esc_cap;
-  int* status;
-  __device__ V2 operator()(int64_t c) const {
-    unsigned k = cnt[c];
-    if (k != 255u) return V2{(long long)k, 0};
-    long long ne = (long long)*n_esc;
-    if (ne > esc_cap) ne = esc_cap;
-    long long lo = 0, hi = ne - 1;
-    while (lo <= hi) {
-      long long mid = (lo + hi) >> 1;
-      long long cm = esc[2 * mid];
-      if (cm == c) return V2{(long long)esc[2 * mid + 1], 1};
-      if (cm < c) lo = mid + 1; else hi = mid - 1;
-    }
-    atomicOr(status, ST_CORRUPT);
-    return V2{0, 1};
-  }
-};
-
-struct U32Count {
-  const uint32_t* cnt;
-  __device__ V2 operator()(int64_t c) const {
-    unsigned k = cnt[c];
-    return V2{(long long)k, k >= 255u ? 1 : 0};
-  }
-};
-
-// Each scan launch serves one or two species: blockIdx.y (blockIdx.x for the
-// one-block kernels) selects the species' getter / output and its partials
-// (stride pstride V2 per species).
-template <class T> struct Pair { T v[2]; };
-
-template <class Get>
-__global__ void __launch_bounds__(SCAN_THREADS) k_scan_reduce(Pair<Get> gets, int64_t n, V2* partial_all,
-                                                            int pstride) {
-  const Get& get = gets.v[blockIdx.y];
-  V2* partial = partial_all + (size_t)blockIdx.y * pstride;
-  const int64_t base = (int64_t)blockIdx.x * SCAN_TILE;
-  V2 s{0, 0};
-  for (int i = threadIdx.x; i < SCAN_TILE; i += SCAN_THREADS) {
-    int64_t j = base + i;
-    if (j < n) s = v2add(s, get(j));
-  }
-  V2 tot;
-  block_excl(s, &tot);
-  if (threadIdx.x == 0) partial[blockIdx.x] = tot;
-}
-
-// Exclusive scan of the partials in place (one block per species); partial[nb] = grand total.
-__global__ void __launch_bounds__(1024) k_scan_partials(V2* partial_all, int nb, int pstride) {
-  V2* partial = partial_all + (size_t)blockIdx.x * pstride;
-  __shared__ V2 carry;
-  if (threadIdx.x == 0) carry = V2{0, 0};
-  __syncthreads();
-  for (int base = 0; base < nb; base += blockDim.x) {
-    int i = base + threadIdx.x;
-    V2 v = i < nb ? partial[i] : V2{0, 0};
-    V2 tot;
-    V2 ex = block_excl(v, &tot);
-    V2 c = carry;
-    if (i < nb) partial[i] = v2add(ex, c);
-    __syncthreads();
-    if (threadIdx.x == 0) carry = v2add(c, tot);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) partial[nb] = carry;
-}
-
-// Decompress offsets: off[c] = sum_{c' < c} count(c'), off[n] = total; checks total == expect.
-struct PutOffsets {
-  int64_t* off;
-  __device__ void operator()(int64_t c, V2 excl, V2) const { off[c] = excl.a; }
-};
-
-// Compress outputs: CSR offsets, count bytes, ordered escape list.
-struct PutCodes {
-  int64_t* off;
-  uint8_t* cnt;
-  uint32_t* esc;
-  int64_t esc_cap;
-  int* status;
-  __device__ void operator()(int64_t c, V2 excl, V2 v) const {
-    off[c] = excl.a;
-    long long k = v.a;
-    cnt[c] = (uint8_t)(k >= 255 ? 255 : k);
-    if (k >= 255) {
-      if ((int64_t)excl.b < esc_cap) {
-        esc[2 * (int64_t)excl.b] = (uint32_t)c;
-        esc[2 * (int64_t)excl.b + 1] = (uint32_t)k;
-      } else {
-        atomicOr(status, ST_OVERFLOW);
-      }
-    }
-  }
-};
-
-template <class Get, class Put>
-__global__ void __launch_bounds__(SCAN_THREADS) k_scan_final(Pair<Get> gets, Pair<Put> puts, int64_t n,
-                                                           const V2* partial_all, int pstride) {
-  const Get& get = gets.v[blockIdx.y];
-  const Put& put = puts.v[blockIdx.y];
-  const V2* partial = partial_all + (size_t)blockIdx.y * pstride;
-  const int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
-  V2 v[SCAN_ITEMS];
-  V2 s{0, 0};
-#pragma unroll
-  for (int k = 0; k < SCAN_ITEMS; ++k) {
-    int64_t j = base + k;
-    v[k] = j < n ? get(j) : V2{0, 0};
-    s = v2add(s, v[k]);
-  }
-  V2 tot;
-  V2 ex = v2add(block_excl(s, &tot), partial[blockIdx.x]);
-#pragma unroll
-  for (int k = 0; k < SCAN_ITEMS; ++k) {
-    int64_t j = base + k;
-    if (j < n) put(j, ex, v[k]);
-    ex = v2add(ex, v[k]);
-  }
-}
-
-struct FinishArgs {
-  int64_t expect;
-  int64_t* off;
-  uint32_t* n_esc_out;   // set for compressed outputs
-  int64_t esc_cap;
-};
-
-// Writes off[n] = total, checks the total, sets n_esc if asked; thread s = species s.
-__global__ void k_scan_finish(const V2* partial_all, int nb, int pstride, int64_t n, Pair<FinishArgs> fa, int nsp,
-                              int* status) {
-  const int s = threadIdx.x;
-  if (s >= nsp) return;
-  const FinishArgs& f = fa.v[s];
-  V2 t = partial_all[(size_t)s * pstride + nb];
-  f.off[n] = t.a;
-  if (t.a != f.expect) atomicOr(status, ST_CORRUPT);
-  if (f.n_esc_out) *f.n_esc_out = (uint32_t)(t.b < f.esc_cap ? t.b : f.esc_cap);
-}
-
-struct EscArgs {
-  const uint8_t* cnt;
-  const uint32_t* esc;
-  const uint32_t* n_esc;
-  int64_t esc_cap;
-  const float* vmax;
-};
-
-// Every escape entry must name a cell whose byte is 255, hold >= 255, ascend; blockIdx.y = species.
-__global__ void k_check_escapes(Pair<EscArgs> ea, int64_t ncell, int* status) {
-  const EscArgs& e = ea.v[blockIdx.y];
-  long long ne = *e.n_esc;
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    float vm = *e.vmax;
-    if (!(vm >= 0.f) || isinf(vm)) atomicOr(status, ST_CORRUPT);
-    if (ne > e.esc_cap) atomicOr(status, ST_CORRUPT);
-  }
-  if (ne > e.esc_cap) ne = e.esc_cap;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < ne; i += (long long)gridDim.x * blockDim.x) {
-    uint32_t c = e.esc[2 * i], k = e.esc[2 * i + 1];
-    bool bad = (int64_t)c >= ncell || k < 255u || e.cnt[c] != 255u || (i > 0 && e.esc[2 * (i - 1)] >= c);
-    if (bad) atomicOr(status, ST_CORRUPT);
-  }
-}
-
-static int scan_blocks(int64_t n) { return (int)((n + SCAN_TILE - 1) / SCAN_TILE); }
-
-// Offsets of nsp (1 or 2) species' input codes in one set of launches.
-static cudaError_t scan_codes_n(const pm_codes_t* in, int nsp, int64_t ncell, int64_t* const* off, void* partial_ws,
-                                int* status, cudaStream_t st) {
-  V2* partial = static_cast<V2*>(partial_ws);
-  const int nb = scan_blocks(ncell), ps = nb + 1;
-  Pair<CodesCount> get{};
-  Pair<PutOffsets> put{};
-  Pair<FinishArgs> fin{};
-  Pair<EscArgs> esc{};
-  for (int s = 0; s < nsp; ++s) {
-    get.v[s] = CodesCount{in[s].cnt, in[s].esc, in[s].n_esc, in[s].esc_cap, status};
-    put.v[s] = PutOffsets{off[s]};
-    fin.v[s] = FinishArgs{in[s].n, off[s], nullptr, 0};
-    esc.v[s] = EscArgs{in[s].cnt, in[s].esc, in[s].n_esc, in[s].esc_cap, in[s].vmax};
-  }
-  k_check_escapes<<<dim3(64, nsp), 256, 0, st>>>(esc, ncell, status);
-  k_scan_reduce<<<dim3(nb, nsp), SCAN_THREADS, 0, st>>>(get, ncell, partial, ps);
-  k_scan_partials<<<nsp, 1024, 0, st>>>(partial, nb, ps);
-  k_scan_final<<<dim3(nb, nsp), SCAN_THREADS, 0, st>>>(get, put, ncell, partial, ps);
-  k_scan_finish<<<1, 32, 0, st>>>(partial, nb, ps, ncell, fin, nsp, status);
-  note_launches(5);
-  return cudaGetLastError();
-}
-
-cudaError_t scan_codes(const pm_codes_t& in, int64_t ncell, int64_t* off, void* partial_ws, int* status,
-                       cudaStream_t st) {
-  int64_t* offs[1] = {off};
-  return scan_codes_n(&in, 1, ncell, offs, partial_ws, status, st);
-}
-
-cudaError_t scan_codes2(const pm_codes_t in[2], int64_t ncell, int64_t* off0, int64_t* off1, void* partial_ws,
-                        int* status, cudaStream_t st) {
-  int64_t* offs[2] = {off0, off1};
-  return scan_codes_n(in, 2, ncell, offs, partial_ws, status, st);
-}
-
-static cudaError_t scan_counts_n(const uint32_t* const* counts, int nsp, int64_t ncell, const int64_t* expect,
-                                 int64_t* const* off, pm_codes_t* out, void* partial_ws, int* status,
-                                 cudaStream_t st) {
-  V2* partial = static_cast<V2*>(partial_ws);
-  const int nb = scan_blocks(ncell), ps = nb + 1;
-  Pair<U32Count> get{};
-  Pair<PutCodes> put{};
-  Pair<FinishArgs> fin{};
-  for (int s = 0; s < nsp; ++s) {
-    get.v[s] = U32Count{counts[s]};
-    put.v[s] = PutCodes{off[s], out[s].cnt, out[s].esc, out[s].esc_cap, status};
-    fin.v[s] = FinishArgs{expect[s], off[s], out[s].n_esc, out[s].esc_cap};
-  }
-  k_scan_reduce<<<dim3(nb, nsp), SCAN_THREADS, 0, st>>>(get, ncell, partial, ps);
-  k_scan_partials<<<nsp, 1024, 0, st>>>(partial, nb, ps);
-  k_scan_final<<<dim3(nb, nsp), SCAN_THREADS, 0, st>>>(get, put, ncell, partial, ps);
-  k_scan_finish<<<1, 32, 0, st>>>(partial, nb, ps, ncell, fin, nsp, status);
-  note_launches(4);
-  return cudaGetLastError();
-}
-
-cudaError_t scan_counts(const uint32_t* counts, int64_t ncell, int64_t expect, int64_t* off, pm_codes_t& out,
-                        void* partial_ws, int* status, cudaStream_t st) {
-  const uint32_t* c[1] = {counts};
-  int64_t* o[1] = {off};
-  return scan_counts_n(c, 1, ncell, &expect, o, &out, partial_ws, status, st);
-}
-
-cudaError_t scan_counts2(const uint32_t* counts0, const uint32_t* counts1, int64_t ncell, const int64_t expect[2],
-                         int64_t* off0, int64_t* off1, pm_codes_t out[2], void* partial_ws, int* status,
-                         cudaStream_t st) {
-  const uint32_t* c[2] = {counts0, counts1};
-  int64_t* o[2] = {off0, off1};
-  return scan_counts_n(c, 2, ncell, expect, o, out, partial_ws, status, st);
-}
-
-// Partials of one species; the two-species scans use twice this.
-size_t scan_partial_bytes(int64_t ncell) { return sizeof(V2) * (size_t)(scan_blocks(ncell) + 1); }
 
 // The same CIC gather when the lower corner's local index (lx, ly, lz) and the
 // upper weights w1 are already known; same weights and order as gather().
@@ -481,10 +187,6 @@ __global__ void k_compress_pass(const float* x, const float* v, int64_t n, Geo g
     }
   }
   if (MODE == 0 && vmax_in == nullptr) block_vmax(local_max, vmax_bits);
-}
-
-__global__ void k_set_vmax(const uint32_t* vmax_bits, const float* vmax_in, float* out) {
-  *out = vmax_in ? *vmax_in : __uint_as_float(*vmax_bits);
 }
 
 // Bound on |v'_d| = |v_d + c_k a_d(x)| before the kick: decoded |v_d| < v_max
@@ -1340,16 +1042,16 @@ static int grid_for(int64_t n, int threads) {
 
 cudaError_t launch_compress(const float* x, const float* v, int64_t n, const Geo& g, uint32_t* counts,
                             uint32_t* vmax_bits, const float* vmax_in, int64_t* off, pm_codes_t& out, bool vel16,
-                            void* partial, int* status, cudaStream_t st) {
+                            void* scan_state, int* status, cudaStream_t st) {
   PCodesOut o{reinterpret_cast<uint32_t*>(out.pos), out.vel, out.vmax, vel16};
   cudaMemsetAsync(vmax_bits, 0, sizeof(uint32_t), st);
   int grid = grid_for(n > 0 ? n : 1, 256);
   k_compress_pass<0><<<grid, 256, 0, st>>>(x, v, n, g, counts, vmax_bits, vmax_in, off, o, status);
-  k_set_vmax<<<1, 1, 0, st>>>(vmax_bits, vmax_in, out.vmax);
-  cudaError_t e = scan_counts(counts, g.ncell, n, off, out, partial, status, st);
+  const uint32_t* vsrc = vmax_in ? reinterpret_cast<const uint32_t*>(vmax_in) : vmax_bits;
+  cudaError_t e = scan_counts(counts, g.ncell, n, off, out, vsrc, scan_state, status, st);
   if (e != cudaSuccess) return e;
   k_compress_pass<1><<<grid, 256, 0, st>>>(x, v, n, g, counts, vmax_bits, vmax_in, off, o, status);
-  note_launches(3);
+  note_launches(2);
   return cudaGetLastError();
 }
 
@@ -1460,23 +1162,6 @@ cudaError_t launch_ikd_scatter(int64_t n0, int64_t n1, const int64_t* off0, cons
 cudaError_t launch_vmax_bound(const float* vin0, const float* vin1, const uint32_t* amax, float ck, float* vout0,
                               float* vout1, cudaStream_t st) {
   k_vmax_bound<<<1, 1, 0, st>>>(vin0, vin1, amax, ck, vout0, vout1);
-  note_launches(1);
-  return cudaGetLastError();
-}
-
-__global__ void k_set_vmax2(const uint32_t* vmax_bits, float* out0, float* out1) {
-  *out0 = __uint_as_float(vmax_bits[0]);
-  *out1 = __uint_as_float(vmax_bits[1]);
-}
-
-cudaError_t launch_set_vmax2(const uint32_t* vmax_bits, float* out0, float* out1, cudaStream_t st) {
-  k_set_vmax2<<<1, 1, 0, st>>>(vmax_bits, out0, out1);
-  note_launches(1);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_set_vmax(const uint32_t* vmax_bits, float* out, cudaStream_t st) {
-  k_set_vmax<<<1, 1, 0, st>>>(vmax_bits, nullptr, out);
   note_launches(1);
   return cudaGetLastError();
 }

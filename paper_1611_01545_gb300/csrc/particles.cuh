@@ -38,17 +38,26 @@ struct PCodesOut {
   bool vel16;
 };
 
-cudaError_t scan_codes(const pm_codes_t& in, int64_t ncell, int64_t* off, void* partial_ws, int* status,
-                       cudaStream_t st);
+// Scans (scan.cu).  state: scan_state_bytes(ncell) per species, zeroed once
+// when it is allocated (each launch leaves it zero again).
+size_t scan_state_bytes(int64_t ncell);
+// Arrays that a step's first scan clears on the way: the new-cell counts of
+// both species and `small_words` 32-bit words (null: nothing).
+struct ScanClear {
+  uint32_t* counts[2];
+  uint32_t* small;
+  int small_words;
+};
+cudaError_t scan_codes(const pm_codes_t& in, int64_t ncell, int64_t* off, void* state, int* status, cudaStream_t st);
+// vmax_bits (float bits): copied to out.vmax when set.
 cudaError_t scan_counts(const uint32_t* counts, int64_t ncell, int64_t expect, int64_t* off, pm_codes_t& out,
-                        void* partial_ws, int* status, cudaStream_t st);
-// Both species in one set of launches (partials: 2 * scan_partial_bytes).
-cudaError_t scan_codes2(const pm_codes_t in[2], int64_t ncell, int64_t* off0, int64_t* off1, void* partial_ws,
-                        int* status, cudaStream_t st);
+                        const uint32_t* vmax_bits, void* state, int* status, cudaStream_t st);
+// Both species in one launch (2 scan_state_bytes of state).
+cudaError_t scan_codes2(const pm_codes_t in[2], int64_t ncell, int64_t* off0, int64_t* off1, void* state, int* status,
+                        const ScanClear* clear, cudaStream_t st);
 cudaError_t scan_counts2(const uint32_t* counts0, const uint32_t* counts1, int64_t ncell, const int64_t expect[2],
-                         int64_t* off0, int64_t* off1, pm_codes_t out[2], void* partial_ws, int* status,
-                         cudaStream_t st);
-size_t scan_partial_bytes(int64_t ncell);
+                         int64_t* off0, int64_t* off1, pm_codes_t out[2], const uint32_t* vmax_bits, void* state,
+                         int* status, cudaStream_t st);
 
 cudaError_t launch_decompress(const PCodes& in, const int64_t* off, const Geo& g, float* x, float* v, cudaStream_t st);
 cudaError_t launch_deposit(const float* x, int64_t n, float m, const Geo& g, float* rho_c, float* rho_f,
@@ -63,7 +72,7 @@ cudaError_t launch_kick_drift(float* x, float* v, int64_t n, const Geo& g, const
                               float ck, float cd, cudaStream_t st);
 cudaError_t launch_compress(const float* x, const float* v, int64_t n, const Geo& g, uint32_t* counts,
                             uint32_t* vmax_bits, const float* vmax_in, int64_t* off, pm_codes_t& out, bool vel16,
-                            void* partial, int* status, cudaStream_t st);
+                            void* scan_state, int* status, cudaStream_t st);
 size_t deposit_codes_smem(const Geo& g, const Blk& bk, bool fixed);
 size_t ikd_count_smem(const Geo& g, const Blk& bk);
 size_t ikd_scatter_smem(const Geo& g, const Blk& bk);
@@ -82,8 +91,6 @@ cudaError_t launch_ikd_scatter(int64_t n0, int64_t n1, const int64_t* off0, cons
                                const Blk& bk, uint32_t* counts0, uint32_t* counts1, const int64_t* newoff0,
                                const int64_t* newoff1, const PCodesOut& o0, const PCodesOut& o1, const uint32_t* tkey,
                                const uint4* tpv, bool coded, int* status, cudaStream_t st);
-cudaError_t launch_set_vmax(const uint32_t* vmax_bits, float* out, cudaStream_t st);
-cudaError_t launch_set_vmax2(const uint32_t* vmax_bits, float* out0, float* out1, cudaStream_t st);
 // v_max' bound of both species from v_max and the maxima amax[3] (coarse mesh,
 // fine mesh, PP accelerations; float bits).
 // PP acceleration (Eq. 4) of every particle of both species into acc[t] (stream index t,
