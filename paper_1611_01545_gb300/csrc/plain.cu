@@ -11,32 +11,99 @@
 
 namespace pm {
 
-// Cell of stream index p: the last c with off[c] <= p (binary search over all cells).
-__device__ __forceinline__ int64_t find_cell(const int64_t* off, int64_t ncell, int64_t p) {
-  int64_t lo = 0, hi = ncell - 1;
+// ---- decompress -----------------------------------------------------------
+//
+// A block owns kDecChunk consecutive particles (cells differ in weight by
+// orders of magnitude on clustered sets, chunks do not), finds the cells of
+// the first and the last of them by a 32-way search, and keeps the offsets
+// and coordinates of the cells between in shared memory, where a particle
+// finds its cell in a few reads.  (One thread per particle with a search over
+// all cells' offsets in global memory, 18 dependent loads on a 64^3 mesh, took
+// 367 us for 16.8M particles with 16-bit codes; this takes 182 us,
+// against 91 us for the bytes alone.)  Positions and velocities go through
+// shared memory so that a warp writes whole 128-byte lines where 12-byte
+// records would touch each line three times.
+
+constexpr int kDecThreads = 256;
+constexpr int kDecChunk = 2048;
+constexpr int kDecCells = 512;   // cells of a chunk kept in shared memory; sparser chunks search global memory
+
+// The last cell c in [lo, hi] with off[c] <= p (off[lo] <= p), by a warp.
+__device__ __forceinline__ int64_t warp_find_cell(const int64_t* off, int64_t lo, int64_t hi, int64_t p) {
   while (lo < hi) {
-    int64_t mid = (lo + hi + 1) >> 1;
-    if (off[mid] <= p) lo = mid; else hi = mid - 1;
+    const int64_t step = (hi - lo) / 32 + 1;
+    const int64_t c = lo + step * ((threadIdx.x & 31) + 1);
+    const int k = __popc(__ballot_sync(0xffffffffu, c <= hi && off[c] <= p));
+    const int64_t end = lo + step * (k + 1) - 1;
+    lo += step * k;
+    hi = end < hi ? end : hi;
   }
   return lo;
 }
 
-__global__ void k_decompress(PCodes in, const int64_t* off, Geo g, float* x, float* v) {
+__global__ void __launch_bounds__(kDecThreads) k_decompress(PCodes in, const int64_t* off, Geo g, float* x, float* v) {
+  __shared__ int64_t ends[2];
+  __shared__ int64_t ro[kDecCells];
+  __shared__ ushort4 at[kDecCells];
+  __shared__ float sx[3 * kDecThreads], sv[3 * kDecThreads];
   const float pscale = (float)g.rcmp / 256.0f;
-  const float vm = *in.vmax;
   const int half = in.vel16 ? 32768 : 128;
-  const float step = __fmul_rn(vm, 1.0f / (float)half);
-  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < in.n; p += (int64_t)gridDim.x * blockDim.x) {
-    int64_t c = find_cell(off, g.ncell, p);
-    int cx = (int)(c % g.ncmp), cy = (int)((c / g.ncmp) % g.ncmp), cz = (int)(c / ((int64_t)g.ncmp * g.ncmp));
-    int q[3], qv[3];
-    unpack_pos(in.pos[p], q);
-    load_vel(in.vel, in.vel16, p, qv);
-    x[3 * p + 0] = decode_pos(cx, q[0], pscale);
-    x[3 * p + 1] = decode_pos(cy, q[1], pscale);
-    x[3 * p + 2] = decode_pos(cz, q[2], pscale);
+  const float step = __fmul_rn(*in.vmax, 1.0f / (float)half);
+  const uint32_t nc = (uint32_t)g.ncmp;
+  for (int64_t p0 = (int64_t)blockIdx.x * kDecChunk; p0 < in.n; p0 += (int64_t)gridDim.x * kDecChunk) {
+    const int64_t p1 = p0 + kDecChunk < in.n ? p0 + kDecChunk : in.n;
+    const int wid = threadIdx.x >> 5;
+    if (wid < 2) {
+      const int64_t c = warp_find_cell(off, 0, g.ncell - 1, wid ? p1 - 1 : p0);
+      if ((threadIdx.x & 31) == 0) ends[wid] = c;
+    }
+    __syncthreads();
+    const int64_t c0 = ends[0], c1 = ends[1];
+    const bool local = c1 - c0 < kDecCells;
+    const int cells = local ? (int)(c1 - c0) + 1 : 0;
+    int top = 1;   // power of two, at least cells / 2
+    while (2 * top < cells) top *= 2;
+    for (int i = threadIdx.x; i < cells; i += kDecThreads) {
+      ro[i] = off[c0 + i];
+      const uint32_t c = (uint32_t)(c0 + i);
+      at[i] = make_ushort4((unsigned short)(c % nc), (unsigned short)(c / nc % nc), (unsigned short)(c / nc / nc), 0);
+    }
+    __syncthreads();
+    for (int64_t pb = p0; pb < p1; pb += kDecThreads) {
+      const int64_t p = pb + threadIdx.x;
+      if (p < p1) {
+        ushort4 c;
+        if (local) {
+          int lo = 0;
+          for (int d = top; d > 0; d >>= 1)
+            if (lo + d < cells && ro[lo + d] <= p) lo += d;
+          c = at[lo];
+        } else {
+          int64_t lo = c0, hi = c1;
+          while (lo < hi) {
+            const int64_t mid = (lo + hi + 1) >> 1;
+            if (off[mid] <= p) lo = mid; else hi = mid - 1;
+          }
+          const uint32_t k = (uint32_t)lo;
+          c = make_ushort4((unsigned short)(k % nc), (unsigned short)(k / nc % nc), (unsigned short)(k / nc / nc), 0);
+        }
+        int q[3], qv[3];
+        unpack_pos(in.pos[p], q);
+        load_vel(in.vel, in.vel16, p, qv);
+        sx[3 * threadIdx.x] = decode_pos(c.x, q[0], pscale);
+        sx[3 * threadIdx.x + 1] = decode_pos(c.y, q[1], pscale);
+        sx[3 * threadIdx.x + 2] = decode_pos(c.z, q[2], pscale);
 #pragma unroll
-    for (int d = 0; d < 3; ++d) v[3 * p + d] = decode_vel(qv[d], half, step);
+        for (int d = 0; d < 3; ++d) sv[3 * threadIdx.x + d] = decode_vel(qv[d], half, step);
+      }
+      __syncthreads();
+      const int m = 3 * (int)(p1 - pb < kDecThreads ? p1 - pb : kDecThreads);
+      for (int i = threadIdx.x; i < m; i += kDecThreads) {
+        x[3 * pb + i] = sx[i];
+        v[3 * pb + i] = sv[i];
+      }
+      __syncthreads();
+    }
   }
 }
 
@@ -478,7 +545,7 @@ cudaError_t launch_deposit_weights(const float* x, int64_t n, const float* w, in
 
 cudaError_t launch_decompress(const PCodes& in, const int64_t* off, const Geo& g, float* x, float* v, cudaStream_t st) {
   if (in.n == 0) return cudaSuccess;
-  k_decompress<<<grid_for(in.n, 256), 256, 0, st>>>(in, off, g, x, v);
+  k_decompress<<<grid_for(in.n, kDecChunk), kDecThreads, 0, st>>>(in, off, g, x, v);
   note_launches(1);
   return cudaGetLastError();
 }

@@ -59,3 +59,23 @@ def test_deposits_of_float_particles(n, order):
         ref = mesh.cic_deposit(x, w[:, q].astype(np.float64), N)
         scale = np.sqrt(np.mean(mesh.cic_deposit(x, np.abs(w[:, q]).astype(np.float64), N) ** 2))
         assert np.sqrt(np.mean((f[q] - ref) ** 2)) < DENSITY_TOL * scale
+
+
+# chunks of 2,048 particles: dense (a few cells), sparse (more cells than a chunk keeps), one heavy cell, remainders
+@pytest.mark.parametrize("vel_bits", [8, 16])
+@pytest.mark.parametrize("n_cdm,heavy", [(1, 0), (700, 0), (2049, 5000), (300007, 9000)])
+def test_decompress_chunks(n_cdm, heavy, vel_bits):
+    from oracle import codec
+    from paper_1611_01545_gb300 import PM
+    from tests.helpers import lib_codes_from_oracle
+    pm = PM(dict(n_fine=N, coarse_ratio=1, tile=N, buffer=0, cmp_ratio=4, vel_bits=vel_bits, G=FOUR_PI_G_ONE,
+                 mass=(8.0, 0.04), count=(0, 0)))
+    x = _positions(n_cdm, "random")
+    x = np.concatenate([x, np.full((heavy, 3), 33.25, np.float32)])
+    v = np.random.default_rng(5).standard_normal(x.shape).astype(np.float32)
+    ref = codec.compress(x, v, N, N // 4, vel_bits)
+    xd, vd = pm.decompress(0, lib_codes_from_oracle(ref))
+    pm.check()
+    xr, vr = codec.decompress(ref, N)
+    np.testing.assert_array_equal(xd.cpu().numpy(), xr)
+    np.testing.assert_array_equal(vd.cpu().numpy(), vr)
