@@ -163,7 +163,7 @@ def step_model_bytes(cfg, counts, vel_bits):
 
 
 # CUDA sources that define each kernel kind (its code and its launcher)
-_PARTICLE_SOURCES = ("particles.cu", "particles.cuh", "pm_common.cuh")
+_PARTICLE_SOURCES = ("particles.cu", "kick.cu", "blocks.cuh", "cic.cuh", "particles.cuh", "pm_common.cuh")
 _SOLVE_SOURCES = ("solve.cu", "fft.cuh", "tma.cuh", "pm_common.cuh")
 KIND_SOURCES = {"deposit": _PARTICLE_SOURCES, "ikd_count": _PARTICLE_SOURCES, "ikd_scatter": _PARTICLE_SOURCES,
                 "fft_a_tiles": _SOLVE_SOURCES, "fft_b_tiles": _SOLVE_SOURCES, "fft_c_tiles": _SOLVE_SOURCES}

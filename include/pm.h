@@ -453,7 +453,9 @@ int pm_set_graphs(pm_handle_t* h, int on);
  *                      drift + recompress passes;
  *  kick_window         half-width in cells of the new-cell window whose
  *                      counts a CTA keeps in shared memory (1..4; particles
- *                      moving further use global counters);
+ *                      moving further use global counters); the library uses
+ *                      a narrower one when the tables of the asked one would
+ *                      exceed 256 MB and a quarter of the particle scratch;
  *  kick_persistent     as deposit_persistent, for those passes;
  *  tile_batch          fine tiles per solve launch, 1..the configured batch.
  * Every block edge must divide n_cmp and the shared memory must fit one block

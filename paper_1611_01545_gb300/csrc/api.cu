@@ -34,7 +34,10 @@ struct pm_handle {
   float* acc_c = nullptr;
   int64_t* off[2] = {nullptr, nullptr};
   int64_t* newoff[2] = {nullptr, nullptr};
-  uint32_t* counts[2] = {nullptr, nullptr};
+  uint32_t* counts[2] = {nullptr, nullptr};   // new-cell counts (a step: of the window movers)
+  uint32_t* far[2] = {nullptr, nullptr};      // a step's far movers per new cell
+  uint32_t* start = nullptr;                  // start of each cell block's share of its window cells
+  size_t start_bytes = 0;
   uint32_t* vmax_bits = nullptr;  // [2]; one allocation with amax and work, cleared together by a step's first scan
   uint32_t* amax = nullptr;       // [3] max |a| over the coarse / fine force meshes and the PP accelerations (float bits)
   float4* app = nullptr;          // per particle PP acceleration (pp = 1), stream order, species 0 first
@@ -263,7 +266,7 @@ Blk choose_blk(const Geom& g, bool fixed, bool deposit) {
   b.D = 2;
   Geo geo{g.nf, g.rc, g.nc, g.rcmp, g.ncmp, g.ncell(), g.two};
   if (!deposit) {
-    while (b.RX > 1 && b.RX % 2 == 0 && ikd_count_smem(geo, b) > 100 * 1024) b.RX /= 2;
+    while (b.RX > 1 && b.RX % 2 == 0 && kick_count_smem(geo, b) > 100 * 1024) b.RX /= 2;
   } else {
     while (b.RX > 1 && b.RX % 2 == 0 && deposit_codes_smem(geo, b, fixed) > 64 * 1024) b.RX /= 2;
   }
@@ -282,8 +285,35 @@ Blk dep_blk(const pm_handle* h) {
   b.brick = block_brick(b);
   return b;
 }
+// Bytes that the start tables may take: a quarter of the per-particle scratch,
+// or 256 MB where that is more.
+size_t table_budget(const pm_handle* h) {
+  const size_t q = (size_t)h->scratch_n * 16 / 4;
+  return q > ((size_t)256 << 20) ? q : (size_t)256 << 20;
+}
+// Makes room for the start tables of kick block b.
+cudaError_t reserve_tables(pm_handle* h, Blk b) {
+  if (h->scratch_n == 0) return cudaSuccess;   // no particles, no tables
+  b.D = table_window(h->geo, b, table_budget(h));
+  const size_t need = table_bytes(h->geo, b);
+  if (need <= h->start_bytes) return cudaSuccess;
+  void* p = nullptr;
+  const cudaError_t e = cudaMalloc(&p, need);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return e;
+  }
+  if (h->start) cudaFree(h->start);   // waits for the work that uses it
+  h->start = static_cast<uint32_t*>(p);
+  h->start_bytes = need;
+  return cudaSuccess;
+}
+RecompressTables tables(const pm_handle* h) {
+  return RecompressTables{h->counts[0], h->counts[1], h->far[0], h->far[1], h->start, 0};
+}
 Blk ikd_blk(const pm_handle* h, int pass) {
   Blk b = h->blk_ikd;
+  b.D = table_window(h->geo, b, table_budget(h));
   b.work = h->persist_ikd ? h->work + 1 + pass : nullptr;
   b.brick = block_brick(b);
   return b;
@@ -449,6 +479,7 @@ int pm_init(const pm_config_t* cfg, pm_handle_t** out) {
     A(&h->off[s], (ncell + 1) * 8);
     A(&h->newoff[s], (ncell + 1) * 8);
     A(&h->counts[s], ncell * 4);
+    A(&h->far[s], ncell * 4);
   }
   A(&h->vmax_bits, kSmallWords * 4);
   if (rc == PM_OK) {
@@ -512,6 +543,10 @@ int pm_init(const pm_config_t* cfg, pm_handle_t** out) {
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
     h->smem_optin = optin > 1024 ? (size_t)optin - 1024 : 0;   // room for the kernels' static shared memory
   }
+  if (rc == PM_OK) {
+    const cudaError_t e = reserve_tables(h, h->blk_ikd);
+    if (e != cudaSuccess) rc = fail(h, PM_ERR_CUDA, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+  }
   if (rc != PM_OK) {
     fprintf(stderr, "pm_init: %s\n", h->err.c_str());
     pm_destroy(h);
@@ -542,6 +577,7 @@ int pm_destroy(pm_handle_t* h) {
   h->timer.flush();
   for (auto e : h->timer.pool) cudaEventDestroy(e);
   for (void* p : h->allocs) cudaFree(p);
+  if (h->start) cudaFree(h->start);
   delete h;
   return PM_OK;
 }
@@ -613,7 +649,7 @@ int pm_deposit_codes(pm_handle_t* h, const pm_codes_t in[2], void* rho_coarse, v
   cudaStream_t st = (cudaStream_t)stream;
   const bool fixed = h->cfg.deposit_mode == 1;
   const bool vel16 = h->cfg.vel_bits == 16;
-  const ScanClear clear{{nullptr, nullptr}, h->vmax_bits, kSmallWords};
+  const ScanClear clear{{nullptr, nullptr}, {nullptr, nullptr}, h->vmax_bits, kSmallWords};
   CK(h, scan_codes2(in, h->gm.ncell(), h->off[0], h->off[1], h->scan_state, h->status, &clear, st));
   long long M0 = llrint(h->cfg.mass[0] * 4294967296.0), M1 = llrint(h->cfg.mass[1] * 4294967296.0);
   CK(h, launch_deposit_codes(view(in[0], vel16), view(in[1], vel16), h->off[0], h->off[1], h->geo, dep_blk(h),
@@ -846,7 +882,7 @@ bool blk_fits(const pm_handle* h, const Blk& b, bool deposit) {
   if (b.RX < 1 || b.RY < 1 || b.RZ < 1 || n % b.RX || n % b.RY || n % b.RZ) return false;
   if (b.D < 1 || b.D > 4) return false;
   if (deposit) return deposit_codes_smem(h->geo, b, h->cfg.deposit_mode == 1) <= h->smem_optin;
-  return ikd_count_smem(h->geo, b) <= h->smem_optin && ikd_scatter_smem(h->geo, b) <= h->smem_optin;
+  return kick_count_smem(h->geo, b) <= h->smem_optin && kick_scatter_smem(h->geo, b) <= h->smem_optin;
 }
 
 Blk make_blk(const pm_handle* h, const int32_t r[3], int D) {
@@ -879,6 +915,7 @@ int apply_tuning(pm_handle* h, const pm_tuning_t* t) {
     return fail(h, PM_ERR_ARG, "tile_batch must lie in [1, the configured tile batch]");
   if ((t->deposit_persistent & ~1) || (t->kick_persistent & ~1)) return fail(h, PM_ERR_ARG, "persistent flags are 0 or 1");
   drop_graphs(h);
+  CK(h, reserve_tables(h, bi));
   h->blk_dep = bd;
   h->blk_ikd = bi;
   h->persist_dep = t->deposit_persistent != 0;
@@ -1024,7 +1061,7 @@ int step_launch(pm_handle_t* h, const pm_codes_t in[2], pm_codes_t out[2], doubl
   const int64_t ncell = g.ncell();
   {
     TimedScope ts(tm, "scan_in", st);
-    const ScanClear clear{{h->counts[0], h->counts[1]}, h->vmax_bits, kSmallWords};
+    const ScanClear clear{{h->counts[0], h->counts[1]}, {h->far[0], h->far[1]}, h->vmax_bits, kSmallWords};
     CK(h, scan_codes2(in, ncell, h->off[0], h->off[1], h->scan_state, h->status, &clear, st));
   }
   void* rc = fixed ? (void*)h->rho_c_fix : (void*)h->rho_c;
@@ -1059,23 +1096,23 @@ int step_launch(pm_handle_t* h, const pm_codes_t in[2], pm_codes_t out[2], doubl
   if (bound) CK(h, launch_vmax_bound(in[0].vmax, in[1].vmax, h->amax, ck, out[0].vmax, out[1].vmax, st));
   {
     TimedScope ts(tm, "ikd_count", st);
-    CK(h, launch_ikd_count(view(in[0], vel16), view(in[1], vel16), h->off[0], h->off[1], h->geo, ikd_blk(h, 0),
-                           h->acc_c, h->acc_f, ck, cd, h->counts[0], h->counts[1], h->vmax_bits, h->tkey, h->tpv,
-                           bound ? out[0].vmax : nullptr, bound ? out[1].vmax : nullptr, h->cfg.pp ? h->app : nullptr,
-                           !via_fine, st));
+    CK(h, launch_kick_count(view(in[0], vel16), view(in[1], vel16), h->off[0], h->off[1], h->geo, ikd_blk(h, 0),
+                            h->acc_c, h->acc_f, ck, cd, tables(h), h->vmax_bits, h->tkey, h->tpv,
+                            bound ? out[0].vmax : nullptr, bound ? out[1].vmax : nullptr, h->cfg.pp ? h->app : nullptr,
+                            !via_fine, st));
   }
   if (h->post_count_record) CK(h, cudaEventRecord(h->post_count_record, st));
   {
     TimedScope ts(tm, "scan_out", st);
     const int64_t expect[2] = {in[0].n, in[1].n};
-    CK(h, scan_counts2(h->counts[0], h->counts[1], ncell, expect, h->newoff[0], h->newoff[1], out,
+    CK(h, scan_counts2(h->counts, h->far, ncell, expect, h->newoff[0], h->newoff[1], out,
                        bound ? nullptr : h->vmax_bits, h->scan_state, h->status, st));
   }
   {
     TimedScope ts(tm, "ikd_scatter", st);
     PCodesOut o0 = oview(out[0], vel16), o1 = oview(out[1], vel16);
-    CK(h, launch_ikd_scatter(in[0].n, in[1].n, h->off[0], h->off[1], h->geo, ikd_blk(h, 1), h->counts[0], h->counts[1],
-                             h->newoff[0], h->newoff[1], o0, o1, h->tkey, h->tpv, bound, h->status, st));
+    CK(h, launch_kick_scatter(in[0].n, in[1].n, h->off[0], h->off[1], h->geo, ikd_blk(h, 1), tables(h), h->newoff[0],
+                              h->newoff[1], o0, o1, h->tkey, h->tpv, bound, h->status, st));
   }
   return PM_OK;
 }

@@ -42,9 +42,10 @@ struct PCodesOut {
 // when it is allocated (each launch leaves it zero again).
 size_t scan_state_bytes(int64_t ncell);
 // Arrays that a step's first scan clears on the way: the new-cell counts of
-// both species and `small_words` 32-bit words (null: nothing).
+// both species, window and far movers, and `small_words` 32-bit words (null: nothing).
 struct ScanClear {
   uint32_t* counts[2];
+  uint32_t* far[2];
   uint32_t* small;
   int small_words;
 };
@@ -55,7 +56,8 @@ cudaError_t scan_counts(const uint32_t* counts, int64_t ncell, int64_t expect, i
 // Both species in one launch (2 scan_state_bytes of state).
 cudaError_t scan_codes2(const pm_codes_t in[2], int64_t ncell, int64_t* off0, int64_t* off1, void* state, int* status,
                         const ScanClear* clear, cudaStream_t st);
-cudaError_t scan_counts2(const uint32_t* counts0, const uint32_t* counts1, int64_t ncell, const int64_t expect[2],
+// (counts: far movers apart)
+cudaError_t scan_counts2(const uint32_t* const counts[2], const uint32_t* const far[2], int64_t ncell, const int64_t expect[2],
                          int64_t* off0, int64_t* off1, pm_codes_t out[2], const uint32_t* vmax_bits, void* state,
                          int* status, cudaStream_t st);
 
@@ -74,23 +76,35 @@ cudaError_t launch_compress(const float* x, const float* v, int64_t n, const Geo
                             uint32_t* vmax_bits, const float* vmax_in, int64_t* off, pm_codes_t& out, bool vel16,
                             void* scan_state, int* status, cudaStream_t st);
 size_t deposit_codes_smem(const Geo& g, const Blk& bk, bool fixed);
-size_t ikd_count_smem(const Geo& g, const Blk& bk);
-size_t ikd_scatter_smem(const Geo& g, const Blk& bk);
+// Recompress passes (kick.cu).
+size_t kick_count_smem(const Geo& g, const Blk& bk);
+size_t kick_scatter_smem(const Geo& g, const Blk& bk);
 int window_cells(const Geo& g, const Blk& bk);
+// New-cell tables between the count pass and the scatter, per species: window
+// movers and far movers per cell, and the start of each block's share.
+struct RecompressTables {
+  uint32_t* counts0;
+  uint32_t* counts1;
+  uint32_t* far0;
+  uint32_t* far1;
+  uint32_t* start;   // null: no particles
+  int kb;            // rank bits of a key (set by the launchers)
+};
+size_t table_bytes(const Geo& g, const Blk& bk);
+int table_window(const Geo& g, Blk bk, size_t budget);
 // Brick edge (block rows) of the block order for a block grid (1: row order).
 int block_brick(const Blk& bk);
 cudaError_t launch_deposit_codes(const PCodes& c0, const PCodes& c1, const int64_t* off0, const int64_t* off1,
                                  const Geo& g, const Blk& bk, float m0, float m1, long long M0, long long M1,
                                  void* rho_c, void* rho_f, bool fixed, cudaStream_t st);
-cudaError_t launch_ikd_count(const PCodes& c0, const PCodes& c1, const int64_t* off0, const int64_t* off1,
-                             const Geo& g, const Blk& bk, const float* acc_c, const float* acc_f, float ck, float cd,
-                             uint32_t* counts0, uint32_t* counts1, uint32_t* vmax_bits, uint32_t* tkey,
-                             uint4* tpv, const float* vq0, const float* vq1, const float4* app, bool coarse,
-                             cudaStream_t st);
-cudaError_t launch_ikd_scatter(int64_t n0, int64_t n1, const int64_t* off0, const int64_t* off1, const Geo& g,
-                               const Blk& bk, uint32_t* counts0, uint32_t* counts1, const int64_t* newoff0,
-                               const int64_t* newoff1, const PCodesOut& o0, const PCodesOut& o1, const uint32_t* tkey,
-                               const uint4* tpv, bool coded, int* status, cudaStream_t st);
+cudaError_t launch_kick_count(const PCodes& c0, const PCodes& c1, const int64_t* off0, const int64_t* off1,
+                              const Geo& g, const Blk& bk, const float* acc_c, const float* acc_f, float ck, float cd,
+                              const RecompressTables& t, uint32_t* vmax_bits, uint32_t* tkey, uint4* tpv,
+                              const float* vq0, const float* vq1, const float4* app, bool coarse, cudaStream_t st);
+cudaError_t launch_kick_scatter(int64_t n0, int64_t n1, const int64_t* off0, const int64_t* off1, const Geo& g,
+                                const Blk& bk, const RecompressTables& t, const int64_t* newoff0,
+                                const int64_t* newoff1, const PCodesOut& o0, const PCodesOut& o1, const uint32_t* tkey,
+                                const uint4* tpv, bool coded, int* status, cudaStream_t st);
 // v_max' bound of both species from v_max and the maxima amax[3] (coarse mesh,
 // fine mesh, PP accelerations; float bits).
 // PP acceleration (Eq. 4) of every particle of both species into acc[t] (stream index t,

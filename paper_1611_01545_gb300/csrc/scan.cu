@@ -184,15 +184,21 @@ struct CodesCount {
 // Counts of the recompressed cells (library memory, 16-byte aligned).
 struct U32Count {
   const uint32_t* cnt;
+  const uint32_t* far;   // counted apart, or null
   static __device__ V2 of(uint32_t k) { return V2{(long long)k, k >= 255u ? 1 : 0}; }
   __device__ void load(int64_t c, int64_t n, V2 (&v)[SCAN_ITEMS]) const {
     if (c + SCAN_ITEMS <= n) {
-      const uint4 p = reinterpret_cast<const uint4*>(cnt + c)[0], q = reinterpret_cast<const uint4*>(cnt + c)[1];
+      uint4 p = reinterpret_cast<const uint4*>(cnt + c)[0], q = reinterpret_cast<const uint4*>(cnt + c)[1];
+      if (far) {
+        const uint4 a = reinterpret_cast<const uint4*>(far + c)[0], b = reinterpret_cast<const uint4*>(far + c)[1];
+        p = make_uint4(p.x + a.x, p.y + a.y, p.z + a.z, p.w + a.w);
+        q = make_uint4(q.x + b.x, q.y + b.y, q.z + b.z, q.w + b.w);
+      }
       v[0] = of(p.x); v[1] = of(p.y); v[2] = of(p.z); v[3] = of(p.w);
       v[4] = of(q.x); v[5] = of(q.y); v[6] = of(q.z); v[7] = of(q.w);
     } else {
 #pragma unroll
-      for (int k = 0; k < SCAN_ITEMS; ++k) v[k] = c + k < n ? of(cnt[c + k]) : V2{0, 0};
+      for (int k = 0; k < SCAN_ITEMS; ++k) v[k] = c + k < n ? of(cnt[c + k] + (far ? far[c + k] : 0u)) : V2{0, 0};
     }
   }
   __device__ void validate(int, int, int64_t) const {}
@@ -218,15 +224,20 @@ __device__ __forceinline__ void put_offsets(int64_t* off, int64_t c, int64_t n, 
 struct PutOffsets {
   int64_t* off;
   uint32_t* clear;
+  uint32_t* clear2;
   __device__ void operator()(int64_t c, int64_t n, V2 ex, const V2 (&v)[SCAN_ITEMS]) const {
     put_offsets(off, c, n, ex, v);
-    if (!clear) return;
+    put_zeros(clear, c, n);
+    put_zeros(clear2, c, n);
+  }
+  static __device__ __forceinline__ void put_zeros(uint32_t* a, int64_t c, int64_t n) {
+    if (!a) return;
     if (c + SCAN_ITEMS <= n) {
-      reinterpret_cast<uint4*>(clear + c)[0] = make_uint4(0, 0, 0, 0);
-      reinterpret_cast<uint4*>(clear + c)[1] = make_uint4(0, 0, 0, 0);
+      reinterpret_cast<uint4*>(a + c)[0] = make_uint4(0, 0, 0, 0);
+      reinterpret_cast<uint4*>(a + c)[1] = make_uint4(0, 0, 0, 0);
     } else {
       for (int k = 0; k < SCAN_ITEMS; ++k)
-        if (c + k < n) clear[c + k] = 0;
+        if (c + k < n) a[c + k] = 0;
     }
   }
 };
@@ -348,7 +359,7 @@ cudaError_t scan_codes_n(const pm_codes_t* in, int nsp, int64_t ncell, int64_t* 
   Pair<FinishArgs> fin{};
   for (int s = 0; s < nsp; ++s) {
     get.v[s] = CodesCount{in[s].cnt, in[s].esc, in[s].n_esc, in[s].esc_cap, in[s].vmax, status};
-    put.v[s] = PutOffsets{off[s], clear ? clear->counts[s] : nullptr};
+    put.v[s] = PutOffsets{off[s], clear ? clear->counts[s] : nullptr, clear ? clear->far[s] : nullptr};
     fin.v[s] = FinishArgs{in[s].n, off[s], nullptr, 0, nullptr, nullptr, s == 0 && clear ? clear->small : nullptr,
                           s == 0 && clear ? clear->small_words : 0};
   }
@@ -359,14 +370,14 @@ cudaError_t scan_codes_n(const pm_codes_t* in, int nsp, int64_t ncell, int64_t* 
   return cudaGetLastError();
 }
 
-cudaError_t scan_counts_n(const uint32_t* const* counts, int nsp, int64_t ncell, const int64_t* expect,
+cudaError_t scan_counts_n(const uint32_t* const* counts, const uint32_t* const* far, int nsp, int64_t ncell, const int64_t* expect,
                           int64_t* const* off, pm_codes_t* out, const uint32_t* const* vmax_bits, void* state,
                           int* status, cudaStream_t st) {
   Pair<U32Count> get{};
   Pair<PutCodes> put{};
   Pair<FinishArgs> fin{};
   for (int s = 0; s < nsp; ++s) {
-    get.v[s] = U32Count{counts[s]};
+    get.v[s] = U32Count{counts[s], far ? far[s] : nullptr};
     put.v[s] = PutCodes{off[s], out[s].cnt, out[s].esc, out[s].esc_cap, status};
     fin.v[s] = FinishArgs{expect[s], off[s], out[s].n_esc, out[s].esc_cap, vmax_bits[s],
                           vmax_bits[s] ? out[s].vmax : nullptr, nullptr, 0};
@@ -400,16 +411,15 @@ cudaError_t scan_counts(const uint32_t* counts, int64_t ncell, int64_t expect, i
   const uint32_t* c[1] = {counts};
   const uint32_t* vb[1] = {vmax_bits};
   int64_t* o[1] = {off};
-  return scan_counts_n(c, 1, ncell, &expect, o, &out, vb, state, status, st);
+  return scan_counts_n(c, nullptr, 1, ncell, &expect, o, &out, vb, state, status, st);
 }
 
-cudaError_t scan_counts2(const uint32_t* counts0, const uint32_t* counts1, int64_t ncell, const int64_t expect[2],
-                         int64_t* off0, int64_t* off1, pm_codes_t out[2], const uint32_t* vmax_bits, void* state,
-                         int* status, cudaStream_t st) {
-  const uint32_t* c[2] = {counts0, counts1};
+cudaError_t scan_counts2(const uint32_t* const counts[2], const uint32_t* const far[2], int64_t ncell,
+                         const int64_t expect[2], int64_t* off0, int64_t* off1, pm_codes_t out[2],
+                         const uint32_t* vmax_bits, void* state, int* status, cudaStream_t st) {
   const uint32_t* vb[2] = {vmax_bits, vmax_bits ? vmax_bits + 1 : nullptr};
   int64_t* o[2] = {off0, off1};
-  return scan_counts_n(c, 2, ncell, expect, o, out, vb, state, status, st);
+  return scan_counts_n(counts, far, 2, ncell, expect, o, out, vb, state, status, st);
 }
 
 }  // namespace pm
