@@ -32,10 +32,12 @@ template <int N> struct SolveCfg {
 #define PM_SOLVE_THREADS 512
 #endif
 #ifndef PM_SOLVE_C_THREADS
-#define PM_SOLVE_C_THREADS 384
+#define PM_SOLVE_C_THREADS 416
+#endif
+#ifndef PM_SOLVE_C_MINB
+#define PM_SOLVE_C_MINB 3
 #endif
   static constexpr int threads = (N >= 96) ? PM_SOLVE_THREADS : 256;
-  static constexpr int threads_c = (N >= 96) ? PM_SOLVE_C_THREADS : 256;
   static constexpr size_t smem_a = sizeof(float2) * (N + (size_t)N * N / 2 + (size_t)N * NP);
 };
 
@@ -310,153 +312,6 @@ __global__ void __launch_bounds__(PassB<N>::threads) k_solve_b_adj(SolveArgs a) 
   }
 }
 
-template <int N>
-__device__ __forceinline__ void solve_c_body(const SolveArgs& a, float2* tw, float2* P, float2* W);
-
-template <int N>
-__global__ void __launch_bounds__(SolveCfg<N>::threads_c) k_solve_c(SolveArgs a) {
-  constexpr int NP = SolveCfg<N>::NP;
-  extern __shared__ float2 sm[];
-  float2* tw = sm;
-  float2* P = sm + N;          // [y][kx], pitch NP
-  float2* W = P + N * NP;      // t/2 packed rows of N
-  for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = a.tw[i];
-  const int zo = blockIdx.x;
-  const int d = blockIdx.y;
-  const int pb = blockIdx.z;
-  const float4* in = reinterpret_cast<const float4*>(a.spec3 + (((size_t)pb * 3 + d) * a.t + zo) * N * NP);
-  float4* P4 = reinterpret_cast<float4*>(P);
-  for (int i = threadIdx.x; i < N * NP / 2; i += blockDim.x) async_copy16(P4 + i, in + i);
-  async_wait();
-  __syncthreads();
-  solve_c_body<N>(a, tw, P, W);
-}
-
-// Pass C after its input plane is in P: inverse y transform, the packed
-// inverse x transform of the output rows, the prolongated coarse force, the
-// output store and the running max |a|.
-template <int N>
-__device__ __forceinline__ void solve_c_body(const SolveArgs& a, float2* tw, float2* P, float2* W) {
-  constexpr int NH = SolveCfg<N>::NH, NP = SolveCfg<N>::NP;
-  const int zo = blockIdx.x;
-  const int d = blockIdx.y;
-  const int pb = blockIdx.z;
-  fft_inv<N, NH, 1, NP>(P, tw);
-  const int half_rows = a.t / 2;
-  // Inverse x transforms of the output rows, two real rows (b + 2j, b + 2j + 1)
-  // packed as one complex row A + i B (A, B their half spectra, extended by
-  // conjugate symmetry).  Step 1 forms its inputs from P directly: slot
-  // N2 k1 + k2 holds frequency k = k1 + N1 k2.
-  {
-    constexpr int N1 = Factor<N>::N1, N2 = Factor<N>::N2;
-    for (int w = threadIdx.x; w < half_rows * N1; w += blockDim.x) {
-      const int j = w / N1, k1 = w - j * N1;
-      const float2* Pa = P + (a.b + 2 * j) * NP;
-      const float2* Pb = Pa + NP;
-      float2 v[N2];
-#pragma unroll
-      for (int k2 = 0; k2 < N2; ++k2) {
-        const int k = k1 + N1 * k2;
-        float2 A, B;
-        if (k <= N / 2) {
-          A = Pa[k];
-          B = Pb[k];
-        } else {
-          A = conjf2(Pa[N - k]);
-          B = conjf2(Pb[N - k]);
-        }
-        v[k2] = make_float2(A.x - B.y, A.y + B.x);   // A + i B
-      }
-      Dft<N2, 1>::run(v);
-#pragma unroll
-      for (int j2 = 1; j2 < N2; ++j2) v[j2] = cmul(v[j2], conjf2(tw[j2 * k1]));
-      float2* base = W + j * N;
-#pragma unroll
-      for (int j2 = 0; j2 < N2; ++j2) base[N2 * k1 + j2] = v[j2];
-    }
-    __syncthreads();
-    for (int w = threadIdx.x; w < half_rows * N2; w += blockDim.x) {
-      const int q = w / N2, j2 = w - q * N2;
-      float2* base = W + q * N;
-      float2 v[N1];
-#pragma unroll
-      for (int k1 = 0; k1 < N1; ++k1) v[k1] = base[N2 * k1 + j2];
-      Dft<N1, 1>::run(v);
-#pragma unroll
-      for (int j1 = 0; j1 < N1; ++j1) base[N2 * j1 + j2] = v[j1];
-    }
-    __syncthreads();
-  }
-  int ox, oy, oz;
-  problem_origin(a, a.p0 + pb, ox, oy, oz);
-  const int n = a.src_n;
-  // Prolongation of the coarse force onto this output plane: the coarse values
-  // around the tile interior, interpolated in z, staged in P (free by now),
-  // then along x onto the output columns (R), so an output cell needs one
-  // interpolation in y.
-  float* Q = reinterpret_cast<float*>(P);
-  const int nq = a.pc ? a.t / a.prc + 1 : 0;
-  float* R = Q + nq * nq;   // [nq][t]
-  int lr = 0;
-  float inv_r = 0.f;
-  if (a.pc) {
-    lr = __ffs(a.prc) - 1;
-    inv_r = 1.0f / (float)a.prc;
-    const int gz = oz + a.b + zo;
-    const int cz0 = gz >> lr, cz1 = cz0 + 1 == a.pnc ? 0 : cz0 + 1;
-    const float wz = (float)(gz & (a.prc - 1)) * inv_r;
-    const int cyb = (oy + a.b) >> lr, cxb = (ox + a.b) >> lr;
-    const float* c0 = a.pc + ((size_t)d * a.pnc + cz0) * a.pnc * a.pnc;
-    const float* c1 = a.pc + ((size_t)d * a.pnc + cz1) * a.pnc * a.pnc;
-    PM_ROWS(qy, nq) {
-      int cy = cyb + qy;
-      if (cy >= a.pnc) cy -= a.pnc;
-      PM_COLS(qx, nq) {
-        int cx = cxb + qx;
-        if (cx >= a.pnc) cx -= a.pnc;
-        const size_t o = (size_t)cy * a.pnc + cx;
-        Q[qy * nq + qx] = (1.0f - wz) * __ldg(c0 + o) + wz * __ldg(c1 + o);
-      }
-    }
-    __syncthreads();
-    PM_ROWS(qy, nq) {
-      const float* q = Q + qy * nq;
-      PM_COLS(xl, a.t) {
-        const int qx = xl >> lr;
-        const float fx = (float)(xl & (a.prc - 1)) * inv_r;
-        R[qy * a.t + xl] = fmaf(fx, q[qx + 1] - q[qx], q[qx]);
-      }
-    }
-    __syncthreads();
-  }
-  // Output cells are interior cells: origin + b + local lies inside [0, n) without wrap.
-  const int gz = oz + a.b + zo;
-  float* dst = a.dst + (size_t)d * n * n * n + ((int64_t)gz * n + oy + a.b) * n + ox + a.b;
-  float m = 0.f;
-  PM_ROWS(yl, a.t) {
-    const float* w = reinterpret_cast<const float*>(W + (yl >> 1) * N + a.b) + (yl & 1);
-    float* drow = dst + (int64_t)yl * n;
-    PM_COLS(xl, a.t) {
-      float val = w[2 * xl];
-      m = fmaxf(m, fabsf(val));
-      if (a.pc) {
-        const int qy = yl >> lr;
-        const float fy = (float)(yl & (a.prc - 1)) * inv_r;
-        const float lo = R[qy * a.t + xl], hi = R[(qy + 1) * a.t + xl];
-        val += fmaf(fy, hi - lo, lo);
-      }
-      drow[xl] = val;
-    }
-  }
-  if (a.amax) {
-    // warp maximum; an atomic only when it raises the running maximum
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0 && m > __uint_as_float(*(volatile unsigned int*)a.amax))
-      atomicMax(a.amax, __float_as_uint(m));
-  }
-}
-
 // ---- 96^3 passes staged by the tensor memory accelerator ----------------
 //
 // The 96^3 transforms (the buffered fine tiles, and a 96^3 periodic mesh)
@@ -472,7 +327,6 @@ __device__ __forceinline__ void solve_c_body(const SolveArgs& a, float2* tw, flo
 //      the forward z transform, the three kernel products and the first step
 //      of each inverse transform run in registers per (column, k1) item; the
 //      output z range of each component leaves as one box store;
-//   C  the input plane arrives as one bulk copy.
 // Spectrum rows are padded to spec_pitch(96) = 50 complex values (400
 // bytes), so rows, boxes and planes start on 16-byte boundaries.
 
@@ -673,36 +527,247 @@ __global__ void __launch_bounds__(PassBT<N>::threads, PM_PASSB_TMA_MINB)
   }
 }
 
-template <int N> struct PassCT {
-  // P [N][NP], W [N/2][N], twiddles
-  static constexpr size_t smem = kTmaAlign + sizeof(float2) * ((size_t)N * spec_pitch(N) + (size_t)N / 2 * N + N);
+// ---- pass C ---------------------------------------------------------------
+//
+// One block per (output z, component): the plane's inverse y transform, the
+// packed inverse x transform of the output rows, the prolongated coarse force,
+// the store and the running max |a|.  What bounds it is shared memory: the
+// earlier form moved 5,280 128-byte wavefronts per 96^3 tile plane, 1,650 of
+// them bank conflicts, at 75% of the load/store pipe, and took 0.288 ms for 64
+// tiles (0.226 without the prolongation).  Here
+//   * an item of the second y step transforms two neighbouring rows at once
+//     and writes only the output rows, both rows of a packed pair in one
+//     16-byte word [pair][kx];
+//   * the x steps give a warp's lanes different pairs (pitches NH 16-byte words
+//     and N + 1 complex values, both odd, so 8 or 16 lanes fall in different
+//     banks) where lanes along a row met 2 to 4 deep in a bank;
+//   * the output takes a pair's two rows from one 8-byte word and one pair of
+//     prolongation reads.
+// 2,600 wavefronts per plane: 0.244 ms (0.18 without the prolongation); 216
+// tiles of 48^3: 0.182 -> 0.143 ms.
+// N = 128 keeps the y rows in place and the x step in registers across a
+// barrier (one buffer of 67 KB instead of two), so that 2 blocks share an SM:
+// 128^3 mesh 33 -> 21 us.
+
+template <int N> struct PassC {
+  static constexpr int N1 = Factor<N>::N1, N2 = Factor<N>::N2;
+  static constexpr int NH = N / 2 + 1, NP = spec_pitch(N);
+  static constexpr bool in_place = N >= 128;
+  // one round of the largest item sets; the last warp of 96, 64 and 128 takes the column at kx = N / 2
+  static constexpr int threads = N == 128 ? 544 : (N == 96 ? PM_SOLVE_C_THREADS : (N == 64 ? 288 : (N == 48 ? 160 : 96)));
+  static constexpr int min_blocks = N == 128 ? 2 : (N == 96 ? PM_SOLVE_C_MINB : 4);
+  static constexpr size_t align = 128;
+  // P [N][NP] (then W [pairs][N + 1]), twiddles, Y [pairs][NH] 16-byte words or, in place, room for the prolongation
+  static size_t smem(int t, int b, int prc, bool prolong) {
+    const size_t pairs = pair_count(t, b);
+    const size_t nq = prolong ? t / prc + 1 : 0;
+    return align + sizeof(float2) * ((size_t)N * NP + N) + (in_place ? 4 * (nq * nq + nq * t) : 16 * pairs * NH);
+  }
+  static size_t smem_max() { return align + sizeof(float2) * ((size_t)N * NP + N) + (size_t)16 * (N / 2) * NH; }
+  // row pairs (2 m, 2 m + 1) that hold the output rows b .. b + t - 1
+  static __host__ __device__ __forceinline__ int pair_count(int t, int b) { return ((b + t - 1) >> 1) - (b >> 1) + 1; }
 };
 
-#ifndef PM_SOLVE_C_MINB
-#define PM_SOLVE_C_MINB 3
-#endif
 template <int N>
-__global__ void __launch_bounds__(SolveCfg<N>::threads_c, PM_SOLVE_C_MINB) k_solve_c_tma(SolveArgs a) {
-  constexpr int NP = SolveCfg<N>::NP;
+__global__ void __launch_bounds__(PassC<N>::threads, PassC<N>::min_blocks) k_solve_c(SolveArgs a) {
+  using C = PassC<N>;
+  constexpr int N1 = C::N1, N2 = C::N2, NH = C::NH, NP = C::NP, WP = N + 1, T = C::threads;
   extern __shared__ unsigned char smraw_c[];
   __shared__ uint64_t bar;
   float2* P = reinterpret_cast<float2*>(tma_align(smraw_c));   // [y][NP]
-  float2* W = P + N * NP;                                        // t/2 packed rows of N
-  float2* tw = W + N * N / 2;
+  float2* W = P;                                                 // [pair][N + 1], once P is read
+  float2* tw = P + N * NP;
+  float4* Y = reinterpret_cast<float4*>(tw + N);                 // [pair][NH]: rows 2 m and 2 m + 1 at kx
   const int zo = blockIdx.x, d = blockIdx.y, pb = blockIdx.z;
+  const float2* in = a.spec3 + (((size_t)pb * 3 + d) * a.t + zo) * N * NP;
+  constexpr unsigned bytes = N * NP * (unsigned)sizeof(float2);
+  static_assert(bytes % 16 == 0, "planes of whole 16-byte words");
   if (threadIdx.x == 0) {
     tma::mbar_init(&bar, 1);
     tma::fence_barrier_init();
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    const unsigned bytes = N * NP * (unsigned)sizeof(float2);
     tma::mbar_arrive_expect_tx(&bar, bytes);
-    tma::bulk_load(P, a.spec3 + (((size_t)pb * 3 + d) * a.t + zo) * N * NP, bytes, &bar);
+    tma::bulk_load(P, in, bytes, &bar);
   }
-  for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = a.tw[i];
+  for (int i = threadIdx.x; i < N; i += T) tw[i] = a.tw[i];
   if (!block_wait(&bar, a.status)) return;
-  solve_c_body<N>(a, tw, P, W);
+  // inverse y transform, step 1: items (k1, column)
+  for (int w = threadIdx.x; w < N1 * NH; w += T) {
+    const int k1 = w / NH, c = w - k1 * NH;
+    float2* base = P + N2 * k1 * NP + c;
+    float2 v[N2];
+#pragma unroll
+    for (int k2 = 0; k2 < N2; ++k2) v[k2] = base[k2 * NP];
+    Dft<N2, 1>::run(v);
+#pragma unroll
+    for (int j2 = 1; j2 < N2; ++j2) v[j2] = cmul(v[j2], conjf2(tw[j2 * k1]));
+#pragma unroll
+    for (int j2 = 0; j2 < N2; ++j2) base[j2 * NP] = v[j2];
+  }
+  __syncthreads();
+  // step 2: items (two neighbouring j2, column) -> rows N2 j1 + j2 and the next
+  const int m0 = a.b >> 1, np = C::pair_count(a.t, a.b);
+  for (int w = threadIdx.x; w < (N2 / 2) * NH; w += T) {
+    const int jp = w / NH, c = w - jp * NH;
+    float2* base = P + 2 * jp * NP + c;
+    float2 u[N1], v[N1];
+#pragma unroll
+    for (int k1 = 0; k1 < N1; ++k1) {
+      u[k1] = base[N2 * k1 * NP];
+      v[k1] = base[(N2 * k1 + 1) * NP];
+    }
+    Dft<N1, 1>::run(u);
+    Dft<N1, 1>::run(v);
+#pragma unroll
+    for (int j1 = 0; j1 < N1; ++j1) {
+      if (C::in_place) {
+        base[N2 * j1 * NP] = u[j1];
+        base[(N2 * j1 + 1) * NP] = v[j1];
+      } else {
+        const int pair = (N2 / 2) * j1 + jp - m0;
+        if (pair >= 0 && pair < np) Y[pair * NH + c] = make_float4(u[j1].x, u[j1].y, v[j1].x, v[j1].y);
+      }
+    }
+  }
+  __syncthreads();
+  // inverse x transforms of the pairs, rows A and B packed as A + i B (A, B
+  // their half spectra, extended by conjugate symmetry).  Step 1: items (k1,
+  // pair), frequencies k = k1 + N1 k2.
+  {
+    static_assert(!C::in_place || (N / 2) * N1 <= T, "in place: one round");
+    for (int w0 = 0; w0 < np * N1; w0 += T) {
+      const int w = w0 + threadIdx.x;
+      const bool live = w < np * N1;
+      const int k1 = live ? w / np : 0, j = live ? w - k1 * np : 0;
+      float2 v[N2];
+#pragma unroll
+      for (int k2 = 0; k2 < N2; ++k2) {
+        const int k = k1 + N1 * k2;
+        const bool low = k2 < N2 / 2 || (k2 == N2 / 2 && k1 == 0);   // k <= N / 2
+        const int kk = low ? k : N - k;
+        float2 A, B;
+        if (C::in_place) {
+          A = P[2 * (m0 + j) * NP + kk];
+          B = P[(2 * (m0 + j) + 1) * NP + kk];
+        } else {
+          const float4 q = Y[j * NH + kk];
+          A = make_float2(q.x, q.y);
+          B = make_float2(q.z, q.w);
+        }
+        if (!low) {
+          A = conjf2(A);
+          B = conjf2(B);
+        }
+        v[k2] = make_float2(A.x - B.y, A.y + B.x);   // A + i B
+      }
+      Dft<N2, 1>::run(v);
+#pragma unroll
+      for (int j2 = 1; j2 < N2; ++j2) v[j2] = cmul(v[j2], conjf2(tw[j2 * k1]));
+      if (C::in_place) __syncthreads();   // every row is read before W overwrites it
+      if (live) {
+        float2* base = W + j * WP + N2 * k1;
+#pragma unroll
+        for (int j2 = 0; j2 < N2; ++j2) base[j2] = v[j2];
+      }
+    }
+  }
+  __syncthreads();
+  int ox, oy, oz;
+  problem_origin(a, a.p0 + pb, ox, oy, oz);
+  const int n = a.src_n;
+  // Prolongation of the coarse force onto this output plane: the coarse values
+  // around the tile interior, interpolated in z (Q; Y is free by now), then
+  // along x onto the output columns (R), so an output cell needs one
+  // interpolation in y.
+  float* Q = reinterpret_cast<float*>(Y);
+  const int nq = a.pc ? a.t / a.prc + 1 : 0;
+  float* R = Q + nq * nq;   // [nq][t]
+  int lr = 0;
+  float inv_r = 0.f;
+  if (a.pc) {
+    lr = __ffs(a.prc) - 1;
+    inv_r = 1.0f / (float)a.prc;
+    const int gz = oz + a.b + zo;
+    const int cz0 = gz >> lr, cz1 = cz0 + 1 == a.pnc ? 0 : cz0 + 1;
+    const float wz = (float)(gz & (a.prc - 1)) * inv_r;
+    const int cyb = (oy + a.b) >> lr, cxb = (ox + a.b) >> lr;
+    const float* c0 = a.pc + ((size_t)d * a.pnc + cz0) * a.pnc * a.pnc;
+    const float* c1 = a.pc + ((size_t)d * a.pnc + cz1) * a.pnc * a.pnc;
+    PM_ROWS(qy, nq) {
+      int cy = cyb + qy;
+      if (cy >= a.pnc) cy -= a.pnc;
+      PM_COLS(qx, nq) {
+        int cx = cxb + qx;
+        if (cx >= a.pnc) cx -= a.pnc;
+        const size_t o = (size_t)cy * a.pnc + cx;
+        Q[qy * nq + qx] = (1.0f - wz) * __ldg(c0 + o) + wz * __ldg(c1 + o);
+      }
+    }
+  }
+  // step 2: items (j2, pair), natural x = N2 j1 + j2
+  for (int w = threadIdx.x; w < np * N2; w += T) {
+    const int j2 = w / np, q = w - j2 * np;
+    float2* base = W + q * WP + j2;
+    float2 v[N1];
+#pragma unroll
+    for (int k1 = 0; k1 < N1; ++k1) v[k1] = base[N2 * k1];
+    Dft<N1, 1>::run(v);
+#pragma unroll
+    for (int j1 = 0; j1 < N1; ++j1) base[N2 * j1] = v[j1];
+  }
+  __syncthreads();
+  if (a.pc) {
+    PM_ROWS(qy, nq) {
+      const float* q = Q + qy * nq;
+      PM_COLS(xl, a.t) {
+        const int qx = xl >> lr;
+        const float fx = (float)(xl & (a.prc - 1)) * inv_r;
+        R[qy * a.t + xl] = fmaf(fx, q[qx + 1] - q[qx], q[qx]);
+      }
+    }
+    __syncthreads();
+  }
+  // Output cells are interior cells: origin + b + local lies inside [0, n) without wrap.
+  const int gz = oz + a.b + zo;
+  float* dst = a.dst + (size_t)d * n * n * n + ((int64_t)gz * n + oy + a.b) * n + ox + a.b;
+  float m = 0.f;
+  PM_ROWS(q, np) {
+    const int y0 = 2 * (m0 + q) - a.b, y1 = y0 + 1;   // the pair's output rows, if inside [0, t)
+    const bool in0 = y0 >= 0, in1 = y1 < a.t;
+    const int q0 = y0 >> lr, q1 = y1 >> lr;
+    const float f0 = (float)(y0 & (a.prc - 1)) * inv_r, f1 = (float)(y1 & (a.prc - 1)) * inv_r;
+    PM_COLS(xl, a.t) {
+      float2 w = W[q * WP + a.b + xl];
+      if (in0) m = fmaxf(m, fabsf(w.x));
+      if (in1) m = fmaxf(m, fabsf(w.y));
+      if (a.pc) {
+        float lo = 0.f, hi = 0.f;
+        if (in0) {
+          lo = R[q0 * a.t + xl];
+          hi = R[(q0 + 1) * a.t + xl];
+          w.x += fmaf(f0, hi - lo, lo);
+        }
+        if (in1) {
+          if (!in0 || q1 != q0) {
+            lo = R[q1 * a.t + xl];
+            hi = R[(q1 + 1) * a.t + xl];
+          }
+          w.y += fmaf(f1, hi - lo, lo);
+        }
+      }
+      if (in0) dst[(int64_t)y0 * n + xl] = w.x;
+      if (in1) dst[(int64_t)y1 * n + xl] = w.y;
+    }
+  }
+  if (a.amax) {
+    // warp maximum; an atomic only when it raises the running maximum
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0 && m > __uint_as_float(*(volatile unsigned int*)a.amax))
+      atomicMax(a.amax, __float_as_uint(m));
+  }
 }
 
 // Tensor maps (encoded on the host; cuTensorMapEncodeTiled reached through
@@ -930,17 +995,16 @@ static cudaError_t solve_n(const SolvePlan& p, const void* src, bool fixed, floa
     cudaFuncSetAttribute(solve_a_kernel<N, false>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem_a);
     cudaFuncSetAttribute(solve_a_kernel<N, true>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem_a);
     cudaFuncSetAttribute(solve_b_kernel<N>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassB<N>::smem);
-    cudaFuncSetAttribute(k_solve_c<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem_a);
+    cudaFuncSetAttribute(k_solve_c<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassC<N>::smem_max());
     if constexpr (N == 96) {
       cudaFuncSetAttribute(k_solve_a_tma<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassAT<N>::smem);
       cudaFuncSetAttribute(k_solve_b_tma<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassBT<N>::smem);
-      cudaFuncSetAttribute(k_solve_c_tma<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassCT<N>::smem);
     }
     attr_done = true;
   }
   // 96^3 passes staged by TMA: pass A wants window origins and the source
   // mesh on 16-cell boundaries (float source), pass B its output z range on
-  // an 8-row boundary; pass C always applies.
+  // an 8-row boundary.
   bool tma_a = false, tma_b = false;
   CUtensorMap src_map, spec_map, spec3_map;
   if constexpr (N == 96) {
@@ -983,8 +1047,7 @@ static cudaError_t solve_n(const SolvePlan& p, const void* src, bool fixed, floa
     }
     {
       TimedScope ts(tm, N == p.src_n && p.b == 0 ? "fft_c_mesh" : "fft_c_tiles", st);
-      if constexpr (N == 96) k_solve_c_tma<N><<<dim3(p.t, 3, nb), C::threads_c, PassCT<N>::smem, st>>>(a);
-      else k_solve_c<N><<<dim3(p.t, 3, nb), C::threads_c, C::smem_a, st>>>(a);
+      k_solve_c<N><<<dim3(p.t, 3, nb), PassC<N>::threads, PassC<N>::smem(p.t, p.b, a.prc, a.pc != nullptr), st>>>(a);
     }
     note_launches(3);
     cudaError_t e = cudaGetLastError();
@@ -1017,13 +1080,13 @@ static cudaError_t solve_adjoint_n(const SolvePlan& p, const float* lam_acc, boo
   const auto ka = interleaved ? k_solve_a<N, false, 4> : solve_a_kernel<N, false>();
   cudaFuncSetAttribute(ka, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem_a);
   cudaFuncSetAttribute(k_solve_b_adj<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(float2) * (N + 2 * (size_t)N * PassB<N>::KC)));
-  cudaFuncSetAttribute(k_solve_c<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem_a);
+  cudaFuncSetAttribute(k_solve_c<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassC<N>::smem_max());
   SolveArgs a{lam_acc, 0, p.src_n, 1, N, 0, 0, spec3comp, p.spec3, p.kern, p.tw, lam_rho, 1, nullptr, nullptr, 0, 1,
               p.status};
   ka<<<dim3(N, 3), C::threads, C::smem_a, st>>>(a);
   a.comp_mode = 0;
   k_solve_b_adj<N><<<dim3(N, 2, 1), PassB<N>::threads, sizeof(float2) * (N + 2 * (size_t)N * PassB<N>::KC), st>>>(a);
-  k_solve_c<N><<<dim3(N, 1, 1), C::threads_c, C::smem_a, st>>>(a);
+  k_solve_c<N><<<dim3(N, 1, 1), PassC<N>::threads, PassC<N>::smem(N, 0, 1, false), st>>>(a);
   note_launches(3);
   return cudaGetLastError();
 }
