@@ -29,7 +29,10 @@ template <int N> struct SolveCfg {
 // Threads per block of passes A and C (compile-time tunables; measured on the
 // 96^3 tiles: 512 for A, 384 for C).
 #ifndef PM_SOLVE_THREADS
-#define PM_SOLVE_THREADS 512
+#define PM_SOLVE_THREADS 416
+#endif
+#ifndef PM_SOLVE_A_MINB
+#define PM_SOLVE_A_MINB 3
 #endif
 #ifndef PM_SOLVE_C_THREADS
 #define PM_SOLVE_C_THREADS 416
@@ -37,8 +40,6 @@ template <int N> struct SolveCfg {
 #ifndef PM_SOLVE_C_MINB
 #define PM_SOLVE_C_MINB 3
 #endif
-  static constexpr int threads = (N >= 96) ? PM_SOLVE_THREADS : 256;
-  static constexpr size_t smem_a = sizeof(float2) * (N + (size_t)N * N / 2 + (size_t)N * NP);
 };
 
 struct SolveArgs {
@@ -100,81 +101,6 @@ __device__ __forceinline__ float src_value(const void* src, int64_t idx) {
 }
 
 __device__ __forceinline__ int wrap1(int g, int n) { return g < 0 ? g + n : (g >= n ? g - n : g); }
-
-// CS > 1 (comp_mode only): the components are interleaved, element i of
-// component pb at src[i * CS + pb] (the adjoint's float4 accumulation mesh).
-template <int N, bool FIXED, int CS = 1>
-__device__ __forceinline__ void solve_a_body(const SolveArgs& a) {
-  constexpr int NH = SolveCfg<N>::NH, NP = SolveCfg<N>::NP;
-  extern __shared__ float2 sm[];
-  float2* tw = sm;
-  float2* W = sm + N;               // N/2 packed rows of N
-  float2* P = W + N * N / 2;        // N rows (y) of NH, pitch NP
-  for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = a.tw[i];
-  const int z = blockIdx.x;
-  const int pb = blockIdx.y;
-  int ox, oy, oz;
-  problem_origin(a, a.p0 + pb, ox, oy, oz);
-  const int n = a.src_n;
-  const void* src = a.src;
-  if (a.comp_mode) {
-    ox = oy = oz = 0;
-    src = static_cast<const float*>(a.src) + (CS > 1 ? (size_t)pb : (size_t)pb * n * n * n);
-  }
-  // origins lie in (-n, n) and N <= n, so one conditional wrap suffices
-  const int gz = wrap1(oz + z, n);
-  PM_ROWS(y, N) {
-    const int64_t rowbase = ((int64_t)gz * n + wrap1(oy + y, n)) * n;
-    float* w = reinterpret_cast<float*>(W + (y >> 1) * N) + (y & 1);
-    if (FIXED) {
-      PM_COLS(x, N) w[2 * x] = src_value<FIXED>(src, rowbase + wrap1(ox + x, n));
-    } else {
-      const float* srow = static_cast<const float*>(src) + rowbase * CS;
-      PM_COLS(x, N) async_copy4(w + 2 * x, srow + wrap1(ox + x, n) * CS);
-    }
-  }
-  if (!FIXED) async_wait();
-  __syncthreads();
-  fft_fwd<N, N / 2, N, 1>(W, tw);
-  // Unpack the two real rows of each packed row: A = (Z_k + conj Z_-k)/2, B = (Z_k - conj Z_-k)/(2i).
-  PM_ROWS(j, N / 2) {
-    const float2* Wj = W + j * N;
-    PM_COLS(k, NH) {
-      float2 zk = Wj[slot_of<N>(k)];
-      float2 zm = Wj[slot_of<N>(k == 0 ? 0 : N - k)];
-      P[(2 * j) * NP + k] = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
-      P[(2 * j + 1) * NP + k] = make_float2(0.5f * (zk.y + zm.y), -0.5f * (zk.x - zm.x));
-    }
-  }
-  __syncthreads();
-  fft_fwd<N, NH, 1, NP>(P, tw);
-  // N * NP is even for every supported N: copy two complex values per access
-  // (the pitch's pad columns are copied too and never read).
-  float4* out = reinterpret_cast<float4*>(a.spec + ((size_t)pb * N + z) * N * NP);
-  const float4* P4 = reinterpret_cast<const float4*>(P);
-  for (int i = threadIdx.x; i < N * NP / 2; i += blockDim.x) out[i] = P4[i];
-}
-
-template <int N, bool FIXED, int CS = 1>
-__global__ void __launch_bounds__(SolveCfg<N>::threads) k_solve_a(SolveArgs a) {
-  solve_a_body<N, FIXED, CS>(a);
-}
-
-// The 96^3 tiles' pass A is compiled for 3 resident blocks per SM (40
-// registers; 3 blocks fit its shared memory): measured 0.205 -> 0.188 ms.
-#ifndef PM_SOLVE_A_MINB
-#define PM_SOLVE_A_MINB 3
-#endif
-template <bool FIXED>
-__global__ void __launch_bounds__(SolveCfg<96>::threads, PM_SOLVE_A_MINB) k_solve_a96(SolveArgs a) {
-  solve_a_body<96, FIXED>(a);
-}
-
-template <int N, bool FIXED>
-constexpr auto solve_a_kernel() {
-  if constexpr (N == 96) return k_solve_a96<FIXED>;
-  else return k_solve_a<N, FIXED>;
-}
 
 // Pass B works on one ky row and one chunk of KC kx columns (KC = ceil(NH/2),
 // i.e. two chunks, up to N = 128): forward z FFT, the three
@@ -351,69 +277,199 @@ __device__ __forceinline__ bool block_wait(uint64_t* bar, int* status) {
   return !bad;
 }
 
-template <int N> struct PassAT {
-  static constexpr int NH = N / 2 + 1, NP = spec_pitch(N), NB = N / kBox;
-  // P [N][NP] (first the staged boxes), W [N/2][N], twiddles
-  static constexpr size_t smem = kTmaAlign + sizeof(float2) * ((size_t)N * NP + (size_t)N / 2 * N + N);
+// ---- pass A ---------------------------------------------------------------
+//
+// One block per z plane of a window: real-to-complex along x (two rows packed
+// as one complex row), complex along y.  Bound by shared memory like pass C:
+// the earlier form moved 6,860 wavefronts per 96^3 tile plane (2,670 of them
+// bank conflicts) at 83% of the load/store pipe, 0.161 ms for 64 tiles.  Here
+//   * the first x step takes its inputs from the staged window boxes, without
+//     a repacking pass: a half warp reads consecutive cells of one row, the two
+//     halves of a warp their two rows in opposite order, so that they meet in
+//     different banks;
+//   * the packed rows have pitch N + 1 (odd) and the second x step gives a
+//     warp's lanes different rows; it leaves the spectrum in natural order
+//     (its items are in registers across a barrier, slots and frequencies
+//     overlap);
+//   * the packed rows are taken apart inside the first y step, two rows per item.
+// 3,100 wavefronts per plane: 0.124 ms; 216 tiles of 48^3: 0.094 -> 0.075 ms;
+// 416 threads against 384: 0.124 and 0.125 ms.
+// Sources that are not staged by TMA (int64 meshes, interleaved components,
+// other sizes) are copied to the packed rows directly.
+enum SourceForm { SRC_FLOAT, SRC_FIXED, SRC_INTERLEAVED, SRC_BOXES };
+
+template <int N> struct PassA {
+  static constexpr int N1 = Factor<N>::N1, N2 = Factor<N>::N2;
+  static constexpr int NH = N / 2 + 1, NP = spec_pitch(N), WP = N + 1, NB = N / kBox;
+  static constexpr bool in_place = N >= 128;   // P over W: 67 KB at 128, so that 2 blocks share an SM
+  static constexpr int threads = N == 128 ? 544 : (N == 96 ? PM_SOLVE_THREADS : (N == 64 ? 288 : (N == 48 ? 160 : (N == 32 ? 96 : 64))));
+  static constexpr int min_blocks = N == 128 ? 2 : (N == 96 ? PM_SOLVE_A_MINB : 4);
+  static constexpr size_t w_vals = ((size_t)N / 2 * WP + 1) / 2 * 2;
+  // P [N][NP] (first the staged boxes), twiddles, W [N/2][WP]
+  static constexpr size_t smem = kTmaAlign + sizeof(float2) * ((size_t)N * NP + N + (in_place ? 0 : w_vals));
 };
 
-template <int N>
-__global__ void __launch_bounds__(SolveCfg<N>::threads, PM_SOLVE_A_MINB)
-    k_solve_a_tma(SolveArgs a, const __grid_constant__ CUtensorMap src_map) {
-  using C = PassAT<N>;
-  constexpr int NH = C::NH, NP = C::NP, NB = C::NB;
-  static_assert((size_t)NB * NB * kBox * kBox <= (size_t)2 * N * NP, "staged window must fit in P");
+template <int N, int SRC>
+__global__ void __launch_bounds__(PassA<N>::threads, PassA<N>::min_blocks)
+    k_solve_a(SolveArgs a, const __grid_constant__ CUtensorMap src_map) {
+  using A = PassA<N>;
+  constexpr int N1 = A::N1, N2 = A::N2, NH = A::NH, NP = A::NP, WP = A::WP, T = A::threads;
+  constexpr int NB = A::NB > 0 ? A::NB : 1;
   extern __shared__ unsigned char smraw_a[];
   __shared__ uint64_t bar;
-  float2* P = reinterpret_cast<float2*>(tma_align(smraw_a));   // [y][NP]; first the staged window boxes
-  float2* W = P + N * NP;                                        // N/2 packed rows of N
-  float2* tw = W + N * N / 2;
-  float* S = reinterpret_cast<float*>(P);                        // box (yb, xb) at S + (yb NB + xb) 256
+  float2* P = reinterpret_cast<float2*>(tma_align(smraw_a));    // [y][NP]
+  float2* tw = P + N * NP;
+  float2* W = A::in_place ? P : tw + N;                           // [row pair][WP]
+  float* S = reinterpret_cast<float*>(P);                         // box (yb, xb) at S + (yb NB + xb) 256
   const int z = blockIdx.x, pb = blockIdx.y;
   int ox, oy, oz;
   problem_origin(a, a.p0 + pb, ox, oy, oz);
   const int n = a.src_n;
-  if (threadIdx.x == 0) {
-    tma::mbar_init(&bar, 1);
-    tma::fence_barrier_init();
+  const void* src = a.src;
+  if (a.comp_mode) {
+    ox = oy = oz = 0;
+    src = static_cast<const float*>(a.src) + (SRC == SRC_INTERLEAVED ? (size_t)pb : (size_t)pb * n * n * n);
   }
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    if (threadIdx.x == 0) tma::mbar_arrive_expect_tx(&bar, NB * NB * kBox * kBox * (unsigned)sizeof(float));
-    __syncwarp();
-    const int gz = wrap1(oz + z, n);
-    for (int k = threadIdx.x; k < NB * NB; k += 32) {
-      const int yb = k / NB, xb = k - yb * NB;
-      tma::tensor_load_3d(S + k * kBox * kBox, &src_map, wrap1(ox + kBox * xb, n), wrap1(oy + kBox * yb, n), gz,
-                          &bar);
+  for (int i = threadIdx.x; i < N; i += T) tw[i] = a.tw[i];
+  // origins lie in (-n, n) and N <= n, so one conditional wrap suffices
+  const int gz = wrap1(oz + z, n);
+  if constexpr (SRC == SRC_BOXES) {
+    static_assert((size_t)NB * NB * kBox * kBox <= (size_t)2 * N * NP, "staged window must fit in P");
+    if (threadIdx.x == 0) {
+      tma::mbar_init(&bar, 1);
+      tma::fence_barrier_init();
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      if (threadIdx.x == 0) tma::mbar_arrive_expect_tx(&bar, NB * NB * kBox * kBox * (unsigned)sizeof(float));
+      __syncwarp();
+      for (int k = threadIdx.x; k < NB * NB; k += 32) {
+        const int yb = k / NB, xb = k - yb * NB;
+        tma::tensor_load_3d(S + k * kBox * kBox, &src_map, wrap1(ox + kBox * xb, n), wrap1(oy + kBox * yb, n), gz,
+                            &bar);
+      }
+    }
+    if (!block_wait(&bar, a.status)) return;
+    // x step 1 from the boxes: 16 lanes per row pair j, N2 of them with an item j2
+    static_assert(N2 <= 16, "a half warp per row pair");
+    for (int w = threadIdx.x; w < (N / 2) * 16; w += T) {
+      const int j = w >> 4, j2 = w & 15;
+      if (j2 < N2) {
+        const int first = (threadIdx.x >> 4) & 1;   // the row this half warp reads first
+        const float* s0 = S + (2 * j / kBox) * NB * kBox * kBox + (2 * j % kBox) * kBox + first * kBox;
+        const int other = first ? -kBox : kBox;
+        float2 v[N1];
+#pragma unroll
+        for (int j1 = 0; j1 < N1; ++j1) {
+          const int x = N2 * j1 + j2;
+          const float* q = s0 + (x / kBox) * kBox * kBox + x % kBox;
+          const float p0 = q[0], p1 = q[other];
+          v[j1] = first ? make_float2(p1, p0) : make_float2(p0, p1);
+        }
+        Dft<N1, -1>::run(v);
+#pragma unroll
+        for (int k1 = 1; k1 < N1; ++k1) v[k1] = cmul(v[k1], tw[j2 * k1]);
+        float2* base = W + j * WP + j2;
+#pragma unroll
+        for (int k1 = 0; k1 < N1; ++k1) base[N2 * k1] = v[k1];
+      }
+    }
+  } else {
+    constexpr int CS = SRC == SRC_INTERLEAVED ? 4 : 1;
+    PM_ROWS(y, N) {
+      const int64_t rowbase = ((int64_t)gz * n + wrap1(oy + y, n)) * n;
+      float* w = reinterpret_cast<float*>(W + (y >> 1) * WP) + (y & 1);
+      if (SRC == SRC_FIXED) {
+        PM_COLS(x, N) w[2 * x] = src_value<true>(src, rowbase + wrap1(ox + x, n));
+      } else {
+        const float* srow = static_cast<const float*>(src) + rowbase * CS;
+        PM_COLS(x, N) async_copy4(w + 2 * x, srow + wrap1(ox + x, n) * CS);
+      }
+    }
+    if (SRC != SRC_FIXED) async_wait();
+    __syncthreads();
+    // x step 1: items (j2, row pair), in place
+    for (int w = threadIdx.x; w < N2 * (N / 2); w += T) {
+      const int j2 = w / (N / 2), j = w - j2 * (N / 2);
+      float2* base = W + j * WP + j2;
+      float2 v[N1];
+#pragma unroll
+      for (int j1 = 0; j1 < N1; ++j1) v[j1] = base[N2 * j1];
+      Dft<N1, -1>::run(v);
+#pragma unroll
+      for (int k1 = 1; k1 < N1; ++k1) v[k1] = cmul(v[k1], tw[j2 * k1]);
+#pragma unroll
+      for (int k1 = 0; k1 < N1; ++k1) base[N2 * k1] = v[k1];
     }
   }
-  for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = a.tw[i];
-  if (!block_wait(&bar, a.status)) return;
-  // W[j][x] = (row 2j, row 2j + 1) at x; both rows lie in the same box row pair
-  for (int i = threadIdx.x; i < (N / 2) * (N / 4); i += blockDim.x) {
-    const int j = i / (N / 4), x = 4 * (i - j * (N / 4));
-    const int y0 = 2 * j;
-    const float* s0 = S + ((y0 / kBox) * NB + x / kBox) * kBox * kBox + (y0 % kBox) * kBox + x % kBox;
-    const float4 r0 = *reinterpret_cast<const float4*>(s0);
-    const float4 r1 = *reinterpret_cast<const float4*>(s0 + kBox);
-    float4* w = reinterpret_cast<float4*>(W + j * N + x);
-    w[0] = make_float4(r0.x, r1.x, r0.y, r1.y);
-    w[1] = make_float4(r0.z, r1.z, r0.w, r1.w);
-  }
   __syncthreads();
-  fft_fwd<N, N / 2, N, 1>(W, tw);
-  PM_ROWS(j, N / 2) {
-    const float2* Wj = W + j * N;
-    PM_COLS(k, NH) {
-      float2 zk = Wj[slot_of<N>(k)];
-      float2 zm = Wj[slot_of<N>(k == 0 ? 0 : N - k)];
-      P[(2 * j) * NP + k] = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
-      P[(2 * j + 1) * NP + k] = make_float2(0.5f * (zk.y + zm.y), -0.5f * (zk.x - zm.x));
+  // x step 2: items (k1, row pair), one round; slots N2 k1 + j2 -> frequencies k1 + N1 k2
+  {
+    static_assert(N1 * (N / 2) <= T, "one round");
+    const int w = threadIdx.x;
+    const bool live = w < N1 * (N / 2);
+    const int k1 = w / (N / 2), j = w - k1 * (N / 2);
+    float2 v[N2];
+    if (live) {
+#pragma unroll
+      for (int j2 = 0; j2 < N2; ++j2) v[j2] = W[j * WP + N2 * k1 + j2];
+      Dft<N2, -1>::run(v);
+    }
+    __syncthreads();
+    if (live) {
+#pragma unroll
+      for (int k2 = 0; k2 < N2; ++k2) W[j * WP + k1 + N1 * k2] = v[k2];
     }
   }
   __syncthreads();
-  fft_fwd<N, NH, 1, NP>(P, tw);
+  // y step 1: items (two neighbouring j2 = rows of one pair, column).  The two
+  // real rows of a pair: (Z_k + conj Z_-k) / 2 and (Z_k - conj Z_-k) / (2i).
+  {
+    static_assert(!A::in_place || (N2 / 2) * NH <= T, "in place: one round");
+    for (int w0 = 0; w0 < (N2 / 2) * NH; w0 += T) {
+      const int w = w0 + threadIdx.x;
+      const bool live = w < (N2 / 2) * NH;
+      const int jp = live ? w / NH : 0, c = live ? w - jp * NH : 0;
+      const int cm = c == 0 ? 0 : N - c;
+      float2 u[N1], v[N1];
+#pragma unroll
+      for (int j1 = 0; j1 < N1; ++j1) {
+        const float2* row = W + ((N2 / 2) * j1 + jp) * WP;
+        const float2 zk = row[c], zm = row[cm];
+        u[j1] = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
+        v[j1] = make_float2(0.5f * (zk.y + zm.y), -0.5f * (zk.x - zm.x));
+      }
+      Dft<N1, -1>::run(u);
+      Dft<N1, -1>::run(v);
+#pragma unroll
+      for (int k1 = 1; k1 < N1; ++k1) {
+        u[k1] = cmul(u[k1], tw[2 * jp * k1]);
+        v[k1] = cmul(v[k1], tw[(2 * jp + 1) * k1]);
+      }
+      if (A::in_place) __syncthreads();   // every packed row is read before P overwrites it
+      if (live) {
+        float2* base = P + 2 * jp * NP + c;
+#pragma unroll
+        for (int k1 = 0; k1 < N1; ++k1) {
+          base[N2 * k1 * NP] = u[k1];
+          base[(N2 * k1 + 1) * NP] = v[k1];
+        }
+      }
+    }
+  }
+  __syncthreads();
+  // y step 2: items (k1, column), in place
+  for (int w = threadIdx.x; w < N1 * NH; w += T) {
+    const int k1 = w / NH, c = w - k1 * NH;
+    float2* base = P + N2 * k1 * NP + c;
+    float2 v[N2];
+#pragma unroll
+    for (int j2 = 0; j2 < N2; ++j2) v[j2] = base[j2 * NP];
+    Dft<N2, -1>::run(v);
+#pragma unroll
+    for (int k2 = 0; k2 < N2; ++k2) base[k2 * NP] = v[k2];
+  }
+  // (the pitch's pad columns are stored too and never read)
   tma::fence_proxy_async();
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -992,12 +1048,12 @@ static cudaError_t solve_n(const SolvePlan& p, const void* src, bool fixed, floa
   using C = SolveCfg<N>;
   static bool attr_done = false;
   if (!attr_done) {
-    cudaFuncSetAttribute(solve_a_kernel<N, false>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem_a);
-    cudaFuncSetAttribute(solve_a_kernel<N, true>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem_a);
+    cudaFuncSetAttribute(k_solve_a<N, SRC_FLOAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassA<N>::smem);
+    cudaFuncSetAttribute(k_solve_a<N, SRC_FIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassA<N>::smem);
     cudaFuncSetAttribute(solve_b_kernel<N>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassB<N>::smem);
     cudaFuncSetAttribute(k_solve_c<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassC<N>::smem_max());
     if constexpr (N == 96) {
-      cudaFuncSetAttribute(k_solve_a_tma<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassAT<N>::smem);
+      cudaFuncSetAttribute(k_solve_a<N, SRC_BOXES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassA<N>::smem);
       cudaFuncSetAttribute(k_solve_b_tma<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassBT<N>::smem);
     }
     attr_done = true;
@@ -1006,7 +1062,7 @@ static cudaError_t solve_n(const SolvePlan& p, const void* src, bool fixed, floa
   // mesh on 16-cell boundaries (float source), pass B its output z range on
   // an 8-row boundary.
   bool tma_a = false, tma_b = false;
-  CUtensorMap src_map, spec_map, spec3_map;
+  CUtensorMap src_map{}, spec_map{}, spec3_map{};
   if constexpr (N == 96) {
     const int n = p.src_n;
     tma_a = !fixed && n % kBox == 0 && p.t % kBox == 0 && p.b % kBox == 0 &&
@@ -1024,13 +1080,12 @@ static cudaError_t solve_n(const SolvePlan& p, const void* src, bool fixed, floa
                 pro ? pro->coarse : nullptr, pro ? pro->nc : 0, pro ? pro->rc : 1, p.status};
     {
       TimedScope ts(tm, N == p.src_n && p.b == 0 ? "fft_a_mesh" : "fft_a_tiles", st);
+      using A = PassA<N>;
+      const auto ka = fixed ? k_solve_a<N, SRC_FIXED> : k_solve_a<N, SRC_FLOAT>;
       if constexpr (N == 96) {
-        if (tma_a) k_solve_a_tma<N><<<dim3(N, nb), C::threads, PassAT<N>::smem, st>>>(a, src_map);
+        if (tma_a) k_solve_a<N, SRC_BOXES><<<dim3(N, nb), A::threads, A::smem, st>>>(a, src_map);
       }
-      if (!tma_a) {
-        if (fixed) solve_a_kernel<N, true>()<<<dim3(N, nb), C::threads, C::smem_a, st>>>(a);
-        else solve_a_kernel<N, false>()<<<dim3(N, nb), C::threads, C::smem_a, st>>>(a);
-      }
+      if (!tma_a) ka<<<dim3(N, nb), A::threads, A::smem, st>>>(a, src_map);
     }
     {
       TimedScope ts(tm, N == p.src_n && p.b == 0 ? "fft_b_mesh" : "fft_b_tiles", st);
@@ -1076,14 +1131,13 @@ cudaError_t solve_launch(const SolvePlan& p, const void* src, bool fixed, float*
 template <int N>
 static cudaError_t solve_adjoint_n(const SolvePlan& p, const float* lam_acc, bool interleaved, float* lam_rho,
                                    float2* spec3comp, cudaStream_t st) {
-  using C = SolveCfg<N>;
-  const auto ka = interleaved ? k_solve_a<N, false, 4> : solve_a_kernel<N, false>();
-  cudaFuncSetAttribute(ka, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem_a);
+  const auto ka = interleaved ? k_solve_a<N, SRC_INTERLEAVED> : k_solve_a<N, SRC_FLOAT>;
+  cudaFuncSetAttribute(ka, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassA<N>::smem);
   cudaFuncSetAttribute(k_solve_b_adj<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(float2) * (N + 2 * (size_t)N * PassB<N>::KC)));
   cudaFuncSetAttribute(k_solve_c<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassC<N>::smem_max());
   SolveArgs a{lam_acc, 0, p.src_n, 1, N, 0, 0, spec3comp, p.spec3, p.kern, p.tw, lam_rho, 1, nullptr, nullptr, 0, 1,
               p.status};
-  ka<<<dim3(N, 3), C::threads, C::smem_a, st>>>(a);
+  ka<<<dim3(N, 3), PassA<N>::threads, PassA<N>::smem, st>>>(a, CUtensorMap{});
   a.comp_mode = 0;
   k_solve_b_adj<N><<<dim3(N, 2, 1), PassB<N>::threads, sizeof(float2) * (N + 2 * (size_t)N * PassB<N>::KC), st>>>(a);
   k_solve_c<N><<<dim3(N, 1, 1), PassC<N>::threads, PassC<N>::smem(N, 0, 1, false), st>>>(a);
