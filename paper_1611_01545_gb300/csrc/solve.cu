@@ -34,6 +34,15 @@ template <int N> struct SolveCfg {
 #ifndef PM_SOLVE_A_MINB
 #define PM_SOLVE_A_MINB 3
 #endif
+#ifndef PM_PASSB_KT
+#define PM_PASSB_KT 26
+#endif
+#ifndef PM_PASSB_TMA_THREADS
+#define PM_PASSB_TMA_THREADS 256
+#endif
+#ifndef PM_PASSB_TMA_MINB
+#define PM_PASSB_TMA_MINB 3
+#endif
 #ifndef PM_SOLVE_C_THREADS
 #define PM_SOLVE_C_THREADS 416
 #endif
@@ -174,23 +183,8 @@ __device__ __forceinline__ void solve_b_body(const SolveArgs& a) {
 }
 
 template <int N>
-__global__ void __launch_bounds__(PassB<N>::threads) k_solve_b(SolveArgs a) {
+__global__ void __launch_bounds__(PassB<N>::threads) k_large_b(SolveArgs a) {
   solve_b_body<N>(a);
-}
-
-// The 96^3 tiles' pass B compiled for 3 resident blocks per SM (its shared
-// memory allows 3 since the forward transform shares the product buffer).
-#ifndef PM_PASSB_MINB
-#define PM_PASSB_MINB 3
-#endif
-__global__ void __launch_bounds__(PassB<96>::threads, PM_PASSB_MINB) k_solve_b96(SolveArgs a) {
-  solve_b_body<96>(a);
-}
-
-template <int N>
-constexpr auto solve_b_kernel() {
-  if constexpr (N == 96) return k_solve_b96;
-  else return k_solve_b<N>;
 }
 
 // Transpose of the solve for one periodic mesh (the adjoint of a_d = K_d * rho):
@@ -479,66 +473,86 @@ __global__ void __launch_bounds__(PassA<N>::threads, PassA<N>::min_blocks)
   }
 }
 
-// Threads and resident blocks per SM of the TMA pass B (compile-time tunables).
-#ifndef PM_PASSB_TMA_THREADS
-#define PM_PASSB_TMA_THREADS 256
-#endif
-#ifndef PM_PASSB_TMA_MINB
-#define PM_PASSB_TMA_MINB 3
-#endif
-template <int N> struct PassBT {
+// ---- pass B ---------------------------------------------------------------
+//
+// One block per ky row and KT kx columns: the forward z transform, the three
+// kernel products and their inverse z transforms.  The second step of the
+// forward transform, the products and the first step of each inverse transform
+// run in registers per (k1, column) item; the second inverse step writes its
+// output rows straight to global memory (KT consecutive complex values each),
+// where it wrote all N rows to shared memory and a box store read back the
+// output ones: 3,140 -> 2,300 wavefronts per block of 96 x 26; 0.214 -> 0.212 ms
+// for 64 tiles, whose kernel-table loads and 24 warps per SM bound it now, and
+// 0.163 -> 0.106 ms for 216 tiles of 48^3, which one block of all 25 columns
+// serves.  Other shapes of 96: 320 threads at 3 blocks per SM 0.210 (spills), at
+// 2 blocks 0.230; 18 columns with 160 threads at 5 blocks 0.212, 224 at 4 0.215.
+template <int N> struct PassBR {
   static constexpr int NH = N / 2 + 1, NP = spec_pitch(N);
-  static constexpr int KT = 26;                        // kx columns per block: KT * 8 bytes is a multiple of 16
+  // columns per block (N = 96: box rows of whole 16-byte words), and threads
+  // that take each item set in few, full rounds
+  static constexpr int KT = N == 128 ? 22 : (N == 96 ? PM_PASSB_KT : (N == 64 ? 17 : NH));
   static constexpr int nchunk = (NH + KT - 1) / KT;
-  static constexpr int threads = PM_PASSB_TMA_THREADS;
-  // G [3][N][KT] (component, z, column), twiddles
+  static constexpr int threads = N == 128 ? 192 : (N == 96 ? PM_PASSB_TMA_THREADS : (N == 48 ? 224 : (N == 16 ? 64 : 160)));
+  static constexpr int min_blocks = N >= 96 ? PM_PASSB_TMA_MINB : (N == 48 ? 3 : 4);
+  // G [3][N][KT] (component, z, column; the forward transform in component 0), twiddles
   static constexpr size_t smem = kTmaAlign + sizeof(float2) * (3 * (size_t)N * KT + N);
 };
 
 template <int N>
-__global__ void __launch_bounds__(PassBT<N>::threads, PM_PASSB_TMA_MINB)
-    k_solve_b_tma(SolveArgs a, const __grid_constant__ CUtensorMap spec_map,
-                  const __grid_constant__ CUtensorMap spec3_map) {
-  using B = PassBT<N>;
-  constexpr int NH = B::NH, KT = B::KT;
+__global__ void __launch_bounds__(PassBR<N>::threads, PassBR<N>::min_blocks)
+    k_solve_b(SolveArgs a, const __grid_constant__ CUtensorMap spec_map) {
+  using B = PassBR<N>;
+  constexpr int NH = B::NH, NP = B::NP, KT = B::KT, T = B::threads;
   constexpr int N1 = Factor<N>::N1, N2 = Factor<N>::N2;
   extern __shared__ unsigned char smraw_b[];
   __shared__ uint64_t bar;
   float2* G = reinterpret_cast<float2*>(tma_align(smraw_b));   // [3][N][KT]
   float2* tw = G + 3 * N * KT;
   const int ys = blockIdx.x, kx0 = blockIdx.y * KT, pb = blockIdx.z;
-  if (threadIdx.x == 0) {
-    tma::mbar_init(&bar, 1);
-    tma::fence_barrier_init();
+  const int ncol = NH - kx0 < KT ? NH - kx0 : KT;
+  for (int i = threadIdx.x; i < N; i += T) tw[i] = a.tw[i];
+  if constexpr (N == 96) {
+    if (threadIdx.x == 0) {
+      tma::mbar_init(&bar, 1);
+      tma::fence_barrier_init();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      tma::mbar_arrive_expect_tx(&bar, N * KT * (unsigned)sizeof(float2));
+      tma::tensor_load_3d(G, &spec_map, 2 * kx0, ys, pb * N, &bar);
+    }
+    if (!block_wait(&bar, a.status)) return;
+  } else {
+    const float2* in = a.spec + ((size_t)pb * N * N + ys) * NP + kx0;
+    for (int i = threadIdx.x; i < N * KT; i += T) {
+      const int z = i / KT, c = i - z * KT;
+      if (c < ncol) async_copy8(G + i, in + (size_t)z * N * NP + c);
+      else G[i] = make_float2(0.f, 0.f);
+    }
+    async_wait();
+    __syncthreads();
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    tma::mbar_arrive_expect_tx(&bar, N * KT * (unsigned)sizeof(float2));
-    tma::tensor_load_3d(G, &spec_map, 2 * kx0, ys, pb * N, &bar);
-  }
-  for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = a.tw[i];
-  if (!block_wait(&bar, a.status)) return;
-  // forward z transform, step 1 (items (j2, column)), in component 0
-  for (int w = threadIdx.x; w < KT * N2; w += blockDim.x) {
+  // forward z transform, step 1: items (j2, column), in component 0
+  for (int w = threadIdx.x; w < KT * N2; w += T) {
     const int j2 = w / KT, c = w - j2 * KT;
-    float2* base = G + c;
+    float2* base = G + j2 * KT + c;
     float2 v[N1];
 #pragma unroll
-    for (int j1 = 0; j1 < N1; ++j1) v[j1] = base[(N2 * j1 + j2) * KT];
+    for (int j1 = 0; j1 < N1; ++j1) v[j1] = base[N2 * j1 * KT];
     Dft<N1, -1>::run(v);
 #pragma unroll
     for (int k1 = 1; k1 < N1; ++k1) v[k1] = cmul(v[k1], tw[j2 * k1]);
 #pragma unroll
-    for (int k1 = 0; k1 < N1; ++k1) base[(N2 * k1 + j2) * KT] = v[k1];
+    for (int k1 = 0; k1 < N1; ++k1) base[N2 * k1 * KT] = v[k1];
   }
   __syncthreads();
   // forward step 2, the products i K_d F and step 1 of each inverse
   // transform, per (k1, column) item: F(kz = k1 + N1 k2) sits at slot N2 k1 + k2
   const float* Kb = a.kern + (size_t)ys * NH + kx0;
-  const size_t kstride = (size_t)N * N * NH;
-  for (int w = threadIdx.x; w < KT * N1; w += blockDim.x) {
+  constexpr size_t kstride = (size_t)N * N * NH;
+  for (int w = threadIdx.x; w < KT * N1; w += T) {
     const int k1 = w / KT, c = w - k1 * KT;
-    const bool live = kx0 + c < NH;
+    const bool live = c < ncol;
     float2 f[N2];
 #pragma unroll
     for (int j2 = 0; j2 < N2; ++j2) f[j2] = G[(N2 * k1 + j2) * KT + c];
@@ -555,31 +569,31 @@ __global__ void __launch_bounds__(PassBT<N>::threads, PM_PASSB_TMA_MINB)
       Dft<N2, 1>::run(g);
 #pragma unroll
       for (int j2 = 1; j2 < N2; ++j2) g[j2] = cmul(g[j2], conjf2(tw[j2 * k1]));
-      float2* gd = G + (size_t)d * N * KT + c;
+      float2* gd = G + d * N * KT + N2 * k1 * KT + c;
 #pragma unroll
-      for (int j2 = 0; j2 < N2; ++j2) gd[(N2 * k1 + j2) * KT] = g[j2];
+      for (int j2 = 0; j2 < N2; ++j2) gd[j2 * KT] = g[j2];
     }
   }
   __syncthreads();
-  // inverse step 2 of the three components -> natural z order
-  for (int w = threadIdx.x; w < 3 * KT * N2; w += blockDim.x) {
-    const int j2 = w / (3 * KT), q = w - j2 * 3 * KT;
-    const int d = q / KT, c = q - d * KT;
-    float2* base = G + (size_t)d * N * KT + c;
+  // inverse step 2: items (component, j2, column) -> rows z = N2 j1 + j2 of the output range
+  float2* out = a.spec3 + ((size_t)pb * 3 * a.t * N + ys) * NP + kx0;
+  for (int w = threadIdx.x; w < 3 * KT * N2; w += T) {
+    const int d = w / (KT * N2), r = w - d * KT * N2;
+    const int j2 = r / KT, c = r - j2 * KT;
+    const float2* base = G + d * N * KT + j2 * KT + c;
     float2 v[N1];
 #pragma unroll
-    for (int k1 = 0; k1 < N1; ++k1) v[k1] = base[(N2 * k1 + j2) * KT];
+    for (int k1 = 0; k1 < N1; ++k1) v[k1] = base[N2 * k1 * KT];
     Dft<N1, 1>::run(v);
+    if (c < ncol) {
+      const int z0 = j2 - a.b;
+      float2* o = out + (ptrdiff_t)(d * a.t + z0) * N * NP + c;
 #pragma unroll
-    for (int j1 = 0; j1 < N1; ++j1) base[(N2 * j1 + j2) * KT] = v[j1];
-  }
-  tma::fence_proxy_async();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int d = 0; d < 3; ++d)
-      tma::tensor_store_3d(&spec3_map, 2 * kx0, ys, (pb * 3 + d) * a.t, G + ((size_t)d * N + a.b) * KT);
-    tma::bulk_commit();
-    tma::bulk_wait_all();
+      for (int j1 = 0; j1 < N1; ++j1) {
+        const int zo = z0 + N2 * j1;
+        if (zo >= 0 && zo < a.t) o[(size_t)N2 * j1 * N * NP] = v[j1];
+      }
+    }
   }
 }
 
@@ -1006,7 +1020,7 @@ static cudaError_t solve_large_n(const SolvePlan& p, const void* src, bool fixed
     cudaFuncSetAttribute(k_large_ax<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::smem_ax);
     cudaFuncSetAttribute(k_large_y<N, -1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::smem_y);
     cudaFuncSetAttribute(k_large_y<N, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::smem_y);
-    cudaFuncSetAttribute(solve_b_kernel<N>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassB<N>::smem);
+    cudaFuncSetAttribute(k_large_b<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassB<N>::smem);
     cudaFuncSetAttribute(k_large_cx<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::smem_cx);
     attr_done = true;
   }
@@ -1019,7 +1033,7 @@ static cudaError_t solve_large_n(const SolvePlan& p, const void* src, bool fixed
   }
   {
     TimedScope ts(tm, "fft_b_mesh", st);
-    solve_b_kernel<N>()<<<dim3(N, PassB<N>::nchunk, 1), PassB<N>::threads, PassB<N>::smem, st>>>(a);
+    k_large_b<N><<<dim3(N, PassB<N>::nchunk, 1), PassB<N>::threads, PassB<N>::smem, st>>>(a);
   }
   {
     TimedScope ts(tm, "fft_c_mesh", st);
@@ -1050,28 +1064,24 @@ static cudaError_t solve_n(const SolvePlan& p, const void* src, bool fixed, floa
   if (!attr_done) {
     cudaFuncSetAttribute(k_solve_a<N, SRC_FLOAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassA<N>::smem);
     cudaFuncSetAttribute(k_solve_a<N, SRC_FIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassA<N>::smem);
-    cudaFuncSetAttribute(solve_b_kernel<N>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassB<N>::smem);
+    cudaFuncSetAttribute(k_solve_b<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassBR<N>::smem);
     cudaFuncSetAttribute(k_solve_c<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassC<N>::smem_max());
     if constexpr (N == 96) {
       cudaFuncSetAttribute(k_solve_a<N, SRC_BOXES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassA<N>::smem);
-      cudaFuncSetAttribute(k_solve_b_tma<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassBT<N>::smem);
     }
     attr_done = true;
   }
   // 96^3 passes staged by TMA: pass A wants window origins and the source
-  // mesh on 16-cell boundaries (float source), pass B its output z range on
-  // an 8-row boundary.
-  bool tma_a = false, tma_b = false;
-  CUtensorMap src_map{}, spec_map{}, spec3_map{};
+  // mesh on 16-cell boundaries (float source); pass B reads boxes of the spectrum.
+  bool tma_a = false;
+  CUtensorMap src_map{}, spec_map{};
   if constexpr (N == 96) {
     const int n = p.src_n;
     tma_a = !fixed && n % kBox == 0 && p.t % kBox == 0 && p.b % kBox == 0 &&
             map_3d(&src_map, src, n, n, n, (uint64_t)n * 4, (uint64_t)n * n * 4, kBox, kBox, 1);
-    tma_b = p.b % 8 == 0 &&
-            map_3d(&spec_map, p.spec, 2 * C::NH, N, (uint64_t)p.batch * N, (uint64_t)C::NP * 8,
-                   (uint64_t)N * C::NP * 8, 2 * PassBT<N>::KT, 1, N) &&
-            map_3d(&spec3_map, p.spec3, 2 * C::NH, N, (uint64_t)p.batch * 3 * p.t, (uint64_t)C::NP * 8,
-                   (uint64_t)N * C::NP * 8, 2 * PassBT<N>::KT, 1, p.t);
+    if (!map_3d(&spec_map, p.spec, 2 * C::NH, N, (uint64_t)p.batch * N, (uint64_t)C::NP * 8, (uint64_t)N * C::NP * 8,
+                2 * PassBR<N>::KT, 1, N))
+      return cudaErrorInvalidValue;
   }
   const int nprob = p.nts * p.nts * p.nts;
   for (int p0 = 0; p0 < nprob; p0 += p.batch) {
@@ -1089,12 +1099,8 @@ static cudaError_t solve_n(const SolvePlan& p, const void* src, bool fixed, floa
     }
     {
       TimedScope ts(tm, N == p.src_n && p.b == 0 ? "fft_b_mesh" : "fft_b_tiles", st);
-      if constexpr (N == 96) {
-        if (tma_b)
-          k_solve_b_tma<N><<<dim3(N, PassBT<N>::nchunk, nb), PassBT<N>::threads, PassBT<N>::smem, st>>>(a, spec_map,
-                                                                                                       spec3_map);
-      }
-      if (!tma_b) solve_b_kernel<N>()<<<dim3(N, PassB<N>::nchunk, nb), PassB<N>::threads, PassB<N>::smem, st>>>(a);
+      using B = PassBR<N>;
+      k_solve_b<N><<<dim3(N, B::nchunk, nb), B::threads, B::smem, st>>>(a, spec_map);
     }
     if (pro && pro->ready && p0 == 0) {
       cudaError_t e = cudaStreamWaitEvent(st, pro->ready, 0);   // the coarse force must be complete
