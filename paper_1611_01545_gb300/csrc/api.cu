@@ -504,6 +504,8 @@ int pm_init(const pm_config_t* cfg, pm_handle_t** out) {
     p.src_n = src_n;
     p.batch = batch;
     A(&p.kern, kern.size() * 4);
+    const size_t quads = kernel_quads(N, nullptr, nullptr, nullptr);
+    if (quads) A(&p.kern_quads, quads);
     A(&p.tw, (size_t)N * sizeof(float2));
     A(&p.spec, (size_t)batch * N * N * p.NP * sizeof(float2));
     A(&p.spec3, (size_t)batch * 3 * t * N * p.NP * sizeof(float2));
@@ -512,6 +514,8 @@ int pm_init(const pm_config_t* cfg, pm_handle_t** out) {
     if (cudaMemcpy(p.kern, kern.data(), kern.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(p.tw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice) != cudaSuccess)
       rc = fail(h, PM_ERR_CUDA, "kernel table upload failed");
+    else if (quads)
+      kernel_quads(N, p.kern, reinterpret_cast<float*>(p.kern_quads), nullptr);
   };
   if (g.two) {
     make_plan(h->plan_mesh, g.nc, 1, g.nc, 0, g.nc, 1, periodic_kernel(g.nc, (double)g.rc, c.G, c.r_split));

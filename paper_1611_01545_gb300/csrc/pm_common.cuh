@@ -47,6 +47,7 @@ struct SolvePlan {
   int src_n = 0;      // periodic source / destination mesh edge
   int batch = 1;      // problems per batch
   float* kern = nullptr;   // device [3][N slot][N slot][NH]
+  float4* kern_quads = nullptr;   // device: pass B's order of the same values (N <= 128)
   float2* tw = nullptr;    // device [N]
   float2* spec = nullptr;  // device [batch][N][N][NP]
   float2* spec3 = nullptr; // device [batch][3][t][N][NP]
@@ -75,6 +76,9 @@ cudaError_t launch_restrict(const float* rho_f, int nf, int rc, float* rho_c, cu
 // (x, y, z, unused) when interleaved.
 cudaError_t solve_adjoint_launch(const SolvePlan& p, const float* lam_acc, bool interleaved, float* lam_rho,
                                  float2* spec3comp, cudaStream_t st);
+// Rewrites a device kernel table in pass B's order (out null: only the size of
+// that, in bytes; 0 for N > 128, which has none).
+size_t kernel_quads(int N, const float* kern, float* out, cudaStream_t st);
 cudaError_t tile_window_launch(const SolvePlan& p, const float* src, int64_t tile, float* out, cudaStream_t st);
 
 // Per-launch CUDA-event timing, accumulated by kind.

@@ -35,16 +35,16 @@ template <int N> struct SolveCfg {
 #define PM_SOLVE_A_MINB 3
 #endif
 #ifndef PM_PASSB_KT
-#define PM_PASSB_KT 26
+#define PM_PASSB_KT 18
 #endif
 #ifndef PM_PASSB_TMA_THREADS
-#define PM_PASSB_TMA_THREADS 256
+#define PM_PASSB_TMA_THREADS 160
 #endif
 #ifndef PM_PASSB_TMA_MINB
-#define PM_PASSB_TMA_MINB 3
+#define PM_PASSB_TMA_MINB 5
 #endif
 #ifndef PM_SOLVE_C_THREADS
-#define PM_SOLVE_C_THREADS 416
+#define PM_SOLVE_C_THREADS 384
 #endif
 #ifndef PM_SOLVE_C_MINB
 #define PM_SOLVE_C_MINB 3
@@ -61,6 +61,7 @@ struct SolveArgs {
   float2* spec;
   float2* spec3;
   const float* kern;
+  const float4* kern_quads;   // pass B's layout of the kernel (null above 128)
   const float2* tw;
   float* dst;
   int comp_mode;   // pass A only: blockIdx.y selects component pb of a 3-component source at origin 0
@@ -481,11 +482,13 @@ __global__ void __launch_bounds__(PassA<N>::threads, PassA<N>::min_blocks)
 // run in registers per (k1, column) item; the second inverse step writes its
 // output rows straight to global memory (KT consecutive complex values each),
 // where it wrote all N rows to shared memory and a box store read back the
-// output ones: 3,140 -> 2,300 wavefronts per block of 96 x 26; 0.214 -> 0.212 ms
-// for 64 tiles, whose kernel-table loads and 24 warps per SM bound it now, and
-// 0.163 -> 0.106 ms for 216 tiles of 48^3, which one block of all 25 columns
-// serves.  Other shapes of 96: 320 threads at 3 blocks per SM 0.210 (spills), at
-// 2 blocks 0.230; 18 columns with 160 threads at 5 blocks 0.212, 224 at 4 0.215.
+// output ones (3,140 -> 2,300 wavefronts per block of 96 x 26).  The kernel
+// values lie in the order the items read them, 16 bytes per load, the first
+// component's fetched before the spectrum arrives and the next one's while the
+// current transform runs: 36 4-byte loads per item, each component's waited for
+// in turn, kept the earlier form at 0.212 ms for 64 tiles; 0.206 now, and 0.196
+// with 18 columns and 160 threads at 5 blocks per SM (18 x 224 at 4: 0.199;
+// 26 x 320 at 3: 0.197).  216 tiles of 48^3 0.163 -> 0.099 ms.
 template <int N> struct PassBR {
   static constexpr int NH = N / 2 + 1, NP = spec_pitch(N);
   // columns per block (N = 96: box rows of whole 16-byte words), and threads
@@ -493,10 +496,18 @@ template <int N> struct PassBR {
   static constexpr int KT = N == 128 ? 22 : (N == 96 ? PM_PASSB_KT : (N == 64 ? 17 : NH));
   static constexpr int nchunk = (NH + KT - 1) / KT;
   static constexpr int threads = N == 128 ? 192 : (N == 96 ? PM_PASSB_TMA_THREADS : (N == 48 ? 224 : (N == 16 ? 64 : 160)));
-  static constexpr int min_blocks = N >= 96 ? PM_PASSB_TMA_MINB : (N == 48 ? 3 : 4);
+  static constexpr int min_blocks = N == 128 ? 3 : (N == 96 ? PM_PASSB_TMA_MINB : (N == 48 ? 3 : 4));
   // G [3][N][KT] (component, z, column; the forward transform in component 0), twiddles
   static constexpr size_t smem = kTmaAlign + sizeof(float2) * (3 * (size_t)N * KT + N);
 };
+
+// Kernel values of one item and component: N2 / 4 words of 16 bytes, items
+// next to each other (kernel_quads lays them out so).
+template <int N>
+__device__ __forceinline__ void load_quads(float4 (&k)[Factor<N>::N2 / 4], const float4* p) {
+#pragma unroll
+  for (int q = 0; q < Factor<N>::N2 / 4; ++q) k[q] = __ldg(p + q * PassBR<N>::KT * Factor<N>::N1);
+}
 
 template <int N>
 __global__ void __launch_bounds__(PassBR<N>::threads, PassBR<N>::min_blocks)
@@ -510,6 +521,11 @@ __global__ void __launch_bounds__(PassBR<N>::threads, PassBR<N>::min_blocks)
   float2* tw = G + 3 * N * KT;
   const int ys = blockIdx.x, kx0 = blockIdx.y * KT, pb = blockIdx.z;
   const int ncol = NH - kx0 < KT ? NH - kx0 : KT;
+  // kernel values of this thread's first item and component: on their way
+  // while the spectrum is loaded and its first transform step runs
+  const float4* Kb = a.kern_quads + (size_t)(ys * B::nchunk + blockIdx.y) * (3 * (N2 / 4) * KT * N1);
+  float4 kq[N2 / 4];
+  if (threadIdx.x < KT * N1) load_quads<N>(kq, Kb + threadIdx.x);
   for (int i = threadIdx.x; i < N; i += T) tw[i] = a.tw[i];
   if constexpr (N == 96) {
     if (threadIdx.x == 0) {
@@ -548,24 +564,23 @@ __global__ void __launch_bounds__(PassBR<N>::threads, PassBR<N>::min_blocks)
   __syncthreads();
   // forward step 2, the products i K_d F and step 1 of each inverse
   // transform, per (k1, column) item: F(kz = k1 + N1 k2) sits at slot N2 k1 + k2
-  const float* Kb = a.kern + (size_t)ys * NH + kx0;
-  constexpr size_t kstride = (size_t)N * N * NH;
   for (int w = threadIdx.x; w < KT * N1; w += T) {
     const int k1 = w / KT, c = w - k1 * KT;
-    const bool live = c < ncol;
     float2 f[N2];
 #pragma unroll
     for (int j2 = 0; j2 < N2; ++j2) f[j2] = G[(N2 * k1 + j2) * KT + c];
     Dft<N2, -1>::run(f);
+    if (w >= T) load_quads<N>(kq, Kb + w);   // later rounds (the first one's are loaded already)
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      const float* Kd = Kb + d * kstride + (size_t)(N2 * k1) * N * NH + c;
       float2 g[N2];
 #pragma unroll
-      for (int k2 = 0; k2 < N2; ++k2) {
-        const float k = live ? __ldg(Kd + (size_t)k2 * N * NH) : 0.f;
-        g[k2] = make_float2(-f[k2].y * k, f[k2].x * k);   // i K f
+      for (int q = 0; q < N2 / 4; ++q) {
+        const float k[4] = {kq[q].x, kq[q].y, kq[q].z, kq[q].w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) g[4 * q + e] = make_float2(-f[4 * q + e].y * k[e], f[4 * q + e].x * k[e]);   // i K f
       }
+      if (d < 2) load_quads<N>(kq, Kb + (size_t)(d + 1) * (N2 / 4) * KT * N1 + w);   // in flight during this transform
       Dft<N2, 1>::run(g);
 #pragma unroll
       for (int j2 = 1; j2 < N2; ++j2) g[j2] = cmul(g[j2], conjf2(tw[j2 * k1]));
@@ -591,7 +606,7 @@ __global__ void __launch_bounds__(PassBR<N>::threads, PassBR<N>::min_blocks)
 #pragma unroll
       for (int j1 = 0; j1 < N1; ++j1) {
         const int zo = z0 + N2 * j1;
-        if (zo >= 0 && zo < a.t) o[(size_t)N2 * j1 * N * NP] = v[j1];
+        if ((unsigned)zo < (unsigned)a.t) o[(size_t)N2 * j1 * N * NP] = v[j1];
       }
     }
   }
@@ -611,13 +626,19 @@ __global__ void __launch_bounds__(PassBR<N>::threads, PassBR<N>::min_blocks)
 //   * the x steps give a warp's lanes different pairs (pitches NH 16-byte words
 //     and N + 1 complex values, both odd, so 8 or 16 lanes fall in different
 //     banks) where lanes along a row met 2 to 4 deep in a bank;
-//   * the output takes a pair's two rows from one 8-byte word and one pair of
-//     prolongation reads.
-// 2,600 wavefronts per plane: 0.244 ms (0.18 without the prolongation); 216
-// tiles of 48^3: 0.182 -> 0.143 ms.
+//   * the output takes a pair's two rows from one 8-byte word and the four rows
+//     between two coarse rows from one x interpolation each of the coarse force
+//     (fetched while the plane is on its way).
+// 2,600 wavefronts per plane, 0.291 -> 0.221 ms for 64 tiles; 216 tiles of 48^3:
+// 0.182 -> 0.103 ms.  It is bound by issue now (73% of the slots); 416 threads
+// (one round of the 392 column items) take 0.250 ms, 2 blocks per SM 0.309.
 // N = 128 keeps the y rows in place and the x step in registers across a
 // barrier (one buffer of 67 KB instead of two), so that 2 blocks share an SM:
 // 128^3 mesh 33 -> 21 us.
+
+// w / n for 0 <= w < 4096, n >= 1, with inv = 1 / n (w + 1/2 keeps the product
+// away from whole numbers by more than its rounding).
+__device__ __forceinline__ int quick_div(int w, float inv) { return (int)(((float)w + 0.5f) * inv); }
 
 template <int N> struct PassC {
   static constexpr int N1 = Factor<N>::N1, N2 = Factor<N>::N2;
@@ -631,7 +652,7 @@ template <int N> struct PassC {
   static size_t smem(int t, int b, int prc, bool prolong) {
     const size_t pairs = pair_count(t, b);
     const size_t nq = prolong ? t / prc + 1 : 0;
-    return align + sizeof(float2) * ((size_t)N * NP + N) + (in_place ? 4 * (nq * nq + nq * t) : 16 * pairs * NH);
+    return align + sizeof(float2) * ((size_t)N * NP + N) + (in_place ? 4 * nq * nq : 16 * pairs * NH);
   }
   static size_t smem_max() { return align + sizeof(float2) * ((size_t)N * NP + N) + (size_t)16 * (N / 2) * NH; }
   // row pairs (2 m, 2 m + 1) that hold the output rows b .. b + t - 1
@@ -661,6 +682,27 @@ __global__ void __launch_bounds__(PassC<N>::threads, PassC<N>::min_blocks) k_sol
     tma::mbar_arrive_expect_tx(&bar, bytes);
     tma::bulk_load(P, in, bytes, &bar);
   }
+  // Prolongation of the coarse force onto this output plane: the coarse values
+  // around the tile interior, interpolated in z.  Each thread fetches one while
+  // the plane is on its way (meshes with more take the rest later).
+  int ox, oy, oz;
+  problem_origin(a, a.p0 + pb, ox, oy, oz);
+  const int n = a.src_n, gz = oz + a.b + zo;
+  const int nq = a.pc ? a.t / a.prc + 1 : 0, lr = a.pc ? __ffs(a.prc) - 1 : 0;
+  const float inv_r = a.pc ? 1.0f / (float)a.prc : 0.f;
+  const auto coarse_value = [&](int i) {
+    const int qy = i / nq, qx = i - qy * nq;
+    const int cz0 = gz >> lr, cz1 = cz0 + 1 == a.pnc ? 0 : cz0 + 1;
+    const float wz = (float)(gz & (a.prc - 1)) * inv_r;
+    int cy = ((oy + a.b) >> lr) + qy, cx = ((ox + a.b) >> lr) + qx;
+    if (cy >= a.pnc) cy -= a.pnc;
+    if (cx >= a.pnc) cx -= a.pnc;
+    const size_t o = (size_t)cy * a.pnc + cx, plane = (size_t)a.pnc * a.pnc;
+    const float* c = a.pc + (size_t)d * a.pnc * plane;
+    return (1.0f - wz) * __ldg(c + cz0 * plane + o) + wz * __ldg(c + cz1 * plane + o);
+  };
+  float q_mine = 0.f;
+  if (threadIdx.x < nq * nq) q_mine = coarse_value(threadIdx.x);
   for (int i = threadIdx.x; i < N; i += T) tw[i] = a.tw[i];
   if (!block_wait(&bar, a.status)) return;
   // inverse y transform, step 1: items (k1, column)
@@ -679,6 +721,7 @@ __global__ void __launch_bounds__(PassC<N>::threads, PassC<N>::min_blocks) k_sol
   __syncthreads();
   // step 2: items (two neighbouring j2, column) -> rows N2 j1 + j2 and the next
   const int m0 = a.b >> 1, np = C::pair_count(a.t, a.b);
+  const float inv_np = 1.0f / (float)np;
   for (int w = threadIdx.x; w < (N2 / 2) * NH; w += T) {
     const int jp = w / NH, c = w - jp * NH;
     float2* base = P + 2 * jp * NP + c;
@@ -697,7 +740,7 @@ __global__ void __launch_bounds__(PassC<N>::threads, PassC<N>::min_blocks) k_sol
         base[(N2 * j1 + 1) * NP] = v[j1];
       } else {
         const int pair = (N2 / 2) * j1 + jp - m0;
-        if (pair >= 0 && pair < np) Y[pair * NH + c] = make_float4(u[j1].x, u[j1].y, v[j1].x, v[j1].y);
+        if ((unsigned)pair < (unsigned)np) Y[pair * NH + c] = make_float4(u[j1].x, u[j1].y, v[j1].x, v[j1].y);
       }
     }
   }
@@ -710,7 +753,7 @@ __global__ void __launch_bounds__(PassC<N>::threads, PassC<N>::min_blocks) k_sol
     for (int w0 = 0; w0 < np * N1; w0 += T) {
       const int w = w0 + threadIdx.x;
       const bool live = w < np * N1;
-      const int k1 = live ? w / np : 0, j = live ? w - k1 * np : 0;
+      const int k1 = live ? quick_div(w, inv_np) : 0, j = live ? w - k1 * np : 0;
       float2 v[N2];
 #pragma unroll
       for (int k2 = 0; k2 < N2; ++k2) {
@@ -744,41 +787,12 @@ __global__ void __launch_bounds__(PassC<N>::threads, PassC<N>::min_blocks) k_sol
     }
   }
   __syncthreads();
-  int ox, oy, oz;
-  problem_origin(a, a.p0 + pb, ox, oy, oz);
-  const int n = a.src_n;
-  // Prolongation of the coarse force onto this output plane: the coarse values
-  // around the tile interior, interpolated in z (Q; Y is free by now), then
-  // along x onto the output columns (R), so an output cell needs one
-  // interpolation in y.
-  float* Q = reinterpret_cast<float*>(Y);
-  const int nq = a.pc ? a.t / a.prc + 1 : 0;
-  float* R = Q + nq * nq;   // [nq][t]
-  int lr = 0;
-  float inv_r = 0.f;
-  if (a.pc) {
-    lr = __ffs(a.prc) - 1;
-    inv_r = 1.0f / (float)a.prc;
-    const int gz = oz + a.b + zo;
-    const int cz0 = gz >> lr, cz1 = cz0 + 1 == a.pnc ? 0 : cz0 + 1;
-    const float wz = (float)(gz & (a.prc - 1)) * inv_r;
-    const int cyb = (oy + a.b) >> lr, cxb = (ox + a.b) >> lr;
-    const float* c0 = a.pc + ((size_t)d * a.pnc + cz0) * a.pnc * a.pnc;
-    const float* c1 = a.pc + ((size_t)d * a.pnc + cz1) * a.pnc * a.pnc;
-    PM_ROWS(qy, nq) {
-      int cy = cyb + qy;
-      if (cy >= a.pnc) cy -= a.pnc;
-      PM_COLS(qx, nq) {
-        int cx = cxb + qx;
-        if (cx >= a.pnc) cx -= a.pnc;
-        const size_t o = (size_t)cy * a.pnc + cx;
-        Q[qy * nq + qx] = (1.0f - wz) * __ldg(c0 + o) + wz * __ldg(c1 + o);
-      }
-    }
-  }
+  float* Q = reinterpret_cast<float*>(Y);   // [nq][nq]; Y is free by now
+  if (threadIdx.x < nq * nq) Q[threadIdx.x] = q_mine;
+  for (int i = threadIdx.x + T; i < nq * nq; i += T) Q[i] = coarse_value(i);
   // step 2: items (j2, pair), natural x = N2 j1 + j2
   for (int w = threadIdx.x; w < np * N2; w += T) {
-    const int j2 = w / np, q = w - j2 * np;
+    const int j2 = quick_div(w, inv_np), q = w - j2 * np;
     float2* base = W + q * WP + j2;
     float2 v[N1];
 #pragma unroll
@@ -788,47 +802,61 @@ __global__ void __launch_bounds__(PassC<N>::threads, PassC<N>::min_blocks) k_sol
     for (int j1 = 0; j1 < N1; ++j1) base[N2 * j1] = v[j1];
   }
   __syncthreads();
-  if (a.pc) {
-    PM_ROWS(qy, nq) {
-      const float* q = Q + qy * nq;
-      PM_COLS(xl, a.t) {
-        const int qx = xl >> lr;
-        const float fx = (float)(xl & (a.prc - 1)) * inv_r;
-        R[qy * a.t + xl] = fmaf(fx, q[qx + 1] - q[qx], q[qx]);
-      }
-    }
-    __syncthreads();
-  }
   // Output cells are interior cells: origin + b + local lies inside [0, n) without wrap.
-  const int gz = oz + a.b + zo;
   float* dst = a.dst + (size_t)d * n * n * n + ((int64_t)gz * n + oy + a.b) * n + ox + a.b;
   float m = 0.f;
-  PM_ROWS(q, np) {
-    const int y0 = 2 * (m0 + q) - a.b, y1 = y0 + 1;   // the pair's output rows, if inside [0, t)
-    const bool in0 = y0 >= 0, in1 = y1 < a.t;
-    const int q0 = y0 >> lr, q1 = y1 >> lr;
-    const float f0 = (float)(y0 & (a.prc - 1)) * inv_r, f1 = (float)(y1 & (a.prc - 1)) * inv_r;
-    PM_COLS(xl, a.t) {
-      float2 w = W[q * WP + a.b + xl];
-      if (in0) m = fmaxf(m, fabsf(w.x));
-      if (in1) m = fmaxf(m, fabsf(w.y));
-      if (a.pc) {
-        float lo = 0.f, hi = 0.f;
-        if (in0) {
-          lo = R[q0 * a.t + xl];
-          hi = R[(q0 + 1) * a.t + xl];
-          w.x += fmaf(f0, hi - lo, lo);
-        }
-        if (in1) {
-          if (!in0 || q1 != q0) {
-            lo = R[q1 * a.t + xl];
-            hi = R[(q1 + 1) * a.t + xl];
-          }
-          w.y += fmaf(f1, hi - lo, lo);
-        }
+  if (a.pc && (a.b & 1) == 0) {
+    // a warp takes 32 columns of the rows between two coarse rows, which share
+    // their prolongation: lo at the lower coarse row, lo + f dlt between
+    const int nxb = (a.t + 31) >> 5, tasks = (nq - 1) * nxb;
+    const float inv_x = 1.0f / (float)nxb;
+    for (int task = threadIdx.x >> 5; task < tasks; task += T / 32) {
+      const int qy = quick_div(task, inv_x), xl = (task - qy * nxb) * 32 + (threadIdx.x & 31);
+      if (xl >= a.t) continue;
+      const float* q = Q + qy * nq + (xl >> lr);
+      const float fx = (float)(xl & (a.prc - 1)) * inv_r;
+      const float lo = fmaf(fx, q[1] - q[0], q[0]), dlt = fmaf(fx, q[nq + 1] - q[nq], q[nq]) - lo;
+      const float2* w = W + ((qy << lr) >> 1) * WP + a.b + xl;
+      float* o = dst + (int64_t)(qy << lr) * n + xl;
+      float f = 0.f;
+      for (int p = 0; p < a.prc; p += 2) {
+        const float2 val = *w;
+        m = fmaxf(m, fmaxf(fabsf(val.x), fabsf(val.y)));
+        o[0] = val.x + fmaf(f, dlt, lo);
+        o[n] = val.y + fmaf(f + inv_r, dlt, lo);
+        f += 2.0f * inv_r;
+        w += WP;
+        o += 2 * (int64_t)n;
       }
-      if (in0) dst[(int64_t)y0 * n + xl] = w.x;
-      if (in1) dst[(int64_t)y1 * n + xl] = w.y;
+    }
+  } else {
+    PM_ROWS(q, np) {
+      const int y0 = 2 * (m0 + q) - a.b, y1 = y0 + 1;   // the pair's output rows, if inside [0, t)
+      const bool in0 = y0 >= 0, in1 = y1 < a.t;
+      const int q0 = y0 >> lr, q1 = y1 >> lr;
+      const float f0 = (float)(y0 & (a.prc - 1)) * inv_r, f1 = (float)(y1 & (a.prc - 1)) * inv_r;
+      PM_COLS(xl, a.t) {
+        float2 w = W[q * WP + a.b + xl];
+        if (in0) m = fmaxf(m, fabsf(w.x));
+        if (in1) m = fmaxf(m, fabsf(w.y));
+        if (a.pc) {
+          const float fx = (float)(xl & (a.prc - 1)) * inv_r;
+          const auto along_x = [&](int qy) {
+            const float* q = Q + qy * nq + (xl >> lr);
+            return fmaf(fx, q[1] - q[0], q[0]);
+          };
+          if (in0) {
+            const float lo = along_x(q0), hi = along_x(q0 + 1);
+            w.x += fmaf(f0, hi - lo, lo);
+          }
+          if (in1) {
+            const float lo = along_x(q1), hi = along_x(q1 + 1);
+            w.y += fmaf(f1, hi - lo, lo);
+          }
+        }
+        if (in0) dst[(int64_t)y0 * n + xl] = w.x;
+        if (in1) dst[(int64_t)y1 * n + xl] = w.y;
+      }
     }
   }
   if (a.amax) {
@@ -1024,7 +1052,7 @@ static cudaError_t solve_large_n(const SolvePlan& p, const void* src, bool fixed
     cudaFuncSetAttribute(k_large_cx<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::smem_cx);
     attr_done = true;
   }
-  SolveArgs a{src, fixed ? 1 : 0, N, 1, N, 0, 0, p.spec, p.spec3, p.kern, p.tw, dst, 0, amax, nullptr, 0, 1, p.status};
+  SolveArgs a{src, fixed ? 1 : 0, N, 1, N, 0, 0, p.spec, p.spec3, p.kern, p.kern_quads, p.tw, dst, 0, amax, nullptr, 0, 1, p.status};
   {
     TimedScope ts(tm, "fft_a_mesh", st);
     if (fixed) k_large_ax<N, true><<<dim3(N / L::R, N), L::threads, L::smem_ax, st>>>(a);
@@ -1053,6 +1081,54 @@ __global__ void k_tile_window(const float* src, int src_n, int nts, int t, int b
     int x = (int)(i % N), y = (int)((i / N) % N), z = (int)(i / ((int64_t)N * N));
     int gx = pmod(ox + x, src_n), gy = pmod(oy + y, src_n), gz = pmod(oz + z, src_n);
     out[i] = src[((int64_t)gz * src_n + gy) * src_n + gx];
+  }
+}
+
+// Kernel table [3][z slot][y slot][NH] -> pass B's order [y slot][chunk][component]
+// [quad][k1][column] of float4: quad q of item (k1, column) holds kz slots
+// N2 k1 + 4 q .. + 3 (zero past the last column), so a warp's loads are
+// consecutive 16-byte words.
+template <int N>
+__global__ void k_kernel_quads(const float* kern, float* out) {
+  using B = PassBR<N>;
+  constexpr int NH = N / 2 + 1, N1 = Factor<N>::N1, N2 = Factor<N>::N2, KT = B::KT;
+  static_assert(N2 % 4 == 0, "whole quads");
+  constexpr int total = N * B::nchunk * 3 * N2 * KT * N1;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+    int r = i;
+    const int e = r % 4;
+    r /= 4;
+    const int c = r % KT;
+    r /= KT;
+    const int k1 = r % N1;
+    r /= N1;
+    const int q = r % (N2 / 4);
+    r /= N2 / 4;
+    const int d = r % 3;
+    r /= 3;
+    const int ch = r % B::nchunk, ys = r / B::nchunk;
+    const int kx = ch * KT + c, zs = N2 * k1 + 4 * q + e;
+    out[i] = kx < NH ? kern[(((size_t)d * N + zs) * N + ys) * NH + kx] : 0.f;
+  }
+}
+template <int N>
+static size_t quads_n(const float* kern, float* out, cudaStream_t st) {
+  using B = PassBR<N>;
+  if (out) {
+    k_kernel_quads<N><<<152 * 4, 256, 0, st>>>(kern, out);
+    note_launches(1);
+  }
+  return (size_t)N * B::nchunk * 3 * Factor<N>::N2 * B::KT * Factor<N>::N1 * sizeof(float);
+}
+size_t kernel_quads(int N, const float* kern, float* out, cudaStream_t st) {
+  switch (N) {
+    case 16: return quads_n<16>(kern, out, st);
+    case 32: return quads_n<32>(kern, out, st);
+    case 48: return quads_n<48>(kern, out, st);
+    case 64: return quads_n<64>(kern, out, st);
+    case 96: return quads_n<96>(kern, out, st);
+    case 128: return quads_n<128>(kern, out, st);
+    default: return 0;
   }
 }
 
@@ -1086,7 +1162,7 @@ static cudaError_t solve_n(const SolvePlan& p, const void* src, bool fixed, floa
   const int nprob = p.nts * p.nts * p.nts;
   for (int p0 = 0; p0 < nprob; p0 += p.batch) {
     int nb = (nprob - p0 < p.batch) ? (nprob - p0) : p.batch;
-    SolveArgs a{src, fixed ? 1 : 0, p.src_n, p.nts, p.t, p.b, p0, p.spec, p.spec3, p.kern, p.tw, dst, 0, amax,
+    SolveArgs a{src, fixed ? 1 : 0, p.src_n, p.nts, p.t, p.b, p0, p.spec, p.spec3, p.kern, p.kern_quads, p.tw, dst, 0, amax,
                 pro ? pro->coarse : nullptr, pro ? pro->nc : 0, pro ? pro->rc : 1, p.status};
     {
       TimedScope ts(tm, N == p.src_n && p.b == 0 ? "fft_a_mesh" : "fft_a_tiles", st);
@@ -1141,7 +1217,7 @@ static cudaError_t solve_adjoint_n(const SolvePlan& p, const float* lam_acc, boo
   cudaFuncSetAttribute(ka, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassA<N>::smem);
   cudaFuncSetAttribute(k_solve_b_adj<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(float2) * (N + 2 * (size_t)N * PassB<N>::KC)));
   cudaFuncSetAttribute(k_solve_c<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassC<N>::smem_max());
-  SolveArgs a{lam_acc, 0, p.src_n, 1, N, 0, 0, spec3comp, p.spec3, p.kern, p.tw, lam_rho, 1, nullptr, nullptr, 0, 1,
+  SolveArgs a{lam_acc, 0, p.src_n, 1, N, 0, 0, spec3comp, p.spec3, p.kern, p.kern_quads, p.tw, lam_rho, 1, nullptr, nullptr, 0, 1,
               p.status};
   ka<<<dim3(N, 3), PassA<N>::threads, PassA<N>::smem, st>>>(a, CUtensorMap{});
   a.comp_mode = 0;
