@@ -268,7 +268,9 @@ Blk choose_blk(const Geom& g, bool fixed, bool deposit) {
   if (!deposit) {
     while (b.RX > 1 && b.RX % 2 == 0 && kick_count_smem(geo, b) > 100 * 1024) b.RX /= 2;
   } else {
-    while (b.RX > 1 && b.RX % 2 == 0 && deposit_codes_smem(geo, b, fixed) > 64 * 1024) b.RX /= 2;
+    // the float deposit of rows of at most 64 cells is the fast one (particles.cu)
+    const int most = !fixed && g.rcmp == 4 ? 64 : g.ncmp;
+    while (b.RX > 1 && b.RX % 2 == 0 && (b.RX > most || deposit_codes_smem(geo, b, fixed) > 64 * 1024)) b.RX /= 2;
   }
   b.nbx = g.ncmp / b.RX;
   b.nby = g.ncmp / b.RY;

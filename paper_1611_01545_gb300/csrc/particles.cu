@@ -109,23 +109,6 @@ __device__ __forceinline__ void global_add(long long* a, long long v) {
   atomicAdd(reinterpret_cast<unsigned long long*>(a), (unsigned long long)v);
 }
 
-// Compile-time cell-block shape: RX_ > 0 fixes RX, RY, RZ and the fine cells per
-// compression cell (the shapes the autotuner picks on the benchmark meshes), so
-// the staged region's strides and the row search are constants; 0 reads them
-// from the arguments.
-#ifndef PM_SHAPE_INSTANCES
-#define PM_SHAPE_INSTANCES 1
-#endif
-template <int RX_, int RY_, int RZ_, int R_>
-__device__ __forceinline__ void fix_shape(Geo& g, Blk& bk) {
-  if (RX_ > 0) {
-    bk.RX = RX_;
-    bk.RY = RY_;
-    bk.RZ = RZ_;
-    g.rcmp = R_;
-  }
-}
-
 // Mass of each CIC corner: float mode m w_x w_y w_z in float32; fixed mode
 // the conservative integer split of the fixed-point deposit (2^-32 units).
 __device__ __forceinline__ void corner_masses(float m, long long, const float w1[3], float out[8]) {
@@ -165,13 +148,10 @@ __device__ __forceinline__ void corner_masses(float, long long M, const float w1
 #else
 #define PM_DEPOSIT_BOUNDS
 #endif
-template <typename Acc, int RX_, int RY_, int RZ_, int R_>
-__global__ void PM_DEPOSIT_BOUNDS k_deposit_codes(PCodes c0, PCodes c1, const int64_t* off0, const int64_t* off1, Geo g_arg, Blk bk_arg,
+template <typename Acc>
+__global__ void PM_DEPOSIT_BOUNDS k_deposit_codes(PCodes c0, PCodes c1, const int64_t* off0, const int64_t* off1, Geo g, Blk bk,
                                 float m0, float m1, long long M0, long long M1, Acc* rho_c, Acc* rho_f) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  Geo g = g_arg;
-  Blk bk = bk_arg;
-  fix_shape<RX_, RY_, RZ_, R_>(g, bk);
   for_each_block(bk, [&](const int bid) {
     const int r = g.rcmp;
     const int fx = bk.RX * r + 1, fy = bk.RY * r + 1, fz = bk.RZ * r + 1;
@@ -389,6 +369,217 @@ __global__ void PM_DEPOSIT_BOUNDS k_deposit_codes(PCodes c0, PCodes c1, const in
   });
 }
 
+// ---- deposit of the shapes in use -------------------------------------------
+//
+// The float deposit for blocks of RX_MAX x RY x RZ compression cells of 4 fine
+// cells or shorter in x (the shapes of the defaults and of tuned programs); other
+// shapes, ratios and the int64 mode take the kernel above.  Issue bound (74% of
+// issue slots), a third of it spent on the block's 1.3 nodes per particle
+// rather than on the particles, so:
+//   * strides are constants, offsets and indices 32-bit and relative to the
+//     cell row, the fine node comes from the code's upper 2 bits and the
+//     weight (2 q + 1) / 128 from its lower 6: weights are kept in units of
+//     1 / 128, exact in float32, and the scaled mass takes the powers of two;
+//   * one walk over the bins converts, adds four nodes at a time to the mesh
+//     (16-byte reductions), and forms the x restriction of the coarse density
+//     from the same four values and the left neighbour's carry.
+// 256^3 workload 0.178 -> 0.118 ms (blocks of 32 x 2 x 1; with its launch 0.192 ->
+// 0.130, 64 x 1 x 1 0.125, 32 x 2 x 2 0.177: 5 instead of 6 CTAs per SM and spills),
+// 768^3 (5.1e8 particles) 4.56 -> 2.98 ms, clustered 512^3 in its default shape
+// 1.71 -> 0.89 ms.
+template <int RX_MAX, int RY, int RZ> struct DepShape {
+  static constexpr int row = 4 * RX_MAX + 4;          // words per bin row (4 RX + 1 used), whole 16-byte words
+  static constexpr int fy = 4 * RY + 1, fz = 4 * RZ + 1, rows = fy * fz;
+  static constexpr int plane = row * fy;
+  static constexpr int cx = RX_MAX + 1, cy = RY + 1, cz = RZ + 1;
+  static constexpr int lists = RY * RZ;                // cell rows
+  // bins, x-restricted rows, xy-restricted rows, relative offsets of both species
+  static constexpr size_t smem = 4 * ((size_t)plane * fz + rows * cx + fz * cy * cx + 2 * lists * RX_MAX);
+};
+// Compile-time tunables: resident CTAs per SM of the deposit.
+#ifndef PM_DEPOSIT_ROWS_MINB
+#define PM_DEPOSIT_ROWS_MINB 6
+#endif
+
+// Weight of the coarse tent at distance k fine cells (ratio 4).
+__device__ __forceinline__ float tent4(int k) { return 1.0f - 0.25f * (float)(k < 0 ? -k : k); }
+
+template <int RX_MAX, int RY, int RZ>
+__global__ void __launch_bounds__(PM_DEPOSIT_THREADS, PM_DEPOSIT_ROWS_MINB)
+    k_deposit_rows(PCodes c0, PCodes c1, const int64_t* off0, const int64_t* off1, Geo g, Blk bk, float m0, float m1,
+                   float* rho_c, float* rho_f) {
+  using D = DepShape<RX_MAX, RY, RZ>;
+  constexpr int T = PM_DEPOSIT_THREADS;
+  constexpr uint32_t kSeg = 1u << 30;   // particles of a cell row handled with one set of 32-bit offsets
+  extern __shared__ __align__(16) unsigned char smraw[];
+  uint32_t* bins = reinterpret_cast<uint32_t*>(smraw);
+  float* T1 = reinterpret_cast<float*>(bins + D::plane * D::fz);   // [fz][fy][cx]
+  float* T2 = T1 + D::rows * D::cx;                                 // [fz][cy][cx]
+  uint32_t* rel = reinterpret_cast<uint32_t*>(T2 + D::fz * D::cy * D::cx);   // [species][list][RX_MAX]
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for_each_block(bk, [&](const int bid) {
+    const int RX = bk.RX, cx = RX + 1;
+    const CellBlock cb = block_of(bk, bid);
+    for (int i = threadIdx.x; i < D::plane * D::fz / 4; i += T) reinterpret_cast<uint4*>(bins)[i] = make_uint4(0, 0, 0, 0);
+    // Offsets of the block's cell rows and the mass of its heaviest cell: 8
+    // times that bounds every node's total (a node receives mass only from the
+    // at most 8 compression cells around it), so with the power of two S =
+    // 2^floor(log2(2^31 / bound)) the scaled totals stay below 2^31, and the
+    // corner roundings below 2^31 more.
+    float cm = 0.f;
+    for (int i = threadIdx.x; i < D::lists * RX_MAX; i += T) {
+      const int l = i / RX_MAX, j = i - l * RX_MAX;
+      uint32_t r0 = kSeg, r1 = kSeg;
+      if (j < RX) {
+        const int64_t c = cb.ix0 + (int64_t)g.ncmp * (cb.iy0 + l % RY + (int64_t)g.ncmp * (cb.iz0 + l / RY));
+        const int64_t a0 = off0[c + j], a1 = off1[c + j];
+        const int64_t d0 = a0 - off0[c], d1 = a1 - off1[c];
+        r0 = d0 < kSeg ? (uint32_t)d0 : kSeg;
+        r1 = d1 < kSeg ? (uint32_t)d1 : kSeg;
+        const int64_t b0 = off0[c + j + 1], b1 = off1[c + j + 1];
+        const int64_t n0 = (b0 < c0.n ? b0 : c0.n) - (a0 < c0.n ? a0 : c0.n);
+        const int64_t n1 = (b1 < c1.n ? b1 : c1.n) - (a1 < c1.n ? a1 : c1.n);
+        cm = fmaxf(cm, __fadd_ru(__fmul_ru((float)n0, m0), __fmul_ru((float)n1, m1)));
+      }
+      rel[i] = r0;
+      rel[D::lists * RX_MAX + i] = r1;
+    }
+    cm = block_max_all(cm);   // (its barriers also order the bins and offsets)
+    float S = 1.f;
+    if (cm > 0.f) {
+      const float x = fminf(__fdiv_rd(268435456.0f, cm), 1.329228e36f);   // 2^31 / (8 cm), at most 2^120
+      S = __uint_as_float(__float_as_uint(x) & 0xff800000u);
+    }
+    for (int s = 0; s < 2; ++s) {
+      const int64_t n = s ? c1.n : c0.n;
+      // corner value m S w_x w_y w_z with weights in units of 1 / 128
+      const float m = __fmul_rn(__fmul_rn(s ? m1 : m0, S), 1.0f / 2097152.0f);
+      for (int l = 0; l < D::lists; ++l) {
+        const int64_t* off = (s ? off1 : off0) + cb.ix0 +
+                             (int64_t)g.ncmp * (cb.iy0 + l % RY + (int64_t)g.ncmp * (cb.iz0 + l / RY));
+        uint32_t* ro = rel + (s * D::lists + l) * RX_MAX;
+        uint32_t* lbins = bins + (l / RY) * 4 * D::plane + (l % RY) * 4 * D::row;
+        // a corrupt stream (flagged by the scan) may claim more particles than
+        // exist; never read past the caller's n records
+        const int64_t o0 = off[0], o1 = off[RX];
+        const int64_t p0 = o0 < n ? o0 : n, p1 = o1 < n ? o1 : n;
+        for (int64_t seg = p0; seg < p1; seg += kSeg) {
+          if (seg > p0) {   // a row of more than 2^30 particles: offsets of its next part
+            __syncthreads();
+            for (int j = threadIdx.x; j < RX; j += T) {
+              const int64_t d = off[j] - seg;
+              ro[j] = d <= 0 ? 0u : (d < kSeg ? (uint32_t)d : kSeg);
+            }
+            __syncthreads();
+          }
+          const uint32_t count = p1 - seg < kSeg ? (uint32_t)(p1 - seg) : kSeg;
+          const uint32_t* pos = (s ? c1.pos : c0.pos) + seg;
+          uint32_t next = threadIdx.x < count ? pos[threadIdx.x] : 0u;
+          for (uint32_t i = threadIdx.x; i < count; i += T) {
+            const uint32_t pw = next;
+            if (i + T < count) next = pos[i + T];
+            // the last cell whose offset is at most i (entries past the row hold 2^30)
+            int k = 0;
+#pragma unroll
+            for (int d = RX_MAX / 2; d > 0; d >>= 1)
+              if (ro[k + d] <= i) k += d;
+            const uint32_t hi = (pw >> 6) & 0x030303u, lo = ((pw & 0x3f3f3fu) << 1) | 0x010101u;
+            uint32_t* b = lbins + 4 * k + (hi & 3u) + D::row * ((hi >> 8) & 3u) + D::plane * (hi >> 16);
+            const float wx1 = __uint2float_rn(lo & 0xffu), wy1 = __uint2float_rn((lo >> 8) & 0xffu),
+                        wz1 = __uint2float_rn(lo >> 16);
+            const float wx0 = 128.0f - wx1, wy0 = 128.0f - wy1;
+            const float mz1 = __fmul_rn(m, wz1), mz0 = __fmul_rn(m, 128.0f - wz1);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+              const float wxy = __fmul_rn(c & 1 ? wx1 : wx0, (c >> 1) & 1 ? wy1 : wy0);   // exact
+              atomicAdd(b + (c & 1) + D::row * ((c >> 1) & 1) + D::plane * (c >> 2),
+                        __float2uint_rn(__fmul_rn(wxy, c >> 2 ? mz1 : mz0)));
+            }
+          }
+        }
+      }
+    }
+    __syncthreads();
+    // One warp per bin row: fixed point -> float32 (S is a power of two: exact),
+    // four nodes per lane, to the mesh; the restriction along x on the way,
+    // R[q] = sum_k w(k) row[4 q + k].
+    const float inv_s = 1.0f / S;
+    const int nf = g.nf, bxf = 4 * cb.ix0;
+    for (int line = warp; line < D::rows; line += T / 32) {
+      const int lz = line / D::fy, ly = line - lz * D::fy;
+      int gy = 4 * cb.iy0 + ly, gz = 4 * cb.iz0 + lz;
+      if (gy >= nf) gy -= nf;
+      if (gz >= nf) gz -= nf;
+      float* grow = rho_f + ((int64_t)gz * nf + gy) * nf;
+      const uint32_t* row = bins + lz * D::plane + ly * D::row;
+      float carry = 0.f;                                  // what the cells left of lane 0 give its coarse cell
+      for (int q0 = 0; q0 < RX; q0 += 32) {
+        const int q = q0 + lane;
+        const bool in = q < RX;
+        const uint4 u = in ? reinterpret_cast<const uint4*>(row)[q] : make_uint4(0, 0, 0, 0);
+        float4 v;
+        v.x = __fmul_rn(__uint2float_rn(u.x), inv_s);
+        v.y = __fmul_rn(__uint2float_rn(u.y), inv_s);
+        v.z = __fmul_rn(__uint2float_rn(u.z), inv_s);
+        v.w = __fmul_rn(__uint2float_rn(u.w), inv_s);
+        if ((u.x | u.y | u.z | u.w) != 0u) atomicAdd(reinterpret_cast<float4*>(grow + bxf) + q, v);
+        const float up = fmaf(0.75f, v.w, fmaf(0.5f, v.z, 0.25f * v.y));          // for the coarse cell to the right
+        const float own = fmaf(0.25f, v.w, fmaf(0.5f, v.z, fmaf(0.75f, v.y, v.x)));
+        float left = __shfl_up_sync(0xffffffffu, up, 1);
+        if (lane == 0) left = carry;
+        if (in) T1[line * D::cx + q] = own + left;
+        carry = __shfl_sync(0xffffffffu, up, RX - q0 < 32 ? RX - 1 - q0 : 31);
+      }
+      if (lane == 0) {                                    // the upper halo node
+        const float v = __fmul_rn(__uint2float_rn(row[4 * RX]), inv_s);
+        const int gx = bxf + 4 * RX == nf ? 0 : bxf + 4 * RX;
+        if (v != 0.f) atomicAdd(grow + gx, v);
+        T1[line * D::cx + RX] = v + carry;
+      }
+    }
+    if (!rho_c) return;
+    __syncthreads();
+    for (int i = threadIdx.x; i < D::fz * D::cy * D::cx; i += T) {
+      const int q = i % D::cx, qy = i / D::cx % D::cy, lz = i / (D::cx * D::cy);
+      if (q >= cx) continue;
+      float t = 0.f;
+#pragma unroll
+      for (int k = -3; k <= 3; ++k) {
+        const int j = 4 * qy + k;
+        if (j >= 0 && j < D::fy) t = fmaf(tent4(k), T1[(lz * D::fy + j) * D::cx + q], t);
+      }
+      T2[i] = t;
+    }
+    __syncthreads();
+    const int nc = g.nc;
+    for (int i = threadIdx.x; i < D::cz * D::cy * D::cx; i += T) {
+      const int q = i % D::cx, qy = i / D::cx % D::cy, qz = i / (D::cx * D::cy);
+      if (q >= cx) continue;
+      float t = 0.f;
+#pragma unroll
+      for (int k = -3; k <= 3; ++k) {
+        const int j = 4 * qz + k;
+        if (j >= 0 && j < D::fz) t = fmaf(tent4(k), T2[(j * D::cy + qy) * D::cx + q], t);
+      }
+      int gx = cb.ix0 + q, gy = cb.iy0 + qy, gz = cb.iz0 + qz;
+      if (gx >= nc) gx -= nc;
+      if (gy >= nc) gy -= nc;
+      if (gz >= nc) gz -= nc;
+      if (t != 0.f) atomicAdd(rho_c + ((int64_t)gz * nc + gy) * nc + gx, t);
+    }
+  });
+}
+
+template <int RX_MAX, int RY, int RZ>
+static void launch_rows(const PCodes& c0, const PCodes& c1, const int64_t* off0, const int64_t* off1, const Geo& g,
+                        const Blk& bk, float m0, float m1, float* rho_c, float* rho_f, cudaStream_t st) {
+  const auto k = k_deposit_rows<RX_MAX, RY, RZ>;
+  constexpr size_t smem = DepShape<RX_MAX, RY, RZ>::smem;
+  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  k<<<block_grid(k, bk, PM_DEPOSIT_THREADS, smem), PM_DEPOSIT_THREADS, smem, st>>>(c0, c1, off0, off1, g, bk, m0, m1,
+                                                                                   g.two ? rho_c : nullptr, rho_f);
+}
+
 // ------------------------------------------------------------ launchers --
 
 static int grid_for(int64_t n, int threads) {
@@ -425,20 +616,25 @@ size_t deposit_codes_smem(const Geo& g, const Blk& bk, bool fixed) {
 cudaError_t launch_deposit_codes(const PCodes& c0, const PCodes& c1, const int64_t* off0, const int64_t* off1,
                                  const Geo& g, const Blk& bk, float m0, float m1, long long M0, long long M1,
                                  void* rho_c, void* rho_f, bool fixed, cudaStream_t st) {
-  size_t smem = deposit_codes_smem(g, bk, fixed);
-  int nblk = bk.nbx * bk.nby * bk.nbz;
-  const bool tuned = PM_SHAPE_INSTANCES && bk.RX == 32 && bk.RY == 2 && bk.RZ == 1 && g.rcmp == 4;
-  if (fixed) {
-    cudaFuncSetAttribute(k_deposit_codes<long long, 0, 0, 0, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    nblk = block_grid(k_deposit_codes<long long, 0, 0, 0, 0>, bk, PM_DEPOSIT_THREADS, smem);
-    k_deposit_codes<long long, 0, 0, 0, 0><<<nblk, PM_DEPOSIT_THREADS, smem, st>>>(c0, c1, off0, off1, g, bk, m0, m1, M0, M1,
-                                                       static_cast<long long*>(rho_c), static_cast<long long*>(rho_f));
-  } else {
-    const auto k = tuned ? k_deposit_codes<float, 32, 2, 1, 4> : k_deposit_codes<float, 0, 0, 0, 0>;
+  const size_t smem = deposit_codes_smem(g, bk, fixed);
+  // the row kernel adds 16-byte words to the mesh: its base must be aligned (its rows are, nf = 4 n_cmp)
+  const bool rows = !fixed && g.rcmp == 4 && (!g.two || g.rc == 4) && (reinterpret_cast<uintptr_t>(rho_f) & 15) == 0;
+  float* rc = static_cast<float*>(rho_c);
+  float* rf = static_cast<float*>(rho_f);
+  if (rows && bk.RX <= 64 && bk.RY == 1 && bk.RZ == 1) {
+    launch_rows<64, 1, 1>(c0, c1, off0, off1, g, bk, m0, m1, rc, rf, st);
+  } else if (rows && bk.RX <= 32 && bk.RY == 2 && bk.RZ == 1) {
+    launch_rows<32, 2, 1>(c0, c1, off0, off1, g, bk, m0, m1, rc, rf, st);
+  } else if (fixed) {
+    const auto k = k_deposit_codes<long long>;
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    nblk = block_grid(k, bk, PM_DEPOSIT_THREADS, smem);
-    k<<<nblk, PM_DEPOSIT_THREADS, smem, st>>>(c0, c1, off0, off1, g, bk, m0, m1, M0, M1, static_cast<float*>(rho_c),
-                                              static_cast<float*>(rho_f));
+    k<<<block_grid(k, bk, PM_DEPOSIT_THREADS, smem), PM_DEPOSIT_THREADS, smem, st>>>(
+        c0, c1, off0, off1, g, bk, m0, m1, M0, M1, static_cast<long long*>(rho_c), static_cast<long long*>(rho_f));
+  } else {
+    const auto k = k_deposit_codes<float>;
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k<<<block_grid(k, bk, PM_DEPOSIT_THREADS, smem), PM_DEPOSIT_THREADS, smem, st>>>(c0, c1, off0, off1, g, bk, m0, m1,
+                                                                                     M0, M1, rc, rf);
   }
   note_launches(1);
   return cudaGetLastError();
