@@ -85,15 +85,18 @@ __device__ __forceinline__ void accel_at(const Geo& g, const float* acc_c, const
   }
 }
 
-__device__ __forceinline__ float wrap_pos(float x, float nf) {
-  if (x < 0.f) x = __fadd_rn(x, nf);
-  if (x >= nf) x = __fsub_rn(x, nf);
-  if (!(x >= 0.f && x < nf)) {      // moved more than one box length, or rounding onto nf
-    x = __fsub_rn(x, __fmul_rn(nf, floorf(__fdiv_rn(x, nf))));
-    if (!(x >= 0.f && x < nf)) x = 0.f;
-  }
-  return x;
+// A position at most one box length outside [0, nf), brought back in; then
+// (wrap_far) one that moved further, or was rounded onto nf, or is no number.
+__device__ __forceinline__ float wrap_near(float x, float nf) {
+  x = x < 0.f ? __fadd_rn(x, nf) : x;
+  return x >= nf ? __fsub_rn(x, nf) : x;
 }
+__device__ __forceinline__ float wrap_far(float x, float nf) {
+  if (x >= 0.f && x < nf) return x;
+  x = __fsub_rn(x, __fmul_rn(nf, floorf(__fdiv_rn(x, nf))));
+  return x >= 0.f && x < nf ? x : 0.f;
+}
+__device__ __forceinline__ float wrap_pos(float x, float nf) { return wrap_far(wrap_near(x, nf), nf); }
 
 // v' = v + c_k a ; x' = wrap(x + c_d v')
 __device__ __forceinline__ void kick_drift(float x[3], float v[3], const float a[3], float ck, float cd, float nf) {

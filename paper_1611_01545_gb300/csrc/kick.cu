@@ -99,14 +99,18 @@ __device__ __forceinline__ Win window_of(const Geo& g, const Blk& bk, CellBlock 
   return w;
 }
 // Window slot of the compression cell with coordinates (cx, cy, cz), or -1.
-__device__ __forceinline__ int window_slot_xyz(const Win& w, int n, int cx, int cy, int cz) {
-  int lx = cx - w.ox, ly = cy - w.oy, lz = cz - w.oz;
-  lx += lx < 0 ? n : (lx >= n ? -n : 0);
-  ly += ly < 0 ? n : (ly >= n ? -n : 0);
-  lz += lz < 0 ? n : (lz >= n ? -n : 0);
-  if (lx >= w.wx || ly >= w.wy || lz >= w.wz) return -1;
-  return (lz * w.wy + ly) * w.wx + lx;
+// The offset from the window's origin lies in (-n, n + D]; of l, l + n and
+// l - n the one in [0, n) is the smallest as an unsigned number.
+__device__ __forceinline__ unsigned window_offset(int c, int o, unsigned n) {
+  const unsigned l = (unsigned)(c - o);
+  return min(min(l, l + n), l - n);
 }
+__device__ __forceinline__ int window_slot_xyz(const Win& w, int n, int cx, int cy, int cz) {
+  const unsigned lx = window_offset(cx, w.ox, n), ly = window_offset(cy, w.oy, n), lz = window_offset(cz, w.oz, n);
+  const bool in = lx < (unsigned)w.wx && ly < (unsigned)w.wy && lz < (unsigned)w.wz;
+  return in ? (int)((lz * w.wy + ly) * w.wx + lx) : -1;
+}
+
 // Per-particle scratch record of the two recompress passes (stream index t
 // of ntot particles, both species).  Exact v_max' mode: one 16-byte record
 // {new position word, v'_x, v'_y, v'_z as float bits}.  Bound mode (codes
@@ -184,23 +188,25 @@ struct KickArgs {
 };
 
 // Rank of the calling lane among the block's particles of its window slot:
-// what atomicAdd(hist + slot, 1) would return.  Consecutive lanes with the
-// same slot form a run (the stream is cell ordered and cold particles stay in
-// their cell); the run's first lane takes the run's ranks with one atomic,
-// since a shared-memory atomic whose lanes share an address and return their
-// values is serialised lane by lane.  All 32 lanes must call it; lanes without
-// a slot pass has = false and a slot of their own (~0u - lane).
-__device__ __forceinline__ uint32_t run_rank(uint32_t* hist, uint32_t slot, bool has) {
+// what atomicAdd(hist + slot, 1) returns.  A shared-memory atomic whose lanes
+// share an address and return their values is serialised lane by lane, and the
+// stream is cell ordered: cold particles stay in their cell, and consecutive
+// lanes have the same slot.  Where half of the lanes continue their
+// neighbour's run, the first lane of each run takes the run's ranks with one
+// atomic; hot particles, which scatter, take them one by one.  All 32 lanes
+// must call it; lanes without a slot pass has = false and a slot of their own
+// (~0u - lane).
+__device__ __forceinline__ uint32_t slot_rank(uint32_t* hist, uint32_t slot, bool has) {
   const int lane = (int)(threadIdx.x & 31);
   const uint32_t prev = __shfl_up_sync(0xffffffffu, slot, 1);
-  const bool head = lane == 0 || prev != slot;
-  const uint32_t heads = __ballot_sync(0xffffffffu, head);
+  const uint32_t heads = __ballot_sync(0xffffffffu, lane == 0 || prev != slot);
+  if (__popc(heads) > 16) return has ? atomicAdd(hist + slot, 1u) : 0u;
   const uint32_t upto = 0xffffffffu >> (31 - lane);   // lanes 0 .. lane
   const int first = 31 - __clz(heads & upto);         // head of this lane's run
   const uint32_t later = heads & ~upto;
   const int end = later ? __ffs(later) - 1 : 32;       // head of the next run
   uint32_t old = 0;
-  if (head && has) old = atomicAdd(hist + slot, (uint32_t)(end - lane));
+  if (lane == first && has) old = atomicAdd(hist + slot, (uint32_t)(end - lane));
   old = __shfl_sync(0xffffffffu, old, first);
   return old + (uint32_t)(lane - first);
 }
@@ -220,7 +226,7 @@ struct Kicked {
 
 // Kick, drift and recode one particle whose gathered acceleration is a, and
 // store its key and record: tk and rec point at the particle's own.  All lanes
-// of the warp call it (run_rank); live: the lane has a particle.
+// of the warp call it (slot_rank); live: the lane has a particle.
 // Positions are recoded in one conversion: x 256 / r is exact (a power of two
 // times x) and below 2^24, so its integer part holds the cell (upper bits) and
 // the in-cell code (low byte), the same as floor(x / r) and floor(256 frac).
@@ -231,11 +237,11 @@ __device__ __forceinline__ void kick_and_store(const Kicked& k, bool live, float
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     v[d] = __fmaf_rn(k.ck, a[d], v[d]);
-    x[d] = __fmaf_rn(k.cd, v[d], x[d]);
+    x[d] = wrap_near(__fmaf_rn(k.cd, v[d], x[d]), k.nf);
   }
   if (!(x[0] >= 0.f && x[0] < k.nf && x[1] >= 0.f && x[1] < k.nf && x[2] >= 0.f && x[2] < k.nf)) {
 #pragma unroll
-    for (int d = 0; d < 3; ++d) x[d] = wrap_pos(x[d], k.nf);
+    for (int d = 0; d < 3; ++d) x[d] = wrap_far(x[d], k.nf);
   }
   int code[3], cell[3];
 #pragma unroll
@@ -245,7 +251,7 @@ __device__ __forceinline__ void kick_and_store(const Kicked& k, bool live, float
   }
   const int slot = window_slot_xyz(k.win, k.n, cell[0], cell[1], cell[2]);
   const bool inw = live && slot >= 0;
-  const uint32_t rank = run_rank(k.hist, inw ? (uint32_t)slot : ~0u - (threadIdx.x & 31), inw);
+  const uint32_t rank = slot_rank(k.hist, inw ? (uint32_t)slot : ~0u - (threadIdx.x & 31), inw);
   if (!live) return;
   uint32_t key;
   if (inw && (rank >> k.kb) == 0) {
