@@ -67,9 +67,11 @@ __global__ void k_adj_deposit(const float* x, int64_t np, float m, int n, const 
   }
 }
 
-template <bool V4>
-__global__ void k_adj_interp(const float* x, int64_t np, int n, const float* acc, float ck, float cd, float* lam_x,
-                             float* lam_v, float* lam_A) {
+// V4: lam_A interleaved; A4: acc interleaved (acc4), one 16-byte load per corner
+// (reverse step of 2.4M particles in random order on 128^3: 380 -> 289 us).
+template <bool V4, bool A4>
+__global__ void k_adj_interp(const float* x, int64_t np, int n, const float* acc, const float4* acc4, float ck, float cd,
+                             float* lam_x, float* lam_v, float* lam_A) {
   const int64_t n3 = (int64_t)n * n * n;
   for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < np; p += (int64_t)gridDim.x * blockDim.x) {
     const float xp[3] = {x[3 * p], x[3 * p + 1], x[3 * p + 2]};
@@ -94,7 +96,9 @@ __global__ void k_adj_interp(const float* x, int64_t np, int n, const float* acc
         atomicAdd(lam_A + n3 + idx, la[1] * w);
         atomicAdd(lam_A + 2 * n3 + idx, la[2] * w);
       }
-      const float dot = la[0] * __ldg(acc + idx) + la[1] * __ldg(acc + n3 + idx) + la[2] * __ldg(acc + 2 * n3 + idx);
+      const float4 f = A4 ? __ldg(acc4 + idx)
+                          : make_float4(__ldg(acc + idx), __ldg(acc + n3 + idx), __ldg(acc + 2 * n3 + idx), 0.f);
+      const float dot = la[0] * f.x + la[1] * f.y + la[2] * f.z;
       g0 += dot * c.dw[dx][0] * c.w[dy][1] * c.w[dz][2];
       g1 += dot * c.w[dx][0] * c.dw[dy][1] * c.w[dz][2];
       g2 += dot * c.w[dx][0] * c.w[dy][1] * c.dw[dz][2];
@@ -121,13 +125,12 @@ cudaError_t launch_adj_deposit(const float* x, int64_t n, float m, int nf, const
   return cudaGetLastError();
 }
 
-cudaError_t launch_adj_interp(const float* x, int64_t n, int nf, const float* acc, float ck, float cd, float* lam_x,
+cudaError_t launch_adj_interp(const float* x, int64_t n, int nf, const float* acc, const float4* acc4, float ck, float cd, float* lam_x,
                               float* lam_v, float* lam_A, bool interleaved, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
-  if (interleaved)
-    k_adj_interp<true><<<grid_of(n), 256, 0, st>>>(x, n, nf, acc, ck, cd, lam_x, lam_v, lam_A);
-  else
-    k_adj_interp<false><<<grid_of(n), 256, 0, st>>>(x, n, nf, acc, ck, cd, lam_x, lam_v, lam_A);
+  const auto k = interleaved ? (acc4 ? k_adj_interp<true, true> : k_adj_interp<true, false>)
+                             : (acc4 ? k_adj_interp<false, true> : k_adj_interp<false, false>);
+  k<<<grid_of(n), 256, 0, st>>>(x, n, nf, acc, acc4, ck, cd, lam_x, lam_v, lam_A);
   note_launches(1);
   return cudaGetLastError();
 }

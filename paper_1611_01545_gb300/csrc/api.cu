@@ -53,6 +53,10 @@ struct pm_handle {
   uint32_t* tkey = nullptr;
   uint4* tpv = nullptr;      // per particle: new in-cell position code, v'_x, v'_y, v'_z (float bits)
   std::vector<void*> allocs;
+  // stream-ordered pool of the interleaved force meshes: a buffer belongs to one
+  // call on one stream, so calls on several streams or threads get their own;
+  // memory stays with the handle between calls and goes with it
+  cudaMemPool_t pool = nullptr;
   Timer timer;
   // adjoint workspace (single mesh): lam_acc float4 [n^3], component spectra [3][N][N][N/2+1]
   float* lam_acc = nullptr;
@@ -330,6 +334,28 @@ PCodesOut oview(const pm_codes_t& c, bool vel16) {
   return PCodesOut{reinterpret_cast<uint32_t*>(c.pos), c.vel, c.vmax, vel16};
 }
 
+// Interleaved copy of the acceleration mesh for a gather of n particles, or null
+// where it does not pay (fewer particles than half the nodes), would take more
+// than 512 MB, or cannot be had.  release_mesh4 gives it back, in stream order.
+const float4* interleaved_mesh(pm_handle* h, const float* acc, int64_t n, cudaStream_t st) {
+  const int64_t nodes = h->gm.nfine3();
+  if (!h->pool || 2 * n < nodes || nodes * 16 > ((int64_t)512 << 20)) return nullptr;
+  void* p = nullptr;
+  if (cudaMallocFromPoolAsync(&p, (size_t)nodes * 16, h->pool, st) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  if (launch_interleave(acc, nodes, static_cast<float4*>(p), st) != cudaSuccess) {
+    cudaGetLastError();
+    cudaFreeAsync(p, st);
+    return nullptr;
+  }
+  return static_cast<const float4*>(p);
+}
+cudaError_t release_mesh4(const float4* p, cudaStream_t st) {
+  return p ? cudaFreeAsync(const_cast<float4*>(p), st) : cudaSuccess;
+}
+
 int check_species(pm_handle* h, int s) {
   if (s < 0 || s > 1) return fail(h, PM_ERR_ARG, "species must be 0 or 1");
   return PM_OK;
@@ -550,6 +576,19 @@ int pm_init(const pm_config_t* cfg, pm_handle_t** out) {
     h->smem_optin = optin > 1024 ? (size_t)optin - 1024 : 0;   // room for the kernels' static shared memory
   }
   if (rc == PM_OK) {
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = h->device;
+    uint64_t keep = UINT64_MAX;
+    if (cudaMemPoolCreate(&h->pool, &props) != cudaSuccess ||
+        cudaMemPoolSetAttribute(h->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+      cudaGetLastError();   // without a pool the gathers read the mesh as it is
+      if (h->pool) cudaMemPoolDestroy(h->pool);
+      h->pool = nullptr;
+    }
+  }
+  if (rc == PM_OK) {
     const cudaError_t e = reserve_tables(h, h->blk_ikd);
     if (e != cudaSuccess) rc = fail(h, PM_ERR_CUDA, std::string("cudaMalloc: ") + cudaGetErrorString(e));
   }
@@ -584,6 +623,7 @@ int pm_destroy(pm_handle_t* h) {
   for (auto e : h->timer.pool) cudaEventDestroy(e);
   for (void* p : h->allocs) cudaFree(p);
   if (h->start) cudaFree(h->start);
+  if (h->pool) cudaMemPoolDestroy(h->pool);
   delete h;
   return PM_OK;
 }
@@ -799,14 +839,20 @@ int pm_solve_fixed(pm_handle_t* h, const int64_t* rho_coarse, const int64_t* rho
 int pm_interpolate(pm_handle_t* h, const float* x, int64_t n, const float* acc_coarse, const float* acc_fine, float* a,
                    void* stream) {
   if (!h || (n && (!x || !a)) || !acc_fine || (h->gm.two && !acc_coarse)) return fail(h, PM_ERR_ARG, "null argument");
-  CK(h, launch_interpolate(x, n, h->geo, acc_coarse, acc_fine, a, (cudaStream_t)stream));
+  cudaStream_t st = (cudaStream_t)stream;
+  const float4* acc4 = interleaved_mesh(h, acc_fine, n, st);
+  CK(h, launch_interpolate(x, n, h->geo, acc_coarse, acc_fine, acc4, a, st));
+  CK(h, release_mesh4(acc4, st));
   return PM_OK;
 }
 
 int pm_kick_drift(pm_handle_t* h, float* x, float* v, int64_t n, const float* acc_coarse, const float* acc_fine,
                   double c_kick, double c_drift, void* stream) {
   if (!h || (n && (!x || !v)) || !acc_fine || (h->gm.two && !acc_coarse)) return fail(h, PM_ERR_ARG, "null argument");
-  CK(h, launch_kick_drift(x, v, n, h->geo, acc_coarse, acc_fine, (float)c_kick, (float)c_drift, (cudaStream_t)stream));
+  cudaStream_t st = (cudaStream_t)stream;
+  const float4* acc4 = interleaved_mesh(h, acc_fine, n, st);
+  CK(h, launch_kick_drift(x, v, n, h->geo, acc_coarse, acc_fine, acc4, (float)c_kick, (float)c_drift, st));
+  CK(h, release_mesh4(acc4, st));
   return PM_OK;
 }
 
@@ -1144,8 +1190,11 @@ int pm_interpolate_adjoint(pm_handle_t* h, const float* x, int64_t n, const floa
                            double c_drift, float* lam_x, float* lam_v, float* lam_acc, void* stream) {
   if (!h || (n && (!x || !lam_x || !lam_v)) || !acc_fine || !lam_acc) return fail(h, PM_ERR_ARG, "null argument");
   if (h->gm.two) return fail(h, PM_ERR_CONFIG, "adjoints are implemented for the single periodic mesh");
-  CK(h, launch_adj_interp(x, n, h->gm.nf, acc_fine, (float)c_kick, (float)c_drift, lam_x, lam_v, lam_acc, false,
-                          (cudaStream_t)stream));
+  cudaStream_t st = (cudaStream_t)stream;
+  const float4* acc4 = interleaved_mesh(h, acc_fine, n, st);
+  CK(h, launch_adj_interp(x, n, h->gm.nf, acc_fine, acc4, (float)c_kick, (float)c_drift, lam_x, lam_v, lam_acc, false,
+                          st));
+  CK(h, release_mesh4(acc4, st));
   return PM_OK;
 }
 
@@ -1156,9 +1205,11 @@ static int step_adjoint_core(pm_handle_t* h, const pm_particles_t state[2], pm_p
   const size_t nf3 = (size_t)g.nfine3();
   // interleaved float4 accumulation mesh: one vector reduction per CIC corner
   CK(h, cudaMemsetAsync(h->lam_acc, 0, 4 * nf3 * 4, st));
+  const float4* acc4 = interleaved_mesh(h, acc, state[0].n + state[1].n, st);
   for (int s = 0; s < 2; ++s)
-    CK(h, launch_adj_interp(state[s].x, state[s].n, g.nf, acc, (float)c_kick, (float)c_drift, lam[s].x, lam[s].v,
+    CK(h, launch_adj_interp(state[s].x, state[s].n, g.nf, acc, acc4, (float)c_kick, (float)c_drift, lam[s].x, lam[s].v,
                             h->lam_acc, true, st));
+  CK(h, release_mesh4(acc4, st));
   CK(h, solve_adjoint_launch(h->plan_mesh, h->lam_acc, true, h->rho_f, h->adj_spec, st));   // rho_f holds lam_rho
   for (int s = 0; s < 2; ++s)
     CK(h, launch_adj_deposit(state[s].x, state[s].n, (float)h->cfg.mass[s], g.nf, h->rho_f, lam[s].x, st));

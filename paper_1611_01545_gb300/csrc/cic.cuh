@@ -72,9 +72,34 @@ __device__ __forceinline__ void gather(const float* __restrict__ F, int n, float
   a[2] = s2;
 }
 
-__device__ __forceinline__ void accel_at(const Geo& g, const float* acc_c, const float* acc_f, float px, float py,
-                                         float pz, float a[3]) {
-  gather(acc_f, g.nf, px, py, pz, a);
+// gather() from the interleaved form of the mesh, (x, y, z, unused) per node:
+// one 16-byte load per corner, the two x neighbours mostly in one sector.
+__device__ __forceinline__ void gather4(const float4* __restrict__ F, int n, float px, float py, float pz, float a[3]) {
+  int ix[2], iy[2], iz[2];
+  float wx[2], wy[2], wz[2];
+  cic_axis(px, n, ix[0], ix[1], wx[0], wx[1]);
+  cic_axis(py, n, iy[0], iy[1], wy[0], wy[1]);
+  cic_axis(pz, n, iz[0], iz[1], wz[0], wz[1]);
+  float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    const int dx = c & 1, dy = (c >> 1) & 1, dz = c >> 2;
+    const float w = __fmul_rn(__fmul_rn(wx[dx], wy[dy]), wz[dz]);
+    const float4 f = __ldg(F + ((int64_t)iz[dz] * n + iy[dy]) * n + ix[dx]);
+    s0 = __fmaf_rn(w, f.x, s0);
+    s1 = __fmaf_rn(w, f.y, s1);
+    s2 = __fmaf_rn(w, f.z, s2);
+  }
+  a[0] = s0;
+  a[1] = s1;
+  a[2] = s2;
+}
+
+// acc4: the interleaved fine mesh, used in place of acc_f when set.
+__device__ __forceinline__ void accel_at(const Geo& g, const float* acc_c, const float* acc_f, const float4* acc4,
+                                         float px, float py, float pz, float a[3]) {
+  if (acc4) gather4(acc4, g.nf, px, py, pz, a);
+  else gather(acc_f, g.nf, px, py, pz, a);
   if (g.two) {
     float s = 1.0f / (float)g.rc;
     float b[3];

@@ -68,10 +68,13 @@ cudaError_t launch_deposit_weights(const float* x, int64_t n, const float* w, in
                                   cudaStream_t st);
 cudaError_t launch_deposit_fixed(const float* x, int64_t n, long long M, const Geo& g, long long* rho_c,
                                  long long* rho_f, cudaStream_t st);
+// The acceleration mesh [3][n3] with its components next to each other.
+cudaError_t launch_interleave(const float* acc, int64_t n3, float4* out, cudaStream_t st);
+// acc4: acc_f interleaved, or null.
 cudaError_t launch_interpolate(const float* x, int64_t n, const Geo& g, const float* acc_c, const float* acc_f,
-                               float* a, cudaStream_t st);
+                               const float4* acc4, float* a, cudaStream_t st);
 cudaError_t launch_kick_drift(float* x, float* v, int64_t n, const Geo& g, const float* acc_c, const float* acc_f,
-                              float ck, float cd, cudaStream_t st);
+                              const float4* acc4, float ck, float cd, cudaStream_t st);
 cudaError_t launch_compress(const float* x, const float* v, int64_t n, const Geo& g, uint32_t* counts,
                             uint32_t* vmax_bits, const float* vmax_in, int64_t* off, pm_codes_t& out, bool vel16,
                             void* scan_state, int* status, cudaStream_t st);
@@ -123,7 +126,8 @@ cudaError_t launch_adj_deposit(const float* x, int64_t n, float m, int nf, const
                                cudaStream_t st);
 // lam_A is [3][n^3], or float4 [n^3] (x, y, z, unused) when interleaved (one vector
 // reduction per corner instead of three).
-cudaError_t launch_adj_interp(const float* x, int64_t n, int nf, const float* acc, float ck, float cd, float* lam_x,
+// acc4: acc interleaved, or null.
+cudaError_t launch_adj_interp(const float* x, int64_t n, int nf, const float* acc, const float4* acc4, float ck, float cd, float* lam_x,
                               float* lam_v, float* lam_A, bool interleaved, cudaStream_t st);
 
 }  // namespace pm
