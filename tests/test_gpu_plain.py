@@ -79,3 +79,52 @@ def test_decompress_chunks(n_cdm, heavy, vel_bits):
     xr, vr = codec.decompress(ref, N)
     np.testing.assert_array_equal(xd.cpu().numpy(), xr)
     np.testing.assert_array_equal(vd.cpu().numpy(), vr)
+
+
+# enough particles for the interleaved mesh (half the nodes) against chunks too small for it: the same bits,
+# on one stream and on two at once
+@pytest.mark.parametrize("n,two", [(32, False), (64, True)])
+def test_interleaved_gathers_equal_direct_ones(n, two):
+    from paper_1611_01545_gb300 import PM
+    cfg = dict(n_fine=n, coarse_ratio=1, tile=n, buffer=0, cmp_ratio=4, vel_bits=16, G=FOUR_PI_G_ONE, mass=(8.0, 0.04),
+               count=(0, 0))
+    if two:
+        cfg.update(coarse_ratio=4, tile=16, buffer=8, r_split=6.0 / 4.5, r_cut=6.0)
+    pm = PM(cfg)
+    g = torch.Generator(device="cuda").manual_seed(n)
+    count = n ** 3 // 2
+    x = torch.rand((count, 3), generator=g, device="cuda") * n
+    x[:64] = torch.tensor([n - 0.25, 0.0, n - 1.0], device="cuda")       # upper nodes wrap
+    v = torch.randn((count, 3), generator=g, device="cuda")
+    af = torch.randn((3, n, n, n), generator=g, device="cuda")
+    ac = torch.randn((3,) + (n // 4,) * 3, generator=g, device="cuda") if two else None
+    chunks = [(i, min(i + 1000, count)) for i in range(0, count, 1000)]
+    a = pm.interpolate(x, ac, af)
+    assert torch.equal(a, torch.cat([pm.interpolate(x[i:j].contiguous(), ac, af) for i, j in chunks]))
+    xk, vk = x.clone(), v.clone()
+    pm.kick_drift(xk, vk, ac, af, 0.3, 0.7)
+    small = [(x[i:j].clone(), v[i:j].clone()) for i, j in chunks]
+    for xs, vs in small:
+        pm.kick_drift(xs, vs, ac, af, 0.3, 0.7)
+    assert torch.equal(xk, torch.cat([s[0] for s in small])) and torch.equal(vk, torch.cat([s[1] for s in small]))
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    meshes = [af, -2.0 * af]
+    torch.cuda.synchronize()
+    got = [[], []]
+    for _ in range(5):
+        for k, st in enumerate(streams):
+            with torch.cuda.stream(st):
+                got[k].append(pm.interpolate(x, None if ac is None else (1.0, -2.0)[k] * ac, meshes[k]))
+    torch.cuda.synchronize()
+    for k, f in enumerate((1.0, -2.0)):
+        for r in got[k]:
+            assert torch.equal(r, f * a)
+    if not two:
+        lam = [torch.randn((count, 3), generator=g, device="cuda") for _ in range(2)]
+        lx, lv, la = lam[0].clone(), lam[1].clone(), torch.zeros_like(af)
+        pm.interpolate_adjoint(x, af, 0.3, 0.7, lx, lv, la)
+        parts = [(lam[0][i:j].clone(), lam[1][i:j].clone()) for i, j in chunks]
+        for (i, j), (px, pv) in zip(chunks, parts):
+            pm.interpolate_adjoint(x[i:j].contiguous(), af, 0.3, 0.7, px, pv, torch.zeros_like(af))
+        assert torch.equal(lx, torch.cat([p[0] for p in parts])) and torch.equal(lv, torch.cat([p[1] for p in parts]))
+    pm.check()
