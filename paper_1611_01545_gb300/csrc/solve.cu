@@ -43,11 +43,8 @@ template <int N> struct SolveCfg {
 #ifndef PM_PASSB_TMA_MINB
 #define PM_PASSB_TMA_MINB 5
 #endif
-#ifndef PM_SOLVE_C_THREADS
-#define PM_SOLVE_C_THREADS 384
-#endif
 #ifndef PM_SOLVE_C_MINB
-#define PM_SOLVE_C_MINB 3
+#define PM_SOLVE_C_MINB 4
 #endif
 };
 
@@ -226,10 +223,10 @@ __global__ void __launch_bounds__(PassB<N>::threads) k_solve_b_adj(SolveArgs a) 
     __syncthreads();
   }
   fft_inv<N, KC, 1, KC>(G, tw);
-  float2* out = a.spec3 + (size_t)ys * NP + kx0;
+  float2* out = a.spec3 + (size_t)ys * NH + kx0;   // spec3 rows have no padding
   for (int i = threadIdx.x; i < N * KC; i += blockDim.x) {
     const int z = i / KC, c = i - z * KC;
-    if (c < ncol) out[(size_t)z * N * NP + c] = G[i];
+    if (c < ncol) out[(size_t)z * N * NH + c] = G[i];
   }
 }
 
@@ -591,7 +588,7 @@ __global__ void __launch_bounds__(PassBR<N>::threads, PassBR<N>::min_blocks)
   }
   __syncthreads();
   // inverse step 2: items (component, j2, column) -> rows z = N2 j1 + j2 of the output range
-  float2* out = a.spec3 + ((size_t)pb * 3 * a.t * N + ys) * NP + kx0;
+  float2* out = a.spec3 + ((size_t)pb * 3 * a.t * N + ys) * NH + kx0;
   for (int w = threadIdx.x; w < 3 * KT * N2; w += T) {
     const int d = w / (KT * N2), r = w - d * KT * N2;
     const int j2 = r / KT, c = r - j2 * KT;
@@ -602,11 +599,11 @@ __global__ void __launch_bounds__(PassBR<N>::threads, PassBR<N>::min_blocks)
     Dft<N1, 1>::run(v);
     if (c < ncol) {
       const int z0 = j2 - a.b;
-      float2* o = out + (ptrdiff_t)(d * a.t + z0) * N * NP + c;
+      float2* o = out + (ptrdiff_t)(d * a.t + z0) * N * NH + c;
 #pragma unroll
       for (int j1 = 0; j1 < N1; ++j1) {
         const int zo = z0 + N2 * j1;
-        if ((unsigned)zo < (unsigned)a.t) o[(size_t)N2 * j1 * N * NP] = v[j1];
+        if ((unsigned)zo < (unsigned)a.t) o[(size_t)N2 * j1 * N * NH] = v[j1];
       }
     }
   }
@@ -620,21 +617,23 @@ __global__ void __launch_bounds__(PassBR<N>::threads, PassBR<N>::min_blocks)
 // earlier form moved 5,280 128-byte wavefronts per 96^3 tile plane, 1,650 of
 // them bank conflicts, at 75% of the load/store pipe, and took 0.288 ms for 64
 // tiles (0.226 without the prolongation).  Here
-//   * an item of the second y step transforms two neighbouring rows at once
-//     and writes only the output rows, both rows of a packed pair in one
-//     16-byte word [pair][kx];
-//   * the x steps give a warp's lanes different pairs (pitches NH 16-byte words
-//     and N + 1 complex values, both odd, so 8 or 16 lanes fall in different
-//     banks) where lanes along a row met 2 to 4 deep in a bank;
+//   * an item of the second y step transforms two neighbouring rows at once;
+//   * the x steps give a warp's lanes different row pairs (odd pitches: the x
+//     step's reads of the pairs are 2 deep in a bank where rows are kept in
+//     place, all else conflict free) where lanes along a row met 2 to 4 deep;
 //   * the output takes a pair's two rows from one 8-byte word and the four rows
 //     between two coarse rows from one x interpolation each of the coarse force
-//     (fetched while the plane is on its way).
-// 2,600 wavefronts per plane, 0.291 -> 0.221 ms for 64 tiles; 216 tiles of 48^3:
-// 0.182 -> 0.103 ms.  It is bound by issue now (73% of the slots); 416 threads
-// (one round of the 392 column items) take 0.250 ms, 2 blocks per SM 0.309.
-// N = 128 keeps the y rows in place and the x step in registers across a
-// barrier (one buffer of 67 KB instead of two), so that 2 blocks share an SM:
-// 128^3 mesh 33 -> 21 us.
+//     (fetched while the plane is on its way);
+//   * for N >= 96 the rows stay in place and the x step holds its items in
+//     registers across a barrier: one buffer (38 KB at 96, 67 KB at 128) instead
+//     of two, so 4 blocks of 256 threads share an SM (2 of 544 at 128); smaller
+//     sizes write the output rows to a second buffer, both rows of a pair in one
+//     16-byte word.
+// 64 tiles of 96^3 0.291 -> 0.197 ms (two buffers, 3 blocks of 384: 0.221; 5
+// blocks of 256 with 48 registers: 0.199), 216 tiles of 48^3 0.182 -> 0.103 ms,
+// 128^3 mesh 33 -> 21 us.  Bound by issue now (75% of the slots).  The spectrum
+// rows between passes B and C are not padded: pass B's stores take 0.182 ms with
+// them in place of 0.195.
 
 // w / n for 0 <= w < 4096, n >= 1, with inv = 1 / n (w + 1/2 keeps the product
 // away from whole numbers by more than its rounding).
@@ -642,11 +641,12 @@ __device__ __forceinline__ int quick_div(int w, float inv) { return (int)(((floa
 
 template <int N> struct PassC {
   static constexpr int N1 = Factor<N>::N1, N2 = Factor<N>::N2;
-  static constexpr int NH = N / 2 + 1, NP = spec_pitch(N);
-  static constexpr bool in_place = N >= 128;
-  // one round of the largest item sets; the last warp of 96, 64 and 128 takes the column at kx = N / 2
-  static constexpr int threads = N == 128 ? 544 : (N == 96 ? PM_SOLVE_C_THREADS : (N == 64 ? 288 : (N == 48 ? 160 : 96)));
-  static constexpr int min_blocks = N == 128 ? 2 : (N == 96 ? PM_SOLVE_C_MINB : 4);
+  static constexpr int NH = N / 2 + 1, NP = N / 2 + 1;   // spec3 rows have no padding
+  static constexpr bool in_place = N >= 96;
+  // in place the x step's items are one round: 256 threads serve 32 row pairs of
+  // 96 (the buffered tiles), 384 all 48; else one round of the largest item set
+  static constexpr int threads = N == 128 ? 544 : (N == 96 ? 384 : (N == 64 ? 288 : (N == 48 ? 160 : 96)));
+  static constexpr int min_blocks(int t) { return N == 128 ? 2 : (N == 96 ? (t == 256 ? PM_SOLVE_C_MINB : 3) : 4); }
   static constexpr size_t align = 128;
   // P [N][NP] (then W [pairs][N + 1]), twiddles, Y [pairs][NH] 16-byte words or, in place, room for the prolongation
   static size_t smem(int t, int b, int prc, bool prolong) {
@@ -655,14 +655,15 @@ template <int N> struct PassC {
     return align + sizeof(float2) * ((size_t)N * NP + N) + (in_place ? 4 * nq * nq : 16 * pairs * NH);
   }
   static size_t smem_max() { return align + sizeof(float2) * ((size_t)N * NP + N) + (size_t)16 * (N / 2) * NH; }
+  static bool narrow(int t, int b) { return N == 96 && pair_count(t, b) * N1 <= 256; }
   // row pairs (2 m, 2 m + 1) that hold the output rows b .. b + t - 1
   static __host__ __device__ __forceinline__ int pair_count(int t, int b) { return ((b + t - 1) >> 1) - (b >> 1) + 1; }
 };
 
-template <int N>
-__global__ void __launch_bounds__(PassC<N>::threads, PassC<N>::min_blocks) k_solve_c(SolveArgs a) {
+template <int N, int T = PassC<N>::threads>
+__global__ void __launch_bounds__(T, PassC<N>::min_blocks(T)) k_solve_c(SolveArgs a) {
   using C = PassC<N>;
-  constexpr int N1 = C::N1, N2 = C::N2, NH = C::NH, NP = C::NP, WP = N + 1, T = C::threads;
+  constexpr int N1 = C::N1, N2 = C::N2, NH = C::NH, NP = C::NP, WP = N + 1;
   extern __shared__ unsigned char smraw_c[];
   __shared__ uint64_t bar;
   float2* P = reinterpret_cast<float2*>(tma_align(smraw_c));   // [y][NP]
@@ -749,8 +750,7 @@ __global__ void __launch_bounds__(PassC<N>::threads, PassC<N>::min_blocks) k_sol
   // their half spectra, extended by conjugate symmetry).  Step 1: items (k1,
   // pair), frequencies k = k1 + N1 k2.
   {
-    static_assert(!C::in_place || (N / 2) * N1 <= T, "in place: one round");
-    for (int w0 = 0; w0 < np * N1; w0 += T) {
+    for (int w0 = 0; w0 < np * N1; w0 += T) {   // (in place: one round)
       const int w = w0 + threadIdx.x;
       const bool live = w < np * N1;
       const int k1 = live ? quick_div(w, inv_np) : 0, j = live ? w - k1 * np : 0;
@@ -1144,6 +1144,7 @@ static cudaError_t solve_n(const SolvePlan& p, const void* src, bool fixed, floa
     cudaFuncSetAttribute(k_solve_c<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassC<N>::smem_max());
     if constexpr (N == 96) {
       cudaFuncSetAttribute(k_solve_a<N, SRC_BOXES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassA<N>::smem);
+      cudaFuncSetAttribute(k_solve_c<N, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassC<N>::smem_max());
     }
     attr_done = true;
   }
@@ -1184,7 +1185,13 @@ static cudaError_t solve_n(const SolvePlan& p, const void* src, bool fixed, floa
     }
     {
       TimedScope ts(tm, N == p.src_n && p.b == 0 ? "fft_c_mesh" : "fft_c_tiles", st);
-      k_solve_c<N><<<dim3(p.t, 3, nb), PassC<N>::threads, PassC<N>::smem(p.t, p.b, a.prc, a.pc != nullptr), st>>>(a);
+      const size_t smem = PassC<N>::smem(p.t, p.b, a.prc, a.pc != nullptr);
+      if constexpr (N == 96) {
+        if (PassC<N>::narrow(p.t, p.b)) k_solve_c<N, 256><<<dim3(p.t, 3, nb), 256, smem, st>>>(a);
+        else k_solve_c<N><<<dim3(p.t, 3, nb), PassC<N>::threads, smem, st>>>(a);
+      } else {
+        k_solve_c<N><<<dim3(p.t, 3, nb), PassC<N>::threads, smem, st>>>(a);
+      }
     }
     note_launches(3);
     cudaError_t e = cudaGetLastError();
