@@ -385,12 +385,14 @@ __global__ void PM_DEPOSIT_BOUNDS k_deposit_codes(PCodes c0, PCodes c1, const in
 //     from the same four values and the left neighbour's carry.
 // 256^3 workload 0.178 -> 0.118 ms (blocks of 32 x 2 x 1; with its launch 0.192 ->
 // 0.130, 64 x 1 x 1 0.125, 32 x 2 x 2 0.177: 5 instead of 6 CTAs per SM and spills),
-// 768^3 (5.1e8 particles) 4.56 -> 2.98 ms, clustered 512^3 in its default shape
+// 768^3 (5.1e8 particles) 4.56 -> 2.98 ms (3.07 with planes 4 banks apart), clustered 512^3 in its default shape
 // 1.71 -> 0.89 ms.
 template <int RX_MAX, int RY, int RZ> struct DepShape {
   static constexpr int row = 4 * RX_MAX + 4;          // words per bin row (4 RX + 1 used), whole 16-byte words
   static constexpr int fy = 4 * RY + 1, fz = 4 * RZ + 1, rows = fy * fz;
-  static constexpr int plane = row * fy;
+  // planes start 16 banks apart modulo 32, rows 4: the 4^3 lower nodes of a cell's particles, which the
+  // lanes of a warp add to, lie at most 2 deep in a bank
+  static constexpr int plane = row * fy + ((16 - row * fy) & 31);
   static constexpr int cx = RX_MAX + 1, cy = RY + 1, cz = RZ + 1;
   static constexpr int lists = RY * RZ;                // cell rows
   // bins, x-restricted rows, xy-restricted rows, relative offsets of both species
