@@ -450,7 +450,8 @@ int pm_set_graphs(pm_handle_t* h, int on);
  *                      counter until none are left (uneven, clustered blocks
  *                      then balance across the SMs);
  *  kick_block[3]       compression cells per CTA of the interpolate + kick +
- *                      drift + recompress passes;
+ *                      drift + recompress passes (single rows of more than 32
+ *                      cells may be dealt out in halves);
  *  kick_window         half-width in cells of the new-cell window whose
  *                      counts a CTA keeps in shared memory (1..4; particles
  *                      moving further use global counters); the library uses

@@ -267,7 +267,7 @@ Blk choose_blk(const Geom& g, bool fixed, bool deposit) {
   Blk b{};
   b.RX = g.ncmp;
   b.RY = b.RZ = 1;
-  b.D = 2;
+  b.D = 1;   // (2 at 256^3: count 0.317 instead of 0.307 ms, scatter 0.257 instead of 0.241)
   Geo geo{g.nf, g.rc, g.nc, g.rcmp, g.ncmp, g.ncell(), g.two};
   if (!deposit) {
     while (b.RX > 1 && b.RX % 2 == 0 && kick_count_smem(geo, b) > 100 * 1024) b.RX /= 2;
@@ -300,6 +300,7 @@ size_t table_budget(const pm_handle* h) {
 // Makes room for the start tables of kick block b.
 cudaError_t reserve_tables(pm_handle* h, Blk b) {
   if (h->scratch_n == 0) return cudaSuccess;   // no particles, no tables
+  b = kick_blocks(h->geo, b, h->scratch_n);
   b.D = table_window(h->geo, b, table_budget(h));
   const size_t need = table_bytes(h->geo, b);
   if (need <= h->start_bytes) return cudaSuccess;
@@ -318,7 +319,7 @@ RecompressTables tables(const pm_handle* h) {
   return RecompressTables{h->counts[0], h->counts[1], h->far[0], h->far[1], h->start, 0};
 }
 Blk ikd_blk(const pm_handle* h, int pass) {
-  Blk b = h->blk_ikd;
+  Blk b = kick_blocks(h->geo, h->blk_ikd, h->scratch_n);
   b.D = table_window(h->geo, b, table_budget(h));
   b.work = h->persist_ikd ? h->work + 1 + pass : nullptr;
   b.brick = block_brick(b);

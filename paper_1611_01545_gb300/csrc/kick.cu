@@ -366,8 +366,9 @@ __device__ __forceinline__ void stage_coarse(const float* acc, const Geo& g, con
 
 // Threads per CTA of the count pass and of the scatter, and the resident CTAs
 // per SM they are compiled for (sets their register budget).
-constexpr int kKickThreads = 512, kKickMinBlocks = 2;
-constexpr int kScatterThreads = 256, kScatterMinBlocks = 5;
+constexpr int kKickThreads = 512, kKickMinBlocks = 2;   // any shape
+// (scatter at 768^3: 4 CTAs per SM 8.02 ms, 5 8.25, 6 8.92, 8 with one particle per thread at a time 8.56)
+constexpr int kScatterThreads = 256, kScatterMinBlocks = 4;
 
 // Count pass, any block shape.
 template <bool V16>
@@ -470,17 +471,25 @@ __global__ void __launch_bounds__(kKickThreads, kKickMinBlocks) k_kick_count(Kic
 // 64-bit shifts, and the next particle's codes are loaded while this one is
 // worked on.  256^3 workload, 8-bit codes: 0.380 ms before, 0.311 now (with the
 // ranks); 768^3, 5.1e8 particles: 9.93 -> 8.31 ms.
-// STAGED: the block's force region is copied to shared memory (80 KB, 2 CTAs
-// per SM).  That costs 300 values per cell, 24 are needed per particle: below
+// CELLS: the longest row, 64, or 32 where a dense set's rows are dealt out in
+// pieces (kick_blocks): with 5 CTAs of 256 threads per SM the staging, the
+// particles and the flush of different blocks overlap better than with 2 of 512
+// over 64 cells (0.307 -> 0.296 ms; 768^3 8.13 -> 7.71; 64 cells with 640 threads
+// 8.37, 32 cells with 320 threads and 4 CTAs 8.23, 16 cells with 128 and 10 CTAs
+// 8.60).  Windows of half-width 2 and sparse sets keep 64 cells: their blocks do
+// more per window cell than per particle (clustered 512^3 with half-width 2:
+// scatter 1.46 ms with 64 cells, 1.72 with 32).
+// STAGED: the block's force region is copied to shared memory (41 or 80 KB).  That costs 300 values per cell, 24 are needed per particle: below
 // kStageFrom particles per cell the forces are gathered from the mesh directly
 // (192^3 mesh with 2.8 particles per cell: 0.114 ms staged, 0.042 direct).
-constexpr int kRowCells = 64;
 constexpr int kStageFrom = 12;
 constexpr int kDirectThreads = 128, kDirectMinBlocks = 8;
-constexpr int kRowStride = 4 * kRowCells + 4;                      // 260: 4 banks modulo 32
-constexpr int kPlaneStride = 5 * kRowStride + 28;                  // 1328: 16 banks modulo 32
-constexpr int kCompStride = 5 * kPlaneStride;
-static_assert(kRowStride % 32 == 4 && kPlaneStride % 32 == 16 && kCompStride % 4 == 0, "bank layout, 16-byte rows");
+template <int CELLS> struct RowRegion {
+  static constexpr int row = 4 * CELLS + 4;                     // 4 banks modulo 32, whole 16-byte words
+  static constexpr int plane = 5 * row + 28;                    // 16 banks modulo 32
+  static constexpr int comp = 5 * plane;
+  static_assert(row % 32 == 4 && plane % 32 == 16 && comp % 4 == 0, "bank layout, 16-byte rows");
+};
 
 __device__ __forceinline__ void copy_async16(float* smem_dst, const float* gmem_src) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
@@ -488,6 +497,7 @@ __device__ __forceinline__ void copy_async16(float* smem_dst, const float* gmem_
 }
 
 // The force at lower node (base) and upper weights w1; same weights and order as gather().
+template <class R>
 __device__ __forceinline__ void gather_row_region(const float* base, const float w1[3], float a[3]) {
   const float w0[3] = {__fsub_rn(1.0f, w1[0]), __fsub_rn(1.0f, w1[1]), __fsub_rn(1.0f, w1[2])};
   float s0 = 0.f, s1 = 0.f, s2 = 0.f;
@@ -495,32 +505,38 @@ __device__ __forceinline__ void gather_row_region(const float* base, const float
   for (int c = 0; c < 8; ++c) {
     const int dx = c & 1, dy = (c >> 1) & 1, dz = c >> 2;
     const float w = __fmul_rn(__fmul_rn(dx ? w1[0] : w0[0], dy ? w1[1] : w0[1]), dz ? w1[2] : w0[2]);
-    const float* q = base + dz * kPlaneStride + dy * kRowStride + dx;
+    const float* q = base + dz * R::plane + dy * R::row + dx;
     s0 = __fmaf_rn(w, q[0], s0);
-    s1 = __fmaf_rn(w, q[kCompStride], s1);
-    s2 = __fmaf_rn(w, q[2 * kCompStride], s2);
+    s1 = __fmaf_rn(w, q[R::comp], s1);
+    s2 = __fmaf_rn(w, q[2 * R::comp], s2);
   }
   a[0] = s0;
   a[1] = s1;
   a[2] = s2;
 }
 
-template <bool V16, bool STAGED>
-__global__ void __launch_bounds__(STAGED ? kKickThreads : kDirectThreads, STAGED ? kKickMinBlocks : kDirectMinBlocks)
+template <bool STAGED, int CELLS> struct RowForm {
+  static constexpr int threads = !STAGED ? kDirectThreads : (CELLS == 32 ? 256 : kKickThreads);
+  static constexpr int min_blocks = !STAGED ? kDirectMinBlocks : (CELLS == 32 ? 5 : kKickMinBlocks);
+};
+template <bool V16, bool STAGED, int CELLS>
+__global__ void __launch_bounds__(RowForm<STAGED, CELLS>::threads, RowForm<STAGED, CELLS>::min_blocks)
     k_kick_count_row(KickArgs k) {
+  using R = RowRegion<CELLS>;
+  constexpr int kRowCells = CELLS;
   extern __shared__ __align__(16) unsigned char smraw[];
   const Geo& g = k.g;
   const Blk& bk = k.bk;
   const bool two_c = g.two && k.coarse != 0;
   constexpr uint32_t kSeg = 1u << 30;   // particles of a row handled with one set of 32-bit offsets
-  constexpr int kThreads = STAGED ? kKickThreads : kDirectThreads;
+  constexpr int kThreads = RowForm<STAGED, CELLS>::threads;
   for_each_block(bk, [&](const int bid) {
     const int RX = bk.RX;
     const CellBlock cb = block_of(bk, bid);
     const Win win = window_of(g, bk, cb);
     const int W = win.wx * win.wy * win.wz;
     float* sf = reinterpret_cast<float*>(smraw);                               // staged region, then the coarse one
-    float* sc = sf + (STAGED ? 3 * kCompStride : 0);
+    float* sc = sf + (STAGED ? 3 * R::comp : 0);
     uint32_t* rel = reinterpret_cast<uint32_t*>(sc + (two_c ? 12 * (kRowCells + 1) : 0));   // [2][kRowCells]
     uint32_t* hist = rel + 2 * kRowCells;
     const int64_t c0 = cb.ix0 + (int64_t)g.ncmp * (cb.iy0 + (int64_t)g.ncmp * cb.iz0);
@@ -543,7 +559,7 @@ __global__ void __launch_bounds__(STAGED ? kKickThreads : kDirectThreads, STAGED
         if (gz >= nf) gz -= nf;
         if (gy >= nf) gy -= nf;
         const float* src = k.acc_f + comp * nf3 + ((int64_t)gz * nf + gy) * nf;
-        float* dst = sf + comp * kCompStride + lz * kPlaneStride + ly * kRowStride;
+        float* dst = sf + comp * R::comp + lz * R::plane + ly * R::row;
         for (int j = threadIdx.x & 31; j <= RX; j += 32) {
           if (j < RX) copy_async16(dst + 4 * j, src + bxf + 4 * j);
           else copy_async4(dst + 4 * j, src + (bxf + 4 * j == nf ? 0 : bxf + 4 * j));
@@ -625,7 +641,7 @@ __global__ void __launch_bounds__(STAGED ? kKickThreads : kDirectThreads, STAGED
 #pragma unroll
           for (int d = 0; d < 3; ++d) v[d] = __fmul_rn(__fsub_rn(__uint2float_rn(u[d]), vmid), step);
           if (STAGED) {
-            gather_row_region(sf + nz * kPlaneStride + ny * kRowStride + nx, w1, a);
+            gather_row_region<R>(sf + nz * R::plane + ny * R::row + nx, w1, a);
             if (two_c && live) {
               // coarse cell == compression cell: corner (ixl, 0, 0), weight (2q + 1) / 512
               float b3[3], u1[3];
@@ -814,6 +830,17 @@ int window_cells(const Geo& g, const Blk& bk) {
 }
 
 
+// The blocks that the passes take for an asked shape: single rows of more than
+// kKickRowCells cells are cut in halves for dense sets and windows of half-width 1.
+Blk kick_blocks(const Geo& g, Blk bk, int64_t particles) {
+  if (g.rcmp == 4 && bk.RY == 1 && bk.RZ == 1 && bk.D == 1 && particles >= (int64_t)kStageFrom * g.ncell)
+    while (bk.RX > kKickRowCells && bk.RX % 2 == 0) {
+      bk.RX /= 2;
+      bk.nbx *= 2;
+    }
+  return bk;
+}
+
 // Window half-width used for a block shape: the asked one, narrowed until the
 // start tables (8 bytes per block and window cell) take at most `budget` bytes
 // or the half-width is 1.  Narrower windows only make more movers far ones.
@@ -835,16 +862,20 @@ static int rank_bits(const Geo& g, const Blk& bk) {
 template <bool V16>
 static cudaError_t kick_count(const KickArgs& k, int64_t particles, cudaStream_t st) {
   const Blk& bk = k.bk;
-  const bool row = bk.RY == 1 && bk.RZ == 1 && bk.RX <= kRowCells && k.g.rcmp == 4;
+  const bool row = bk.RY == 1 && bk.RZ == 1 && bk.RX <= 64 && k.g.rcmp == 4;
+  const bool halves = row && bk.RX <= kKickRowCells && bk.D == 1;
   const bool staged = particles >= (int64_t)kStageFrom * k.g.ncell;
   size_t smem;
   int threads = kKickThreads;
   void (*f)(KickArgs);
   if (row) {
-    f = staged ? k_kick_count_row<V16, true> : k_kick_count_row<V16, false>;
-    if (!staged) threads = kDirectThreads;
-    smem = 4 * ((staged ? 3 * (size_t)kCompStride : 0) + (k.g.two && k.coarse ? 12 * (kRowCells + 1) : 0) +
-                2 * kRowCells + 2 * (size_t)window_cells(k.g, bk));
+    const int cells = staged && halves ? 32 : 64;
+    if (!staged) f = k_kick_count_row<V16, false, 64>;
+    else if (halves) f = k_kick_count_row<V16, true, 32>;
+    else f = k_kick_count_row<V16, true, 64>;
+    threads = !staged ? kDirectThreads : (halves ? RowForm<true, 32>::threads : kKickThreads);
+    smem = 4 * ((staged ? 3 * (size_t)(halves ? RowRegion<32>::comp : RowRegion<64>::comp) : 0) +
+                (k.g.two && k.coarse ? 12 * (cells + 1) : 0) + 2 * cells + 2 * (size_t)window_cells(k.g, bk));
   } else {
     f = k_kick_count<V16>;
     smem = kick_count_smem(k.g, bk);

@@ -94,6 +94,8 @@ struct RecompressTables {
   int kb;            // rank bits of a key (set by the launchers)
 };
 size_t table_bytes(const Geo& g, const Blk& bk);
+constexpr int kKickRowCells = 32;
+Blk kick_blocks(const Geo& g, Blk bk, int64_t particles);
 int table_window(const Geo& g, Blk bk, size_t budget);
 // Brick edge (block rows) of the block order for a block grid (1: row order).
 int block_brick(const Blk& bk);
