@@ -696,7 +696,7 @@ int pm_deposit_codes(pm_handle_t* h, const pm_codes_t in[2], void* rho_coarse, v
   cudaStream_t st = (cudaStream_t)stream;
   const bool fixed = h->cfg.deposit_mode == 1;
   const bool vel16 = h->cfg.vel_bits == 16;
-  const ScanClear clear{{nullptr, nullptr}, {nullptr, nullptr}, h->vmax_bits, kSmallWords};
+  const ScanClear clear{{nullptr, nullptr}, {nullptr, nullptr}, h->vmax_bits, kSmallWords, nullptr, 0};
   CK(h, scan_codes2(in, h->gm.ncell(), h->off[0], h->off[1], h->scan_state, h->status, &clear, st));
   long long M0 = llrint(h->cfg.mass[0] * 4294967296.0), M1 = llrint(h->cfg.mass[1] * 4294967296.0);
   CK(h, launch_deposit_codes(view(in[0], vel16), view(in[1], vel16), h->off[0], h->off[1], h->geo, dep_blk(h),
@@ -1114,7 +1114,10 @@ int step_launch(pm_handle_t* h, const pm_codes_t in[2], pm_codes_t out[2], doubl
   const int64_t ncell = g.ncell();
   {
     TimedScope ts(tm, "scan_in", st);
-    const ScanClear clear{{h->counts[0], h->counts[1]}, {h->far[0], h->far[1]}, h->vmax_bits, kSmallWords};
+    // clears the meshes (the coarse one follows the fine one) and the step's counters on the way
+    const ScanClear clear{{h->counts[0], h->counts[1]}, {h->far[0], h->far[1]}, h->vmax_bits, kSmallWords,
+                          fixed ? (void*)h->rho_f_fix : (void*)h->rho_f,
+                          (g.nfine3() + g.ncoarse3()) * (fixed ? 8 : 4) / 16};
     CK(h, scan_codes2(in, ncell, h->off[0], h->off[1], h->scan_state, h->status, &clear, st));
   }
   void* rc = fixed ? (void*)h->rho_c_fix : (void*)h->rho_c;
@@ -1127,7 +1130,6 @@ int step_launch(pm_handle_t* h, const pm_codes_t in[2], pm_codes_t out[2], doubl
   const bool via_fine = g.two && !fixed;
   {
     TimedScope ts(tm, "deposit", st);
-    CK(h, cudaMemsetAsync(rf, 0, (size_t)(g.nfine3() + g.ncoarse3()) * (fixed ? 8 : 4), st));   // and rc after it
     long long M0 = llrint(h->cfg.mass[0] * 4294967296.0), M1 = llrint(h->cfg.mass[1] * 4294967296.0);
     // (float: the coarse density is restricted from each block's fine tile as it flushes)
     CK(h, launch_deposit_codes(view(in[0], vel16), view(in[1], vel16), h->off[0], h->off[1], h->geo, dep_blk(h),

@@ -609,9 +609,9 @@ __global__ void __launch_bounds__(RowForm<STAGED, CELLS>::threads, RowForm<STAGE
           const uint32_t cpw = pw;
           const uint2 cvw = vw;
           if (i + kThreads < m) {
-            pw = pos[i + kThreads];
-            if (V16) vw = vel_w[i + kThreads];
-            else vw.x = vel_b[i + kThreads];
+            pw = __ldcs(pos + i + kThreads);   // read once
+            if (V16) vw = __ldcs(vel_w + i + kThreads);
+            else vw.x = __ldcs(vel_b + i + kThreads);
           }
           // the last cell whose offset is at most i (entries past the row hold 2^30)
           int ixl = 0;
@@ -880,7 +880,7 @@ static cudaError_t kick_count(const KickArgs& k, int64_t particles, cudaStream_t
     f = k_kick_count<V16>;
     smem = kick_count_smem(k.g, bk);
   }
-  cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_smem(f, smem);
   f<<<block_grid(f, bk, threads, smem), threads, smem, st>>>(k);
   note_launches(1);
   return cudaGetLastError();
@@ -903,7 +903,7 @@ cudaError_t launch_kick_scatter(int64_t n0, int64_t n1, const int64_t* off0, con
   k.t.kb = rank_bits(g, bk);
   const size_t smem = 2 * (size_t)window_cells(g, bk) * sizeof(int64_t);
   const auto f = o0.vel16 ? k_kick_scatter<true> : k_kick_scatter<false>;
-  cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_smem(f, smem);
   f<<<block_grid(f, bk, kScatterThreads, smem), kScatterThreads, smem, st>>>(k);
   note_launches(1);
   return cudaGetLastError();

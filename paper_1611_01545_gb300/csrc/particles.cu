@@ -577,7 +577,7 @@ static void launch_rows(const PCodes& c0, const PCodes& c1, const int64_t* off0,
                         const Blk& bk, float m0, float m1, float* rho_c, float* rho_f, cudaStream_t st) {
   const auto k = k_deposit_rows<RX_MAX, RY, RZ>;
   constexpr size_t smem = DepShape<RX_MAX, RY, RZ>::smem;
-  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_smem(k, smem);
   k<<<block_grid(k, bk, PM_DEPOSIT_THREADS, smem), PM_DEPOSIT_THREADS, smem, st>>>(c0, c1, off0, off1, g, bk, m0, m1,
                                                                                    g.two ? rho_c : nullptr, rho_f);
 }
@@ -629,12 +629,12 @@ cudaError_t launch_deposit_codes(const PCodes& c0, const PCodes& c1, const int64
     launch_rows<32, 2, 1>(c0, c1, off0, off1, g, bk, m0, m1, rc, rf, st);
   } else if (fixed) {
     const auto k = k_deposit_codes<long long>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(k, smem);
     k<<<block_grid(k, bk, PM_DEPOSIT_THREADS, smem), PM_DEPOSIT_THREADS, smem, st>>>(
         c0, c1, off0, off1, g, bk, m0, m1, M0, M1, static_cast<long long*>(rho_c), static_cast<long long*>(rho_f));
   } else {
     const auto k = k_deposit_codes<float>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(k, smem);
     k<<<block_grid(k, bk, PM_DEPOSIT_THREADS, smem), PM_DEPOSIT_THREADS, smem, st>>>(c0, c1, off0, off1, g, bk, m0, m1,
                                                                                      M0, M1, rc, rf);
   }

@@ -48,6 +48,8 @@ struct ScanClear {
   uint32_t* far[2];
   uint32_t* small;
   int small_words;
+  void* mesh;            // 16-byte aligned
+  int64_t mesh_words;    // 16-byte words
 };
 cudaError_t scan_codes(const pm_codes_t& in, int64_t ncell, int64_t* off, void* state, int* status, cudaStream_t st);
 // vmax_bits (float bits): copied to out.vmax when set.

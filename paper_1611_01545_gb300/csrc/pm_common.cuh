@@ -53,6 +53,13 @@ struct SolvePlan {
   float2* spec3 = nullptr; // device [batch][3][t][N][NP]
 };
 
+// Lets a kernel use smem bytes of dynamic shared memory: up to 48 KB need no
+// call, which the launch-bound small meshes notice.
+template <class K>
+inline void allow_smem(K kernel, size_t smem) {
+  if (smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
+
 // Counts kernel launches made by the library (all handles); read by pm_launch_count.
 void note_launches(int k);
 

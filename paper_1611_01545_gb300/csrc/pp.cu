@@ -231,7 +231,7 @@ cudaError_t launch_pp(const PCodes& c0, const PCodes& c1, const int64_t* off0, c
   if (g.ncmp % rx) return cudaErrorInvalidValue;
   PPArgs a{c0, c1, off0, off1, g, m0, m1, G, r_soft * r_soft, acc, amax, rx};
   const size_t smem = pp_smem(g);
-  cudaFuncSetAttribute(k_pp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_smem(k_pp, smem);
   const long long nblk = (long long)g.ncmp * g.ncmp * (g.ncmp / rx);
   k_pp<<<(unsigned)nblk, PP_THREADS, smem, st>>>(a);
   note_launches(1);

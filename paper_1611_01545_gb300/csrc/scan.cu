@@ -288,6 +288,8 @@ struct FinishArgs {
   float* vmax_out;
   uint32_t* clear;
   int words;
+  uint4* mesh;           // and a mesh of mesh_words 16-byte words, a slice per tile and species
+  int64_t mesh_words;
 };
 
 template <class T> struct Pair { T v[2]; };
@@ -328,6 +330,13 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan(Pair<Get> gets, Pair<Put>
     if (threadIdx.x == 0 && f.vmax_out) *f.vmax_out = __uint_as_float(*f.vmax_bits);
     for (int i = threadIdx.x; i < f.words; i += SCAN_THREADS) f.clear[i] = 0u;
   }
+  if (f.mesh) {
+    const int64_t slices = (int64_t)tiles * gridDim.y;
+    const int64_t per = (f.mesh_words + slices - 1) / slices;
+    const int64_t from = ((int64_t)blockIdx.y * tiles + tile) * per;
+    const int64_t to = from + per < f.mesh_words ? from + per : f.mesh_words;
+    for (int64_t i = from + threadIdx.x; i < to; i += SCAN_THREADS) f.mesh[i] = make_uint4(0, 0, 0, 0);
+  }
   __syncthreads();
   const V2 prefix = s_prefix;
   ex = v2add(ex, prefix);
@@ -361,7 +370,8 @@ cudaError_t scan_codes_n(const pm_codes_t* in, int nsp, int64_t ncell, int64_t* 
     get.v[s] = CodesCount{in[s].cnt, in[s].esc, in[s].n_esc, in[s].esc_cap, in[s].vmax, status};
     put.v[s] = PutOffsets{off[s], clear ? clear->counts[s] : nullptr, clear ? clear->far[s] : nullptr};
     fin.v[s] = FinishArgs{in[s].n, off[s], nullptr, 0, nullptr, nullptr, s == 0 && clear ? clear->small : nullptr,
-                          s == 0 && clear ? clear->small_words : 0};
+                          s == 0 && clear ? clear->small_words : 0,
+                          clear ? static_cast<uint4*>(clear->mesh) : nullptr, clear ? clear->mesh_words : 0};
   }
   const int tiles = scan_tiles(ncell);
   k_scan<<<dim3(tiles, nsp), SCAN_THREADS, 0, st>>>(get, put, fin, ncell, tiles, static_cast<unsigned char*>(state),
@@ -380,7 +390,7 @@ cudaError_t scan_counts_n(const uint32_t* const* counts, const uint32_t* const* 
     get.v[s] = U32Count{counts[s], far ? far[s] : nullptr};
     put.v[s] = PutCodes{off[s], out[s].cnt, out[s].esc, out[s].esc_cap, status};
     fin.v[s] = FinishArgs{expect[s], off[s], out[s].n_esc, out[s].esc_cap, vmax_bits[s],
-                          vmax_bits[s] ? out[s].vmax : nullptr, nullptr, 0};
+                          vmax_bits[s] ? out[s].vmax : nullptr, nullptr, 0, nullptr, 0};
   }
   const int tiles = scan_tiles(ncell);
   k_scan<<<dim3(tiles, nsp), SCAN_THREADS, 0, st>>>(get, put, fin, ncell, tiles, static_cast<unsigned char*>(state),
