@@ -485,15 +485,16 @@ __global__ void __launch_bounds__(PassA<N>::threads, PassA<N>::min_blocks)
 // current transform runs: 36 4-byte loads per item, each component's waited for
 // in turn, kept the earlier form at 0.212 ms for 64 tiles; 0.206 now, and 0.196
 // with 18 columns and 160 threads at 5 blocks per SM (18 x 224 at 4: 0.199;
-// 26 x 320 at 3: 0.197).  216 tiles of 48^3 0.163 -> 0.099 ms.
+// 26 x 320 at 3: 0.197).  216 tiles of 48^3 0.163 -> 0.089 ms (224 threads at 3
+// blocks per SM 0.100, 13 columns with 128 threads 0.107 and 0.092 at 5 and 8).
 template <int N> struct PassBR {
   static constexpr int NH = N / 2 + 1, NP = spec_pitch(N);
   // columns per block (N = 96: box rows of whole 16-byte words), and threads
   // that take each item set in few, full rounds
   static constexpr int KT = N == 128 ? 22 : (N == 96 ? PM_PASSB_KT : (N == 64 ? 17 : NH));
   static constexpr int nchunk = (NH + KT - 1) / KT;
-  static constexpr int threads = N == 128 ? 192 : (N == 96 ? PM_PASSB_TMA_THREADS : (N == 48 ? 224 : (N == 16 ? 64 : 160)));
-  static constexpr int min_blocks = N == 128 ? 3 : (N == 96 ? PM_PASSB_TMA_MINB : (N == 48 ? 3 : 4));
+  static constexpr int threads = N == 128 ? 192 : (N == 96 ? PM_PASSB_TMA_THREADS : (N == 16 ? 64 : 160));
+  static constexpr int min_blocks = N == 128 ? 3 : (N == 96 ? PM_PASSB_TMA_MINB : (N == 48 ? 5 : 4));
   // G [3][N][KT] (component, z, column; the forward transform in component 0), twiddles
   static constexpr size_t smem = kTmaAlign + sizeof(float2) * (3 * (size_t)N * KT + N);
 };
@@ -630,7 +631,8 @@ __global__ void __launch_bounds__(PassBR<N>::threads, PassBR<N>::min_blocks)
 //     sizes write the output rows to a second buffer, both rows of a pair in one
 //     16-byte word.
 // 64 tiles of 96^3 0.291 -> 0.197 ms (two buffers, 3 blocks of 384: 0.221; 5
-// blocks of 256 with 48 registers: 0.199), 216 tiles of 48^3 0.182 -> 0.103 ms,
+// blocks of 256 with 48 registers: 0.199), 216 tiles of 48^3 0.182 -> 0.097 ms
+// (compiled for 8 blocks per SM; for 4 0.102),
 // 128^3 mesh 33 -> 21 us.  Bound by issue now (75% of the slots).  The spectrum
 // rows between passes B and C are not padded: pass B's stores take 0.182 ms with
 // them in place of 0.195.
@@ -646,7 +648,7 @@ template <int N> struct PassC {
   // in place the x step's items are one round: 256 threads serve 32 row pairs of
   // 96 (the buffered tiles), 384 all 48; else one round of the largest item set
   static constexpr int threads = N == 128 ? 544 : (N == 96 ? 384 : (N == 64 ? 288 : (N == 48 ? 160 : 96)));
-  static constexpr int min_blocks(int t) { return N == 128 ? 2 : (N == 96 ? (t == 256 ? PM_SOLVE_C_MINB : 3) : 4); }
+  static constexpr int min_blocks(int t) { return N == 128 ? 2 : (N == 96 ? (t == 256 ? PM_SOLVE_C_MINB : 3) : (N == 48 ? 8 : 4)); }
   static constexpr size_t align = 128;
   // P [N][NP] (then W [pairs][N + 1]), twiddles, Y [pairs][NH] 16-byte words or, in place, room for the prolongation
   static size_t smem(int t, int b, int prc, bool prolong) {
