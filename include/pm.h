@@ -461,7 +461,10 @@ int pm_set_graphs(pm_handle_t* h, int on);
  *  tile_batch          fine tiles per solve launch, 1..the configured batch.
  * Every block edge must divide n_cmp and the shared memory must fit one block
  * of the device (PM_ERR_ARG otherwise).  pm_set_tuning drops captured step
- * graphs (synchronising the device first). */
+ * graphs (synchronising the device first).  A kick block and window that need
+ * larger tables than the handle holds allocate them (those they replace stay
+ * until pm_destroy); where memory for them is short, the passes run with the
+ * block that pm_init chose, with the same results. */
 typedef struct pm_tuning {
   int32_t deposit_block[3];
   int32_t deposit_persistent;

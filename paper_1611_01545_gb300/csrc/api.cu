@@ -38,6 +38,7 @@ struct pm_handle {
   uint32_t* far[2] = {nullptr, nullptr};      // a step's far movers per new cell
   uint32_t* start = nullptr;                  // start of each cell block's share of its window cells
   size_t start_bytes = 0;
+  std::vector<uint32_t*> old_starts;   // tables that a larger one has replaced
   uint32_t* vmax_bits = nullptr;  // [2]; one allocation with amax and work, cleared together by a step's first scan
   uint32_t* amax = nullptr;       // [3] max |a| over the coarse / fine force meshes and the PP accelerations (float bits)
   float4* app = nullptr;          // per particle PP acceleration (pp = 1), stream order, species 0 first
@@ -297,7 +298,9 @@ size_t table_budget(const pm_handle* h) {
   const size_t q = (size_t)h->scratch_n * 16 / 4;
   return q > ((size_t)256 << 20) ? q : (size_t)256 << 20;
 }
-// Makes room for the start tables of kick block b.
+// Makes room for the start tables of kick block b.  A table that a larger one
+// replaces lives on until the handle ends: graphs that a caller captured hold its
+// address.  The allocation is no part of a capture that the thread has open.
 cudaError_t reserve_tables(pm_handle* h, Blk b) {
   if (h->scratch_n == 0) return cudaSuccess;   // no particles, no tables
   b = kick_blocks(h->geo, b, h->scratch_n);
@@ -305,12 +308,15 @@ cudaError_t reserve_tables(pm_handle* h, Blk b) {
   const size_t need = table_bytes(h->geo, b);
   if (need <= h->start_bytes) return cudaSuccess;
   void* p = nullptr;
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaThreadExchangeStreamCaptureMode(&mode);
   const cudaError_t e = cudaMalloc(&p, need);
+  cudaThreadExchangeStreamCaptureMode(&mode);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return e;
   }
-  if (h->start) cudaFree(h->start);   // waits for the work that uses it
+  if (h->start) h->old_starts.push_back(h->start);
   h->start = static_cast<uint32_t*>(p);
   h->start_bytes = need;
   return cudaSuccess;
@@ -321,6 +327,10 @@ RecompressTables tables(const pm_handle* h) {
 Blk ikd_blk(const pm_handle* h, int pass) {
   Blk b = kick_blocks(h->geo, h->blk_ikd, h->scratch_n);
   b.D = table_window(h->geo, b, table_budget(h));
+  if (table_bytes(h->geo, b) > h->start_bytes) {   // no memory was left for this shape's tables: the shape of pm_init
+    b = kick_blocks(h->geo, choose_blk(h->gm, h->cfg.deposit_mode == 1, false), h->scratch_n);
+    b.D = table_window(h->geo, b, table_budget(h));
+  }
   b.work = h->persist_ikd ? h->work + 1 + pass : nullptr;
   b.brick = block_brick(b);
   return b;
@@ -624,6 +634,7 @@ int pm_destroy(pm_handle_t* h) {
   for (auto e : h->timer.pool) cudaEventDestroy(e);
   for (void* p : h->allocs) cudaFree(p);
   if (h->start) cudaFree(h->start);
+  for (uint32_t* p : h->old_starts) cudaFree(p);
   if (h->pool) cudaMemPoolDestroy(h->pool);
   delete h;
   return PM_OK;
@@ -968,7 +979,7 @@ int apply_tuning(pm_handle* h, const pm_tuning_t* t) {
     return fail(h, PM_ERR_ARG, "tile_batch must lie in [1, the configured tile batch]");
   if ((t->deposit_persistent & ~1) || (t->kick_persistent & ~1)) return fail(h, PM_ERR_ARG, "persistent flags are 0 or 1");
   drop_graphs(h);
-  CK(h, reserve_tables(h, bi));
+  reserve_tables(h, bi);   // where memory is short, the passes run with the shape of pm_init (ikd_blk)
   h->blk_dep = bd;
   h->blk_ikd = bi;
   h->persist_dep = t->deposit_persistent != 0;

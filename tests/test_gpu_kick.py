@@ -96,3 +96,46 @@ def test_ranks_beyond_the_key():
     pm = _pm(n, (11, x.shape[0]), 16)
     pm.set_tuning({"kick_block": (16, 1, 1), "kick_window": 4})
     _check(pm, codes, n, 16)
+
+
+# a tuning that needs larger tables than the handle holds: with no memory left for
+# them the step runs all the same, and a graph captured before keeps its own
+@pytest.mark.parametrize("short", [False, True])
+def test_tuning_with_larger_tables(short):
+    n, counts = 128, (3000, 60000)
+    rng = np.random.default_rng(7)
+    codes = [_species(rng, n, counts[s], 2.0, 8) for s in range(2)]
+    pm = _pm(n, counts, 8)
+    din = [lib_codes_from_oracle(c) for c in codes]
+    dout = [pm.empty_codes(c.n, esc_cap=(n // 4) ** 3) for c in codes]
+
+    def check():
+        torch.cuda.synchronize()
+        pm.check()
+        for c, d in zip(codes, dout):
+            got, ref = oracle_codes_from_lib(d, n // 4, 8), _drifted(c, n, 8)
+            assert got.vmax == ref.vmax
+            np.testing.assert_array_equal(got.cnt, ref.cnt)
+            np.testing.assert_array_equal(records(got), records(ref))
+            d.pos.zero_()
+            d.cnt.zero_()
+
+    pm.step(din, dout, 0.0, 1.0)
+    check()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        pm.step(din, dout, 0.0, 1.0)
+    filler = None
+    if short:
+        torch.cuda.empty_cache()
+        free, _ = torch.cuda.mem_get_info()
+        filler = torch.empty(free - (100 << 20), dtype=torch.uint8, device="cuda")   # the tables take 191 MB
+    tuning = {"kick_block": (1, 1, 1), "kick_window": 4}
+    pm.set_tuning(tuning)
+    assert pm.get_tuning()["kick_window"] == 4
+    pm.step(din, dout, 0.0, 1.0)
+    del filler
+    torch.cuda.empty_cache()
+    check()
+    graph.replay()
+    check()
