@@ -26,8 +26,9 @@ using namespace pmfft;
 template <int N> struct SolveCfg {
   static constexpr int NH = N / 2 + 1;
   static constexpr int NP = spec_pitch(N);   // row pitch (complex values) of the spectrum buffers
-// Threads per block of passes A and C (compile-time tunables; measured on the
-// 96^3 tiles: 512 for A, 384 for C).
+// Compile-time tunables of the 96^3 passes (the alternatives' times stand at each
+// pass): threads of pass A, blocks per SM of A and C, columns, threads and blocks
+// per SM of pass B.
 #ifndef PM_SOLVE_THREADS
 #define PM_SOLVE_THREADS 416
 #endif
