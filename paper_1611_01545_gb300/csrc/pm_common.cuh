@@ -53,11 +53,13 @@ struct SolvePlan {
   float2* spec3 = nullptr; // device [batch][3][t][N][NP]
 };
 
-// Lets a kernel use smem bytes of dynamic shared memory: up to 48 KB need no
-// call, which the launch-bound small meshes notice.
+// Lets a kernel use smem bytes of dynamic shared memory.  A block's static and
+// dynamic shared memory together need no call up to 48 KB, which the launch-bound
+// small meshes notice; the static part of these kernels is at most 272 bytes (k_pp),
+// so the last KB below 48 is left to it.
 template <class K>
 inline void allow_smem(K kernel, size_t smem) {
-  if (smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (smem > 47 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
 // Counts kernel launches made by the library (all handles); read by pm_launch_count.
