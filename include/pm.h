@@ -30,6 +30,12 @@
  *     found while launching are returned; errors found on the device (a
  *     corrupt stream, a capacity overflow) set a sticky status word that
  *     pm_check() returns;
+ *   - calls on one handle share its workspace, so they follow one another on
+ *     the device (one stream, or streams that wait for each other); only
+ *     pm_decompress and pm_compress of different species, and calls that take
+ *     meshes and float particles of the caller's (pm_deposit, _fixed and
+ *     _weights, pm_interpolate, pm_kick_drift, pm_interpolate_adjoint,
+ *     pm_deposit_adjoint, pm_restrict, pm_tile_density), may overlap;
  *   - sizes and indices are 64-bit.
  * Return value of every int function: PM_OK or one PM_ERR_* code; the text
  * of the last error is available from pm_last_error().
@@ -193,8 +199,8 @@ int pm_decompress(pm_handle_t* h, int species, const pm_codes_t* in, float* x, f
  * whole device memory budget and forbid libraries to allocate, and for host
  * threads that must not pay the device-wide synchronisation cudaMalloc and
  * cudaFree can cause.  No handle is needed and nothing is allocated: the
- * scratch (CSR offsets of at most 64^3 compression cells, scan partials and a
- * status word, about 2.1 MB) is one fixed __device__ array inside the library,
+ * scratch (CSR offsets of at most 64^3 compression cells, the scan's state and
+ * a status word, about 2.1 MB) is one fixed __device__ array inside the library,
  * which every GPU that loads the library keeps until the process exits.
  *  n_fine, cmp_ratio, vel_bits  as in pm_config_t; (n_fine/cmp_ratio)^3 must
  *                               not exceed 64^3, else PM_ERR_ARG;

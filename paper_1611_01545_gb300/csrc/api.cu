@@ -42,7 +42,7 @@ struct pm_handle {
   uint32_t* vmax_bits = nullptr;  // [2]; one allocation with amax and work, cleared together by a step's first scan
   uint32_t* amax = nullptr;       // [3] max |a| over the coarse / fine force meshes and the PP accelerations (float bits)
   float4* app = nullptr;          // per particle PP acceleration (pp = 1), stream order, species 0 first
-  void* scan_state = nullptr;     // look-back state of the scans, both species (zero between launches)
+  void* scan_state = nullptr;     // look-back state of the scans, one part per species
   int* status = nullptr;
   Blk blk_dep{}, blk_ikd{};
   bool persist_dep = false, persist_ikd = false;   // persistent launches of the particle passes
@@ -320,6 +320,10 @@ cudaError_t reserve_tables(pm_handle* h, Blk b) {
   h->start = static_cast<uint32_t*>(p);
   h->start_bytes = need;
   return cudaSuccess;
+}
+// The part of one species, for the calls that scan only its counts.
+void* scan_state_of(const pm_handle* h, int species) {
+  return static_cast<unsigned char*>(h->scan_state) + (size_t)species * scan_state_bytes(h->gm.ncell());
 }
 RecompressTables tables(const pm_handle* h) {
   return RecompressTables{h->counts[0], h->counts[1], h->far[0], h->far[1], h->start, 0};
@@ -654,7 +658,7 @@ int pm_decompress(pm_handle_t* h, int species, const pm_codes_t* in, float* x, f
   if (int r = check_species(h, species)) return r;
   cudaStream_t st = (cudaStream_t)stream;
   const bool vel16 = h->cfg.vel_bits == 16;
-  CK(h, scan_codes(*in, h->gm.ncell(), h->off[species], h->scan_state, h->status, st));
+  CK(h, scan_codes(*in, h->gm.ncell(), h->off[species], scan_state_of(h, species), h->status, st));
   CK(h, launch_decompress(view(*in, vel16), h->off[species], h->geo, x, v, st));
   return PM_OK;
 }
@@ -668,7 +672,7 @@ int pm_compress(pm_handle_t* h, int species, const float* x, const float* v, con
   cudaStream_t st = (cudaStream_t)stream;
   CK(h, cudaMemsetAsync(h->counts[species], 0, (size_t)h->gm.ncell() * 4, st));
   CK(h, launch_compress(x, v, out->n, h->geo, h->counts[species], h->vmax_bits + species, vmax_in,
-                        h->newoff[species], *out, h->cfg.vel_bits == 16, h->scan_state, h->status, st));
+                        h->newoff[species], *out, h->cfg.vel_bits == 16, scan_state_of(h, species), h->status, st));
   return PM_OK;
 }
 

@@ -5,7 +5,7 @@
 // the device's whole memory budget and hands libraries only the buffers they
 // are given, or a host thread that must not pay the device-wide
 // synchronisation that cudaMalloc / cudaFree can cause.  pm_decompress_noalloc
-// serves them: its only scratch (the per-cell CSR offsets, the scan partials
+// serves them: its only scratch (the per-cell CSR offsets, the scan's state
 // and a status word) lives in one file-scope __device__ array of fixed size,
 // which every GPU that loads the library keeps until the process exits.
 #include <cuda_runtime.h>
@@ -20,9 +20,9 @@ namespace {
 
 constexpr int64_t kMaxCells = (int64_t)64 * 64 * 64;   // n_cmp <= 64
 constexpr size_t kOffBytes = (size_t)(kMaxCells + 1) * sizeof(int64_t);
-constexpr size_t kPartialOffset = (kOffBytes + 255) / 256 * 256;
-constexpr size_t kPartialBytes = 4096;                  // >= pm::scan_state_bytes(kMaxCells); zero at load, and again after each scan
-constexpr size_t kStatusOffset = kPartialOffset + kPartialBytes;
+constexpr size_t kStateOffset = (kOffBytes + 255) / 256 * 256;
+constexpr size_t kStateBytes = 4096;                    // >= pm::scan_state_bytes(kMaxCells)
+constexpr size_t kStatusOffset = kStateOffset + kStateBytes;
 constexpr size_t kScratchBytes = kStatusOffset + 256;
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
@@ -60,16 +60,17 @@ extern "C" int pm_decompress_noalloc(int32_t n_fine, int32_t cmp_ratio, int32_t 
   if (n_fine <= 0 || cmp_ratio <= 0 || (cmp_ratio & (cmp_ratio - 1)) || n_fine % cmp_ratio) return PM_ERR_ARG;
   const int ncmp = n_fine / cmp_ratio;
   const int64_t ncell = (int64_t)ncmp * ncmp * ncmp;
-  if (ncell > kMaxCells || pm::scan_state_bytes(ncell) > kPartialBytes) return PM_ERR_ARG;
+  if (ncell > kMaxCells || pm::scan_state_bytes(ncell) > kStateBytes) return PM_ERR_ARG;
   unsigned char* base = nullptr;
   if (scratch_address(&base) != cudaSuccess) return PM_ERR_CUDA;
   int64_t* off = reinterpret_cast<int64_t*>(base);
-  void* partial = base + kPartialOffset;
+  void* state = base + kStateOffset;
   int* status = reinterpret_cast<int*>(base + kStatusOffset);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess) return PM_ERR_CUDA;
+  // the state, whose tiles are another mesh's in every call, and the status behind it
+  if (cudaMemsetAsync(state, 0, kStateBytes + sizeof(int), st) != cudaSuccess) return PM_ERR_CUDA;
   pm::Geo g{n_fine, 1, 0, cmp_ratio, ncmp, ncell, false};
-  if (pm::scan_codes(*in, ncell, off, partial, status, st) != cudaSuccess) return PM_ERR_CUDA;
+  if (pm::scan_codes(*in, ncell, off, state, status, st) != cudaSuccess) return PM_ERR_CUDA;
   pm::PCodes view{reinterpret_cast<const uint32_t*>(in->pos), in->vel, in->vmax, in->n, vel_bits == 16};
   if (pm::launch_decompress(view, off, g, x, v, st) != cudaSuccess) return PM_ERR_CUDA;
   int host_status = 0;

@@ -38,8 +38,8 @@ struct PCodesOut {
   bool vel16;
 };
 
-// Scans (scan.cu).  state: scan_state_bytes(ncell) per species, zeroed once
-// when it is allocated (each launch leaves it zero again).
+// Scans (scan.cu).  state: scan_state_bytes(ncell) per species, zeroed once before
+// its first scan; every scan on it has the same ncell, and they follow one another.
 size_t scan_state_bytes(int64_t ncell);
 // Arrays that a step's first scan clears on the way: the new-cell counts of
 // both species, window and far movers, and `small_words` 32-bit words (null: nothing).

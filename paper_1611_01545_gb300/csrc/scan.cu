@@ -11,7 +11,10 @@
 // publishes its own sum, then walks back over the published sums, a warp's 32
 // at a time, until it meets a tile whose whole prefix is known.  Tiles are
 // numbered by a ticket drawn when their block starts, so every tile waited for
-// is already running.  Per scan of two species this saves 14 to 16 us on 64^3
+// is already running.  Tickets count on from launch to launch and published sums
+// carry their launch's number: a launch relies on nothing that an earlier one has
+// to clear, and launches that overlap on one state, which callers must not let
+// happen, spoil no later one.  Per scan of two species this saves 14 to 16 us on 64^3
 // cells and 20 us on 16^3 (two steps and a deposit on a 64^3 mesh: 272 -> 171
 // us, with the step's memsets folded in).
 #include <cuda_runtime.h>
@@ -62,63 +65,70 @@ __device__ __forceinline__ V2 block_excl(V2 v, V2* total) {
   return before;
 }
 
-// A tile's published sum in one 64-bit word, so that value and state arrive
-// together: particles in the low 35 bits, escapes in the next 27, state on
-// top.  3.4e10 particles and 1.3e8 escape cells (each of >= 255 particles)
-// exceed what a device can hold; a corrupt stream that claims more saturates
-// and fails the check of the total.
-constexpr unsigned long long kSumMask = (1ull << 35) - 1, kEscMask = (1ull << 27) - 1;
-constexpr unsigned long long kOwnSum = 1ull << 62, kPrefix = 2ull << 62;   // states: 0 nothing yet
+// A tile's published sum in two 64-bit words, particles and cells with an escape
+// entry, each under a head that says what it is: the launch's number in the top 28
+// bits, then a bit for a whole prefix (else the tile's own sum).  A pair whose heads
+// agree belongs together.  Below the head fit 3.4e10, more particles than a device
+// can hold; a corrupt stream that claims more saturates and fails the check of the
+// total.
+constexpr int kHeadShift = 35;
+constexpr unsigned long long kValueMask = (1ull << kHeadShift) - 1;
+constexpr unsigned kLaunchMask = (1u << 28) - 1;
 
-__device__ __forceinline__ unsigned long long pack(V2 v) {
-  const unsigned long long a = (unsigned long long)v.a < kSumMask ? (unsigned long long)v.a : kSumMask;
-  const unsigned long long b = (unsigned long long)v.b < kEscMask ? (unsigned long long)v.b : kEscMask;
-  return a | (b << 35);
+struct alignas(16) TileSum {
+  unsigned long long a, b;
+};
+__device__ __forceinline__ TileSum tile_sum(V2 v, unsigned launch, bool whole) {
+  const unsigned long long head = ((unsigned long long)launch << 1 | (whole ? 1u : 0u)) << kHeadShift;
+  const unsigned long long a = (unsigned long long)v.a < kValueMask ? (unsigned long long)v.a : kValueMask;
+  return TileSum{head | a, head | (unsigned)v.b};
 }
-__device__ __forceinline__ V2 unpack(unsigned long long w) {
-  return V2{(long long)(w & kSumMask), (int)((w >> 35) & kEscMask)};
+__device__ __forceinline__ V2 value_of(const TileSum& t) {
+  return V2{(long long)(t.a & kValueMask), (int)(t.b & kValueMask)};
 }
 
-// Device state of one species' scan: all zero between launches (the last
-// block to finish clears it again).
+// Device state of one species' scan, zeroed once before its first launch.  Every
+// launch on it draws as many tickets as it has tiles, the same number each time.
 struct ScanState {
-  unsigned ticket;   // tiles handed out
-  unsigned done;     // tiles whose look-back is over
-  unsigned long long pad;
-  __device__ unsigned long long* tiles() { return reinterpret_cast<unsigned long long*>(this + 1); }
+  unsigned long long ticket, pad;
+  __device__ TileSum* tiles() { return reinterpret_cast<TileSum*>(this + 1); }
 };
 static_assert(sizeof(ScanState) == 16, "one 16-byte header");
 
-__device__ __forceinline__ unsigned long long load_word(const unsigned long long* p) {
-  unsigned long long w;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];\n" : "=l"(w) : "l"(p) : "memory");
-  return w;
+__device__ __forceinline__ TileSum load_sum(const TileSum* p) {
+  TileSum t;
+  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];\n" : "=l"(t.a), "=l"(t.b) : "l"(p) : "memory");
+  return t;
 }
-__device__ __forceinline__ void store_word(unsigned long long* p, unsigned long long w) {
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;\n" ::"l"(p), "l"(w) : "memory");
+__device__ __forceinline__ void store_sum(TileSum* p, TileSum t) {
+  asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};\n" ::"l"(p), "l"(t.a), "l"(t.b) : "memory");
 }
 
-// Prefix of tile `tile` over the earlier tiles, by the first warp.  A wait is
-// given up after about a second (status ST_TIMEOUT).
-__device__ __forceinline__ V2 look_back(const unsigned long long* tiles, int tile, int* status) {
+// Prefix of tile `tile` over the earlier tiles of launch number `launch`, by the
+// first warp.  A wait is given up after about a second, or at once where a later
+// launch has overwritten what it waits for (status ST_TIMEOUT).
+__device__ __forceinline__ V2 look_back(const TileSum* tiles, int tile, unsigned launch, int* status) {
   const int lane = threadIdx.x & 31;
   V2 sum{0, 0};
   for (int last = tile - 1; last >= 0; last -= 32) {
     const int i = last - lane;
-    unsigned long long w = i >= 0 ? load_word(tiles + i) : kPrefix;
-    if (__any_sync(0xffffffffu, (w >> 62) == 0)) {
+    TileSum w = i >= 0 ? load_sum(tiles + i) : tile_sum(V2{0, 0}, launch, true);
+    const auto waiting = [&] { return (unsigned)(w.a >> (kHeadShift + 1)) != launch || ((w.a ^ w.b) >> kHeadShift) != 0; };
+    if (__any_sync(0xffffffffu, waiting())) {
       const long long t0 = clock64();
-      while (__any_sync(0xffffffffu, (w >> 62) == 0)) {
-        if (i >= 0) w = load_word(tiles + i);
-        if (__any_sync(0xffffffffu, clock64() - t0 > 2000000000LL)) {
+      while (__any_sync(0xffffffffu, waiting())) {
+        if (i >= 0) w = load_sum(tiles + i);
+        const unsigned ahead = ((unsigned)(w.a >> (kHeadShift + 1)) - launch) & kLaunchMask;
+        const bool later = ahead != 0 && ahead <= kLaunchMask / 2;
+        if (__any_sync(0xffffffffu, later || clock64() - t0 > 2000000000LL)) {
           if (lane == 0) atomicOr(status, ST_TIMEOUT);
           return sum;
         }
       }
     }
-    const unsigned known = __ballot_sync(0xffffffffu, (w >> 62) == 2);
+    const unsigned known = __ballot_sync(0xffffffffu, (w.a >> kHeadShift & 1u) != 0);
     const int upto = known ? __ffs(known) - 1 : 31;   // nearest tile whose whole prefix is known
-    V2 v = lane <= upto ? unpack(w) : V2{0, 0};
+    V2 v = lane <= upto ? value_of(w) : V2{0, 0};
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       v.a += __shfl_xor_sync(0xffffffffu, v.a, o);
@@ -301,11 +311,17 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan(Pair<Get> gets, Pair<Put>
   const Get& get = gets.v[blockIdx.y];
   const FinishArgs& f = fin.v[blockIdx.y];
   ScanState* st = reinterpret_cast<ScanState*>(state + blockIdx.y * stride);
-  __shared__ int s_tile, s_last;
+  __shared__ int s_tile;
+  __shared__ unsigned s_launch;
   __shared__ V2 s_prefix;
-  if (threadIdx.x == 0) s_tile = (int)atomicAdd(&st->ticket, 1u);
+  if (threadIdx.x == 0) {
+    const unsigned long long t = atomicAdd(&st->ticket, 1ull), l = t / (unsigned)tiles;
+    s_tile = (int)(t - l * (unsigned)tiles);
+    s_launch = (unsigned)(l + 1) & kLaunchMask;   // (zeroed words are no launch's)
+  }
   __syncthreads();
   const int tile = s_tile;
+  const unsigned launch = s_launch;
   const int64_t c = (int64_t)tile * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
   V2 v[SCAN_ITEMS];
   get.load(c, n, v);
@@ -313,15 +329,15 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan(Pair<Get> gets, Pair<Put>
 #pragma unroll
   for (int k = 0; k < SCAN_ITEMS; ++k) own = v2add(own, v[k]);
   V2 ex = block_excl(own, &total);
-  unsigned long long* words = st->tiles();
+  TileSum* sums = st->tiles();
   if (threadIdx.x < 32) {
     V2 before{0, 0};
     if (tile > 0) {
-      if (threadIdx.x == 0) store_word(words + tile, kOwnSum | pack(total));
-      before = look_back(words, tile, status);
+      if (threadIdx.x == 0) store_sum(sums + tile, tile_sum(total, launch, false));
+      before = look_back(sums, tile, launch, status);
     }
     if (threadIdx.x == 0) {
-      store_word(words + tile, kPrefix | pack(v2add(before, total)));
+      store_sum(sums + tile, tile_sum(v2add(before, total), launch, true));
       s_prefix = before;
     }
   }
@@ -341,20 +357,11 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan(Pair<Get> gets, Pair<Put>
   const V2 prefix = s_prefix;
   ex = v2add(ex, prefix);
   puts.v[blockIdx.y](c, n, ex, v);
-  if (threadIdx.x == 0) {
-    if (tile == tiles - 1) {
-      const V2 t = v2add(prefix, total);
-      f.off[n] = t.a;
-      if (t.a != f.expect) atomicOr(status, ST_CORRUPT);
-      if (f.n_esc_out) *f.n_esc_out = (uint32_t)(t.b < f.esc_cap ? t.b : f.esc_cap);
-    }
-    __threadfence();
-    s_last = atomicAdd(&st->done, 1u) == (unsigned)tiles - 1u;
-  }
-  __syncthreads();
-  if (s_last) {   // every look-back is over: clear the state for the next launch
-    for (int i = threadIdx.x; i < tiles; i += SCAN_THREADS) words[i] = 0ull;
-    if (threadIdx.x == 0) st->ticket = st->done = 0u;
+  if (threadIdx.x == 0 && tile == tiles - 1) {
+    const V2 t = v2add(prefix, total);
+    f.off[n] = t.a;
+    if (t.a != f.expect) atomicOr(status, ST_CORRUPT);
+    if (f.n_esc_out) *f.n_esc_out = (uint32_t)(t.b < f.esc_cap ? t.b : f.esc_cap);
   }
 }
 
@@ -402,7 +409,7 @@ cudaError_t scan_counts_n(const uint32_t* const* counts, const uint32_t* const* 
 }  // namespace
 
 // State of one species' scan; the two-species scans use twice this.  Zero it once.
-size_t scan_state_bytes(int64_t ncell) { return sizeof(ScanState) + 8 * (size_t)((scan_tiles(ncell) + 1) / 2 * 2); }
+size_t scan_state_bytes(int64_t ncell) { return sizeof(ScanState) + sizeof(TileSum) * (size_t)scan_tiles(ncell); }
 
 cudaError_t scan_codes(const pm_codes_t& in, int64_t ncell, int64_t* off, void* state, int* status,
                        cudaStream_t st) {
