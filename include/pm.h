@@ -214,7 +214,8 @@ int pm_decompress(pm_handle_t* h, int species, const pm_codes_t* in, float* x, f
  * leaves its contents behind; calls that overlap on the GPU (other streams,
  * other host threads) race on it, so the caller must serialise them.  The
  * call synchronises `stream` before returning and reports a corrupt stream
- * as PM_ERR_CORRUPT directly (there is no handle to query). */
+ * as PM_ERR_CORRUPT and a device wait that ran out as PM_ERR_TIMEOUT directly
+ * (there is no handle to query). */
 int pm_decompress_noalloc(int32_t n_fine, int32_t cmp_ratio, int32_t vel_bits, const pm_codes_t* in, float* x,
                           float* v, void* stream);
 

@@ -1595,11 +1595,13 @@ int pm_check(pm_handle_t* h, void* stream) {
   int s = 0;
   CK(h, cudaMemcpy(&s, h->status, 4, cudaMemcpyDeviceToHost));
   CK(h, cudaMemset(h->status, 0, 4));
-  if (s & ST_RANGE) return fail(h, PM_ERR_RANGE, "device validation: position outside [0, n_fine)");
-  if (s & ST_OVERFLOW) return fail(h, PM_ERR_OVERFLOW, "device validation: escape list capacity exceeded");
-  if (s & ST_CORRUPT) return fail(h, PM_ERR_CORRUPT, "device validation: corrupt compressed stream");
-  if (s & ST_TIMEOUT) return fail(h, PM_ERR_TIMEOUT, "device wait timed out");
-  return PM_OK;
+  switch (const int code = status_error(s)) {
+    case PM_ERR_RANGE: return fail(h, code, "device validation: position outside [0, n_fine)");
+    case PM_ERR_OVERFLOW: return fail(h, code, "device validation: escape list capacity exceeded");
+    case PM_ERR_CORRUPT: return fail(h, code, "device validation: corrupt compressed stream");
+    case PM_ERR_TIMEOUT: return fail(h, code, "device wait timed out");
+    default: return code;
+  }
 }
 
 int pm_wait_probe(pm_handle_t* h, int64_t limit_cycles, void* stream) {

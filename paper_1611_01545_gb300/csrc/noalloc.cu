@@ -76,6 +76,5 @@ extern "C" int pm_decompress_noalloc(int32_t n_fine, int32_t cmp_ratio, int32_t 
   int host_status = 0;
   if (cudaMemcpyAsync(&host_status, status, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess) return PM_ERR_CUDA;
   if (cudaStreamSynchronize(st) != cudaSuccess) return PM_ERR_CUDA;
-  if (host_status & pm::ST_CORRUPT) return PM_ERR_CORRUPT;
-  return PM_OK;
+  return pm::status_error(host_status);
 }

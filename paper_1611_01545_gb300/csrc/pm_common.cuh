@@ -7,10 +7,9 @@
 #include <vector>
 
 #include "pm.h"
+#include "status.h"
 
 namespace pm {
-
-enum StatusBits : int { ST_CORRUPT = 1, ST_OVERFLOW = 2, ST_RANGE = 4, ST_TIMEOUT = 8 };
 
 // Mesh / tile / compression-cell geometry derived from pm_config_t.
 struct Geom {

@@ -105,9 +105,10 @@ __device__ __forceinline__ void store_sum(TileSum* p, TileSum t) {
 }
 
 // Prefix of tile `tile` over the earlier tiles of launch number `launch`, by the
-// first warp.  A wait is given up after about a second, or at once where a later
+// first warp.  A wait is given up after `limit` cycles, or at once where a later
 // launch has overwritten what it waits for (status ST_TIMEOUT).
-__device__ __forceinline__ V2 look_back(const TileSum* tiles, int tile, unsigned launch, int* status) {
+constexpr long long kWaitLimit = 2000000000LL;   // about a second
+__device__ __forceinline__ V2 look_back(const TileSum* tiles, int tile, unsigned launch, long long limit, int* status) {
   const int lane = threadIdx.x & 31;
   V2 sum{0, 0};
   for (int last = tile - 1; last >= 0; last -= 32) {
@@ -120,7 +121,7 @@ __device__ __forceinline__ V2 look_back(const TileSum* tiles, int tile, unsigned
         if (i >= 0) w = load_sum(tiles + i);
         const unsigned ahead = ((unsigned)(w.a >> (kHeadShift + 1)) - launch) & kLaunchMask;
         const bool later = ahead != 0 && ahead <= kLaunchMask / 2;
-        if (__any_sync(0xffffffffu, later || clock64() - t0 > 2000000000LL)) {
+        if (__any_sync(0xffffffffu, later || clock64() - t0 > limit)) {
           if (lane == 0) atomicOr(status, ST_TIMEOUT);
           return sum;
         }
@@ -307,7 +308,7 @@ template <class T> struct Pair { T v[2]; };
 template <class Get, class Put>
 __global__ void __launch_bounds__(SCAN_THREADS) k_scan(Pair<Get> gets, Pair<Put> puts, Pair<FinishArgs> fin,
                                                      int64_t n, int tiles, unsigned char* state, size_t stride,
-                                                     int* status) {
+                                                     long long limit, int* status) {
   const Get& get = gets.v[blockIdx.y];
   const FinishArgs& f = fin.v[blockIdx.y];
   ScanState* st = reinterpret_cast<ScanState*>(state + blockIdx.y * stride);
@@ -334,7 +335,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan(Pair<Get> gets, Pair<Put>
     V2 before{0, 0};
     if (tile > 0) {
       if (threadIdx.x == 0) store_sum(sums + tile, tile_sum(total, launch, false));
-      before = look_back(sums, tile, launch, status);
+      before = look_back(sums, tile, launch, limit, status);
     }
     if (threadIdx.x == 0) {
       store_sum(sums + tile, tile_sum(v2add(before, total), launch, true));
@@ -382,7 +383,7 @@ cudaError_t scan_codes_n(const pm_codes_t* in, int nsp, int64_t ncell, int64_t* 
   }
   const int tiles = scan_tiles(ncell);
   k_scan<<<dim3(tiles, nsp), SCAN_THREADS, 0, st>>>(get, put, fin, ncell, tiles, static_cast<unsigned char*>(state),
-                                                    scan_state_bytes(ncell), status);
+                                                    scan_state_bytes(ncell), kWaitLimit, status);
   note_launches(1);
   return cudaGetLastError();
 }
@@ -401,7 +402,7 @@ cudaError_t scan_counts_n(const uint32_t* const* counts, const uint32_t* const* 
   }
   const int tiles = scan_tiles(ncell);
   k_scan<<<dim3(tiles, nsp), SCAN_THREADS, 0, st>>>(get, put, fin, ncell, tiles, static_cast<unsigned char*>(state),
-                                                    scan_state_bytes(ncell), status);
+                                                    scan_state_bytes(ncell), kWaitLimit, status);
   note_launches(1);
   return cudaGetLastError();
 }

@@ -1,6 +1,6 @@
 """State that a scan leaves for the next one: both species' codecs on two streams,
-then steps on the same handle; and scans whose blocks overlapped on one state,
-after which the next one is right all the same."""
+then steps on the same handle; scans whose blocks overlapped on one state, or that
+waited in vain for a tile, after which the next one is right all the same."""
 import ctypes
 import os
 import subprocess
@@ -15,6 +15,7 @@ from tests.test_gpu_kick import _check, _pm, _species
 
 pytestmark = pytest.mark.gpu
 
+ST_TIMEOUT = 8
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
@@ -56,7 +57,8 @@ def probe(tmp_path_factory):
     lib = ctypes.CDLL(so)
     lib.scan_probe_state.restype = ctypes.c_longlong
     lib.scan_probe_state.argtypes = [ctypes.c_longlong]
-    lib.scan_probe.argtypes = [ctypes.c_void_p] * 4 + [ctypes.c_longlong] * 2 + [ctypes.c_void_p] * 3 + [ctypes.c_int]
+    lib.scan_probe.argtypes = [ctypes.c_void_p] * 4 + [ctypes.c_longlong] * 2 + [ctypes.c_void_p] * 3 + [ctypes.c_int, ctypes.c_int,
+                                                                                                   ctypes.c_longlong]
     return lib
 
 
@@ -72,18 +74,24 @@ def test_scans_that_overlapped_spoil_no_later_one(probe, ncell):
     status = torch.zeros(1, dtype=torch.int32, device="cuda")
     torch.cuda.synchronize()
 
-    def scan(launches):
+    def scan(launches, skip=0, limit=0):
         off = torch.full((ncell + 1,), -1, dtype=torch.int64, device="cuda")
         status.zero_()
         torch.cuda.synchronize()
         rc = probe.scan_probe(cnt.data_ptr(), vmax.data_ptr(), none.data_ptr(), none.data_ptr(), ncell, int(want[-1]),
-                              off.data_ptr(), state.data_ptr(), status.data_ptr(), launches)
+                              off.data_ptr(), state.data_ptr(), status.data_ptr(), launches, skip, limit)
         assert rc == 0
         return off, int(status)
 
     for launches in (1, 2, 3, 2):
         for _ in range(20):
             scan(launches)                     # of those that overlap only the end is asked for
+        off, bad = scan(1)
+        assert bad == 0
+        assert torch.equal(off, want)
+    # a first tile that publishes nothing: the others give up after 0.1 ms and say so
+    if ncell > 2048:
+        assert scan(1, skip=1, limit=200000)[1] & ST_TIMEOUT
         off, bad = scan(1)
         assert bad == 0
         assert torch.equal(off, want)
