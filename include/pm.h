@@ -461,17 +461,21 @@ int pm_set_graphs(pm_handle_t* h, int on);
  *                      cells may be dealt out in halves);
  *  kick_window         half-width in cells of the new-cell window whose
  *                      counts a CTA keeps in shared memory (1..4; particles
- *                      moving further use global counters); the library uses
- *                      a narrower one when the tables of the asked one would
- *                      exceed 256 MB and a quarter of the particle scratch;
+ *                      moving further use global counters).  Its tables take
+ *                      8 bytes per block and window cell; the library uses a
+ *                      narrower window, down to none, when they would exceed
+ *                      256 MB and, for half-widths above 1, a quarter of the
+ *                      particle records (16 bytes per particle of the
+ *                      configured counts), else all of the particle scratch
+ *                      (20 bytes per particle);
  *  kick_persistent     as deposit_persistent, for those passes;
  *  tile_batch          fine tiles per solve launch, 1..the configured batch.
  * Every block edge must divide n_cmp and the shared memory must fit one block
  * of the device (PM_ERR_ARG otherwise).  pm_set_tuning drops captured step
  * graphs (synchronising the device first).  A kick block and window that need
  * larger tables than the handle holds allocate them (those they replace stay
- * until pm_destroy); where memory for them is short, the passes run with the
- * block that pm_init chose, with the same results. */
+ * until pm_destroy); where memory for them is short, here or in pm_init, the
+ * passes run with a narrower window, with the same results. */
 typedef struct pm_tuning {
   int32_t deposit_block[3];
   int32_t deposit_persistent;

@@ -292,34 +292,48 @@ Blk dep_blk(const pm_handle* h) {
   b.brick = block_brick(b);
   return b;
 }
-// Bytes that the start tables may take: a quarter of the per-particle scratch,
-// or 256 MB where that is more.
-size_t table_budget(const pm_handle* h) {
-  const size_t q = (size_t)h->scratch_n * 16 / 4;
-  return q > ((size_t)256 << 20) ? q : (size_t)256 << 20;
+// Bytes that the start tables may take for windows of half-width D: 256 MB, or, where
+// that is more, a quarter of the 16-byte particle records for D > 1 and all of the
+// per-particle scratch (20 bytes) for the narrower ones.  The latter line lies at 3.7
+// particles per cell of the default rows.
+size_t table_budget(const pm_handle* h, int D) {
+  const size_t own = (size_t)h->scratch_n * (D > 1 ? 4 : 20);
+  return own > ((size_t)256 << 20) ? own : (size_t)256 << 20;
 }
-// Makes room for the start tables of kick block b.  A table that a larger one
-// replaces lives on until the handle ends: graphs that a caller captured hold its
-// address.  The allocation is no part of a capture that the thread has open.
-cudaError_t reserve_tables(pm_handle* h, Blk b) {
-  if (h->scratch_n == 0) return cudaSuccess;   // no particles, no tables
+// The blocks that the passes take for kick block b, with the widest window up to the
+// asked one whose tables are within their budget and within `room` bytes.  Narrower
+// windows only make more movers far ones; half-width 0 holds the block's own cells,
+// and -1 (no window, no tables) makes every particle a far mover.
+Blk window_within(const pm_handle* h, Blk b, size_t room) {
   b = kick_blocks(h->geo, b, h->scratch_n);
-  b.D = table_window(h->geo, b, table_budget(h));
-  const size_t need = table_bytes(h->geo, b);
-  if (need <= h->start_bytes) return cudaSuccess;
-  void* p = nullptr;
-  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-  cudaThreadExchangeStreamCaptureMode(&mode);
-  const cudaError_t e = cudaMalloc(&p, need);
-  cudaThreadExchangeStreamCaptureMode(&mode);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return e;
+  for (; b.D >= 0; --b.D) {
+    const size_t need = table_bytes(h->geo, b);
+    if (need <= table_budget(h, b.D) && need <= room) break;
   }
-  if (h->start) h->old_starts.push_back(h->start);
-  h->start = static_cast<uint32_t*>(p);
-  h->start_bytes = need;
-  return cudaSuccess;
+  return b;
+}
+// Makes room for the start tables of kick block b, or, where memory is short, of a
+// narrower window.  A table that a larger one replaces lives on until the handle
+// ends: graphs that a caller captured hold its address.  The allocation is no part of
+// a capture that the thread has open.
+void reserve_tables(pm_handle* h, const Blk& b) {
+  if (h->scratch_n == 0) return;   // no particles, no tables
+  size_t need = table_bytes(h->geo, window_within(h, b, SIZE_MAX));
+  while (need > h->start_bytes) {
+    void* p = nullptr;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    const cudaError_t e = cudaMalloc(&p, need);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e == cudaSuccess) {
+      if (h->start) h->old_starts.push_back(h->start);
+      h->start = static_cast<uint32_t*>(p);
+      h->start_bytes = need;
+      return;
+    }
+    cudaGetLastError();
+    need = table_bytes(h->geo, window_within(h, b, need - 1));
+  }
 }
 // The part of one species, for the calls that scan only its counts.
 void* scan_state_of(const pm_handle* h, int species) {
@@ -329,12 +343,7 @@ RecompressTables tables(const pm_handle* h) {
   return RecompressTables{h->counts[0], h->counts[1], h->far[0], h->far[1], h->start, 0};
 }
 Blk ikd_blk(const pm_handle* h, int pass) {
-  Blk b = kick_blocks(h->geo, h->blk_ikd, h->scratch_n);
-  b.D = table_window(h->geo, b, table_budget(h));
-  if (table_bytes(h->geo, b) > h->start_bytes) {   // no memory was left for this shape's tables: the shape of pm_init
-    b = kick_blocks(h->geo, choose_blk(h->gm, h->cfg.deposit_mode == 1, false), h->scratch_n);
-    b.D = table_window(h->geo, b, table_budget(h));
-  }
+  Blk b = window_within(h, h->blk_ikd, h->start_bytes);
   b.work = h->persist_ikd ? h->work + 1 + pass : nullptr;
   b.brick = block_brick(b);
   return b;
@@ -603,10 +612,7 @@ int pm_init(const pm_config_t* cfg, pm_handle_t** out) {
       h->pool = nullptr;
     }
   }
-  if (rc == PM_OK) {
-    const cudaError_t e = reserve_tables(h, h->blk_ikd);
-    if (e != cudaSuccess) rc = fail(h, PM_ERR_CUDA, std::string("cudaMalloc: ") + cudaGetErrorString(e));
-  }
+  if (rc == PM_OK) reserve_tables(h, h->blk_ikd);
   if (rc != PM_OK) {
     fprintf(stderr, "pm_init: %s\n", h->err.c_str());
     pm_destroy(h);
@@ -983,7 +989,7 @@ int apply_tuning(pm_handle* h, const pm_tuning_t* t) {
     return fail(h, PM_ERR_ARG, "tile_batch must lie in [1, the configured tile batch]");
   if ((t->deposit_persistent & ~1) || (t->kick_persistent & ~1)) return fail(h, PM_ERR_ARG, "persistent flags are 0 or 1");
   drop_graphs(h);
-  reserve_tables(h, bi);   // where memory is short, the passes run with the shape of pm_init (ikd_blk)
+  reserve_tables(h, bi);
   h->blk_dep = bd;
   h->blk_ikd = bi;
   h->persist_dep = t->deposit_persistent != 0;

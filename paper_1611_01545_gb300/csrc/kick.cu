@@ -88,6 +88,7 @@ struct Win {
   int ox, oy, oz, wx, wy, wz;
 };
 __device__ __forceinline__ Win window_of(const Geo& g, const Blk& bk, CellBlock cb) {
+  if (bk.D < 0) return Win{0, 0, 0, 0, 0, 0};
   Win w;
   const int n = g.ncmp, D = bk.D;
   w.wx = bk.RX + 2 * D < n ? bk.RX + 2 * D : n;
@@ -717,7 +718,7 @@ __global__ void __launch_bounds__(kScatterThreads, kScatterMinBlocks) k_kick_sca
     for (int i = threadIdx.x; i < 2 * W; i += blockDim.x) {
       const int sp = i >= W ? 1 : 0, r = i - sp * W;
       const int row = r / win.wx, lx = r - row * win.wx;
-      base[i] = (sp ? k.newoff1 : k.newoff0)[window_row(g, win, row) + window_x(g, win, lx)] + (k.t.start ? (int64_t)start[i] : 0);
+      base[i] = (sp ? k.newoff1 : k.newoff0)[window_row(g, win, row) + window_x(g, win, lx)] + (int64_t)start[i];
     }
     __syncthreads();
     const uint32_t rank_mask = (1u << k.t.kb) - 1u;
@@ -822,6 +823,7 @@ int block_brick(const Blk& bk) {
 }
 
 int window_cells(const Geo& g, const Blk& bk) {
+  if (bk.D < 0) return 0;
   const int n = g.ncmp;
   int wx = bk.RX + 2 * bk.D < n ? bk.RX + 2 * bk.D : n;
   int wy = bk.RY + 2 * bk.D < n ? bk.RY + 2 * bk.D : n;
@@ -841,13 +843,7 @@ Blk kick_blocks(const Geo& g, Blk bk, int64_t particles) {
   return bk;
 }
 
-// Window half-width used for a block shape: the asked one, narrowed until the
-// start tables (8 bytes per block and window cell) take at most `budget` bytes
-// or the half-width is 1.  Narrower windows only make more movers far ones.
-int table_window(const Geo& g, Blk bk, size_t budget) {
-  while (bk.D > 1 && table_bytes(g, bk) > budget) --bk.D;
-  return bk.D;
-}
+// Start tables: 8 bytes per block and window cell.
 size_t table_bytes(const Geo& g, const Blk& bk) {
   return (size_t)bk.nbx * bk.nby * bk.nbz * 2 * (size_t)window_cells(g, bk) * 4;
 }

@@ -18,7 +18,7 @@ struct Geo {
 struct Blk {
   int RX, RY, RZ;     // cells per block along x, y, z
   int nbx, nby, nbz;  // blocks along x, y, z
-  int D;              // half-width (cells) of the new-cell histogram window
+  int D;              // half-width (cells) of the new-cell histogram window; -1: no window
   int brick;          // blocks are handed out in bricks of brick x brick (y, z) block rows (1: row order)
   int* work;          // persistent launch: device counter of cell blocks taken (zeroed before the launch); null: one CTA per block
 };
@@ -92,13 +92,12 @@ struct RecompressTables {
   uint32_t* counts1;
   uint32_t* far0;
   uint32_t* far1;
-  uint32_t* start;   // null: no particles
+  uint32_t* start;   // null: no window (half-width -1)
   int kb;            // rank bits of a key (set by the launchers)
 };
 size_t table_bytes(const Geo& g, const Blk& bk);
 constexpr int kKickRowCells = 32;
 Blk kick_blocks(const Geo& g, Blk bk, int64_t particles);
-int table_window(const Geo& g, Blk bk, size_t budget);
 // Brick edge (block rows) of the block order for a block grid (1: row order).
 int block_brick(const Blk& bk);
 cudaError_t launch_deposit_codes(const PCodes& c0, const PCodes& c1, const int64_t* off0, const int64_t* off1,
