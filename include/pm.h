@@ -495,7 +495,10 @@ int pm_set_tuning(pm_handle_t* h, const pm_tuning_t* t);
  * fastest and writes it to *chosen (may be NULL).  It writes `out` (any
  * earlier content is lost) and never `in`; blocks the calling thread until
  * the timing is done.  Per-stage timing and step graphs are suspended while
- * it runs.  On error the previous tuning is restored. */
+ * it runs.  Kick shapes whose tables exceed their bound or the free memory are no
+ * candidates; beside the tables held before, those of one candidate at a time
+ * take memory, and afterwards those of the shape kept.  On error the previous
+ * tuning is restored. */
 int pm_autotune(pm_handle_t* h, const pm_codes_t in[2], pm_codes_t out[2], double c_kick, double c_drift, int32_t reps,
                 void* stream, pm_tuning_t* chosen);
 

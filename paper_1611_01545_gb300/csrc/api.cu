@@ -980,7 +980,8 @@ void drop_graphs(pm_handle* h) {
   h->step_graphs.clear();
 }
 
-int apply_tuning(pm_handle* h, const pm_tuning_t* t) {
+// Checks a tuning and takes its shapes; the start tables stay as they are.
+int take_shapes(pm_handle* h, const pm_tuning_t* t) {
   const Blk bd = make_blk(h, t->deposit_block, 2);
   const Blk bi = make_blk(h, t->kick_block, t->kick_window);
   if (!blk_fits(h, bd, true)) return fail(h, PM_ERR_ARG, "deposit_block does not tile the mesh or exceeds shared memory");
@@ -989,7 +990,6 @@ int apply_tuning(pm_handle* h, const pm_tuning_t* t) {
     return fail(h, PM_ERR_ARG, "tile_batch must lie in [1, the configured tile batch]");
   if ((t->deposit_persistent & ~1) || (t->kick_persistent & ~1)) return fail(h, PM_ERR_ARG, "persistent flags are 0 or 1");
   drop_graphs(h);
-  reserve_tables(h, bi);
   h->blk_dep = bd;
   h->blk_ikd = bi;
   h->persist_dep = t->deposit_persistent != 0;
@@ -997,6 +997,48 @@ int apply_tuning(pm_handle* h, const pm_tuning_t* t) {
   if (h->gm.two) h->plan_tiles.batch = t->tile_batch;
   return PM_OK;
 }
+
+int apply_tuning(pm_handle* h, const pm_tuning_t* t) {
+  const int r = take_shapes(h, t);
+  if (r == PM_OK) reserve_tables(h, h->blk_ikd);
+  return r;
+}
+
+// Start tables during a search over tunings: the table held on entry, or one larger
+// one on trial in its place.  The search launches its steps directly and waits for
+// them, so no graph holds the address of a table on trial, and it can be freed.
+class TableTrial {
+ public:
+  explicit TableTrial(pm_handle* h) : h_(h), entry_(h->start), entry_bytes_(h->start_bytes) {}
+  // Whether the passes would run kick block b with its own window; makes room for it.
+  bool has_room(const Blk& b) {
+    const Blk w = window_within(h_, b, SIZE_MAX);
+    if (w.D != b.D) return false;
+    const size_t need = table_bytes(h_->geo, w);
+    if (need <= h_->start_bytes) return true;
+    drop();
+    if (need <= h_->start_bytes) return true;
+    void* p = nullptr;
+    if (cudaMalloc(&p, need) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    h_->start = static_cast<uint32_t*>(p);
+    h_->start_bytes = need;
+    return true;
+  }
+  // Back to the table held on entry.
+  void drop() {
+    if (h_->start != entry_) cudaFree(h_->start);
+    h_->start = entry_;
+    h_->start_bytes = entry_bytes_;
+  }
+
+ private:
+  pm_handle* h_;
+  uint32_t* entry_;
+  size_t entry_bytes_;
+};
 }  // namespace
 
 int pm_get_tuning(const pm_handle_t* h, pm_tuning_t* t) {
@@ -1033,7 +1075,12 @@ int pm_autotune(pm_handle_t* h, const pm_codes_t in[2], pm_codes_t out[2], doubl
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   int rc = PM_OK;
   float best_ms = 0.f;
-  auto restore = [&](int code) {
+  TableTrial trial(h);
+  // ends the search with tuning t
+  auto finish = [&](int code, const pm_tuning_t& t) {
+    cudaStreamSynchronize(st);   // (after an error steps may still run)
+    trial.drop();
+    apply_tuning(h, &t);
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     h->timer.on = timing;
@@ -1041,10 +1088,10 @@ int pm_autotune(pm_handle_t* h, const pm_codes_t in[2], pm_codes_t out[2], doubl
     return code;
   };
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
-    return restore(fail(h, PM_ERR_CUDA, "event create"));
+    return finish(fail(h, PM_ERR_CUDA, "event create"), start);
   // mean step time of a tuning: one untimed step, then reps steps between events
   auto time_of = [&](const pm_tuning_t& t, float* ms) -> int {
-    if (int r = apply_tuning(h, &t)) return r;
+    if (int r = take_shapes(h, &t)) return r;
     if (int r = step_launch(h, in, out, c_kick, c_drift, st)) return r;
     if (cudaEventRecord(e0, st) != cudaSuccess) return fail(h, PM_ERR_CUDA, "event record");
     for (int i = 0; i < reps; ++i)
@@ -1055,13 +1102,16 @@ int pm_autotune(pm_handle_t* h, const pm_codes_t in[2], pm_codes_t out[2], doubl
     *ms /= (float)reps;
     return PM_OK;
   };
-  if ((rc = time_of(best, &best_ms))) {
-    apply_tuning(h, &start);
-    return restore(rc);
-  }
+  if ((rc = time_of(best, &best_ms))) return finish(rc, start);
+  const Blk entry_kick = h->blk_ikd;
   auto consider = [&](const pm_tuning_t& t) -> int {
     const Blk bd = make_blk(h, t.deposit_block, 2), bi = make_blk(h, t.kick_block, t.kick_window);
     if (!blk_fits(h, bd, true) || !blk_fits(h, bi, false)) return PM_OK;   // not a candidate on this mesh
+    // nor is a kick shape that would run with a narrower window than its own (the
+    // shape on entry runs as it did)
+    const bool entry = bi.RX == entry_kick.RX && bi.RY == entry_kick.RY && bi.RZ == entry_kick.RZ && bi.D == entry_kick.D;
+    if (entry) trial.drop();
+    else if (!trial.has_room(bi)) return PM_OK;
     float ms = 0.f;
     if (int r = time_of(t, &ms)) return r;
     if (ms < best_ms) {
@@ -1100,13 +1150,9 @@ int pm_autotune(pm_handle_t* h, const pm_codes_t in[2], pm_codes_t out[2], doubl
     t.tile_batch = h->tile_batch_alloc / k > 0 ? h->tile_batch_alloc / k : 1;
     rc = consider(t);
   }
-  if (rc != PM_OK) {
-    apply_tuning(h, &start);
-    return restore(rc);
-  }
-  apply_tuning(h, &best);
+  if (rc != PM_OK) return finish(rc, start);
   if (chosen) *chosen = best;
-  return restore(PM_OK);
+  return finish(PM_OK, best);
 }
 
 int pm_step(pm_handle_t* h, const pm_codes_t in[2], pm_codes_t out[2], double c_kick, double c_drift, void* stream) {

@@ -1,6 +1,7 @@
-"""Memory of the recompress passes' start tables: a mesh with few particles does not
-take tables larger than its bound, and a handle with no room for them still
-steps, with the codes that the oracle gives."""
+"""Memory of the recompress passes' start tables: the autotuner gives back what
+its candidates took and never picks a shape whose tables cannot be had, a mesh
+with few particles does not take tables larger than its bound, and a handle
+with no room for them still steps, with the codes that the oracle gives."""
 import numpy as np
 import pytest
 import torch
@@ -52,6 +53,43 @@ def _free():
     torch.cuda.synchronize()
     torch.cuda.empty_cache()
     return torch.cuda.mem_get_info()[0]
+
+
+def _table(n_cmp, tuning):
+    """Bytes of the tables of a tuning: a word per block, species and window cell."""
+    window = blocks = 1
+    for r in tuning["kick_block"]:
+        window *= min(r + 2 * tuning["kick_window"], n_cmp)
+        blocks *= n_cmp // r
+    return 8 * window * blocks
+
+
+def test_autotune_gives_its_tables_back():
+    from paper_1611_01545_gb300 import PM
+    n, counts = 256, (3000, 60000)
+    codes = _codes(n, 4, counts, 1)
+    cfg = _cfg(n, 4, 64, 16, counts)
+    pm = PM(cfg)
+    din = [lib_codes_from_oracle(c) for c in codes]
+    dout = [pm.empty_codes(c.n, esc_cap=64) for c in codes]
+    pm.step(din, dout, 0.0, 1.0)
+    before = _free()
+    chosen = pm.autotune(din, dout, 0.0, 1.0, reps=1)
+    # beside the chosen shape's tables only what the kernels used for the first time take to load
+    assert before - _free() <= _table(n // 4, chosen) + 48 * MB
+    _drift_matches(pm, codes, n, 4)
+    pm.close()
+    # with 40 MB left, shapes whose tables exceed that and what pm_init reserved are no candidates
+    pm = PM(cfg)
+    held = _table(n // 4, pm.get_tuning())
+    pm.step(din, dout, 0.0, 1.0)
+    filler = torch.empty(_free() - 40 * MB, dtype=torch.uint8, device="cuda")
+    for _ in range(5):
+        chosen = pm.autotune(din, dout, 0.0, 1.0, reps=1)
+        assert _table(n // 4, chosen) <= held + 40 * MB
+    del filler
+    torch.cuda.empty_cache()
+    _drift_matches(pm, codes, n, 4)
 
 
 def test_tables_of_a_sparse_mesh_are_bounded():
