@@ -149,8 +149,13 @@ struct WarpBox {
 __device__ __forceinline__ int box_cap(int count) { return 4 * count < kBoxCells ? 4 * count : kBoxCells; }
 
 // Box of the particles first .. first + count - 1 (count > 0), the same on every lane.
+// FINITE: a group with a coordinate that is no number has none, because its corner
+// terms are no numbers either, which integer bins cannot hold and the mesh has to
+// show (float bins can).
+template <bool FINITE>
 __device__ __forceinline__ WarpBox warp_box(const float* x, int64_t first, int count, int nf, int cap) {
   int lo[3] = {INT_MAX, INT_MAX, INT_MAX}, hi[3] = {INT_MIN, INT_MIN, INT_MIN};
+  float odd = 0.f;   // 0 x summed over the coordinates: 0, or NaN
   // the first 32 particles, then (unless their box is too large already: a
   // random order is found out after 1 / PER of the work) the others
   for (int part = 0; part < 2; ++part) {
@@ -159,7 +164,9 @@ __device__ __forceinline__ WarpBox warp_box(const float* x, int64_t first, int c
     for (int k = from + (threadIdx.x & 31); k < to; k += 32) {
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
-        int i0 = (int)floorf(x[3 * (first + k) + d]);
+        const float xd = x[3 * (first + k) + d];
+        if (FINITE) odd = __fmaf_rn(xd, 0.f, odd);
+        int i0 = (int)floorf(xd);
         if (i0 >= nf) i0 -= nf;
         if (i0 < 0) i0 += nf;
         lo[d] = min(lo[d], i0);
@@ -174,6 +181,7 @@ __device__ __forceinline__ WarpBox warp_box(const float* x, int64_t first, int c
     if ((float)(hi[0] - lo[0] + 2) * (float)(hi[1] - lo[1] + 2) * (float)(hi[2] - lo[2] + 2) > (float)cap) break;
   }
   WarpBox b{lo[0], lo[1], lo[2], 0, 0, 0, false};
+  if (FINITE && __any_sync(0xffffffffu, odd != 0.f)) return b;
   // extents are checked one by one, so that no product overflows
   const long long e0 = (long long)hi[0] - lo[0] + 2, e1 = (long long)hi[1] - lo[1] + 2,
                   e2 = (long long)hi[2] - lo[2] + 2;
@@ -191,7 +199,7 @@ __device__ __forceinline__ WarpBox warp_box(const float* x, int64_t first, int c
 // shared memory take 402 us in place of 339 for the neutrinos above).  int64: the
 // term itself (the caller bounds the mass so that neither word overflows).
 // float32: the term in units of 2^-16 / scale, scale a power of two such that
-// the mass of a whole group stays below 2^30 / scale: finer than 2^-38 of the
+// the mass of a whole group stays below 2^30 / scale: at most 2^-37 of the
 // particle mass, so the bins add no error of their own (one 32-bit word in
 // units of 2^-22 of the mass raised the acceleration error of the sparse
 // species from 1.0e-6 to 2.5e-6).
@@ -328,7 +336,7 @@ __global__ void __launch_bounds__(kDepThreads) k_deposit(const float* x, int64_t
   for (int64_t gr = (int64_t)blockIdx.x * kDepWarps + (threadIdx.x >> 5); gr < groups; gr += warps) {
     const int64_t first = gr * kGroup;
     const int count = n - first < kGroup ? (int)(n - first) : kGroup;
-    WarpBox b = warp_box(x, first, count, g.nf, box_cap(count));
+    WarpBox b = warp_box<true>(x, first, count, g.nf, box_cap(count));
     b.fits = b.fits && scale != 0.f;
     if (b.fits) {
       const int vol = b.ex * b.ey * b.ez;
@@ -423,7 +431,7 @@ __global__ void __launch_bounds__(kDepThreads) k_deposit_weights(const float* x,
   for (int64_t gr = (int64_t)blockIdx.x * kDepWarps + (threadIdx.x >> 5); gr < groups; gr += warps) {
     const int64_t first = gr * kGroup;
     const int count = n - first < kGroup ? (int)(n - first) : kGroup;
-    const WarpBox b = warp_box(x, first, count, g.nf, box_cap(count));
+    const WarpBox b = warp_box<false>(x, first, count, g.nf, box_cap(count));
     if (!b.fits) {
       for (int k = lane; k < count; k += 32) {
         const float* xp = x + 3 * (first + k);

@@ -1,0 +1,45 @@
+"""Float particles outside the ordinary: a position that is no number shows in the
+density, wherever its neighbours are."""
+import pytest
+import torch
+
+from synth.generators import FOUR_PI_G_ONE
+
+pytestmark = pytest.mark.gpu
+
+
+def _pm(n, two=False):
+    from paper_1611_01545_gb300 import PM
+    cfg = dict(n_fine=n, coarse_ratio=1, tile=n, buffer=0, cmp_ratio=4, vel_bits=16, G=FOUR_PI_G_ONE, mass=(8.0, 0.04),
+               count=(0, 0))
+    if two:
+        cfg.update(coarse_ratio=4, tile=16 if n == 64 else 64, buffer=8 if n == 64 else 16, r_split=6.0 / 4.5, r_cut=6.0)
+    return PM(cfg)
+
+
+# groups whose box lies at node 0 of the axis, at another node, and in both group sizes
+@pytest.mark.parametrize("axis", [0, 1, 2])
+@pytest.mark.parametrize("at", [0, 20])
+@pytest.mark.parametrize("count", [40, 2490401])
+def test_a_position_that_is_no_number_shows(axis, at, count):
+    n = 64
+    pm = _pm(n, two=True)
+    x = torch.rand((count, 3), generator=torch.Generator(device="cuda").manual_seed(at), device="cuda") * 2.0 + at
+    rc0, rf0 = pm.zeros_meshes()
+    pm.deposit(0, torch.cat([x[:17], x[18:]]), rc0, rf0)
+    x[17, axis] = float("nan")
+    rc, rf = pm.zeros_meshes()
+    pm.deposit(0, x, rc, rf)
+    w = torch.ones((count, 1), device="cuda")
+    f = pm.deposit_weights(x, w)[0]
+    pm.check()
+    # the eight corners of that particle: nodes 0 and 1 along the axis that is no number
+    for mesh, edge, ratio in ((rf, n, 1), (rc, n // 4, 4), (f, n, 1)):
+        want = torch.zeros((edge,) * 3, dtype=torch.bool, device="cuda")
+        base = [0 if d == axis else int(x[17, d] / ratio) for d in range(3)]
+        want[base[2]:base[2] + 2, base[1]:base[1] + 2, base[0]:base[0] + 2] = True
+        assert torch.equal(torch.isnan(mesh), want)
+    # everything else as without it (float32 sums of `count` corners in another order)
+    for mesh, ref in ((rf, rf0), (rc, rc0)):
+        ok = ~torch.isnan(mesh)
+        assert torch.allclose(mesh[ok], ref[ok], rtol=1e-4, atol=1e-4 * float(ref.max()))
