@@ -275,7 +275,13 @@ int pm_solve_fixed(pm_handle_t* h, const int64_t* rho_coarse, const int64_t* rho
                    float* acc_fine, void* stream);
 
 /* CIC force interpolation: a [n][3] = coarse CIC gather (positions /
- * coarse_ratio) + fine CIC gather, at device positions x [n][3]. */
+ * coarse_ratio) + fine CIC gather, at device positions x [n][3].
+ * Device memory: where 2 n >= n_fine^3 and 16 n_fine^3 bytes are at most 512 MB,
+ * this call, pm_kick_drift, pm_interpolate_adjoint and the reverse steps copy
+ * the fine mesh into a buffer of that size (one per call in flight, allocated
+ * and freed on `stream`) and read that; where it cannot be had they read the
+ * mesh, with the same result.  Up to 512 MB of it stay with the handle between
+ * calls, until pm_destroy. */
 int pm_interpolate(pm_handle_t* h, const float* x, int64_t n, const float* acc_coarse,
                    const float* acc_fine, float* a, void* stream);
 

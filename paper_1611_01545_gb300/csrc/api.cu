@@ -56,7 +56,7 @@ struct pm_handle {
   std::vector<void*> allocs;
   // stream-ordered pool of the interleaved force meshes: a buffer belongs to one
   // call on one stream, so calls on several streams or threads get their own;
-  // memory stays with the handle between calls and goes with it
+  // at most kMesh4Bytes stay with the handle between calls and go with it
   cudaMemPool_t pool = nullptr;
   Timer timer;
   // adjoint workspace (single mesh): lam_acc float4 [n^3], component spectra [3][N][N][N/2+1]
@@ -360,10 +360,11 @@ PCodesOut oview(const pm_codes_t& c, bool vel16) {
 
 // Interleaved copy of the acceleration mesh for a gather of n particles, or null
 // where it does not pay (fewer particles than half the nodes), would take more
-// than 512 MB, or cannot be had.  release_mesh4 gives it back, in stream order.
+// than kMesh4Bytes, or cannot be had.  release_mesh4 gives it back, in stream order.
+constexpr int64_t kMesh4Bytes = (int64_t)512 << 20;
 const float4* interleaved_mesh(pm_handle* h, const float* acc, int64_t n, cudaStream_t st) {
   const int64_t nodes = h->gm.nfine3();
-  if (!h->pool || 2 * n < nodes || nodes * 16 > ((int64_t)512 << 20)) return nullptr;
+  if (!h->pool || 2 * n < nodes || nodes * 16 > kMesh4Bytes) return nullptr;
   void* p = nullptr;
   if (cudaMallocFromPoolAsync(&p, (size_t)nodes * 16, h->pool, st) != cudaSuccess) {
     cudaGetLastError();
@@ -604,7 +605,7 @@ int pm_init(const pm_config_t* cfg, pm_handle_t** out) {
     props.allocType = cudaMemAllocationTypePinned;
     props.location.type = cudaMemLocationTypeDevice;
     props.location.id = h->device;
-    uint64_t keep = UINT64_MAX;
+    uint64_t keep = kMesh4Bytes;   // what stays with the handle once the calls on the device have ended
     if (cudaMemPoolCreate(&h->pool, &props) != cudaSuccess ||
         cudaMemPoolSetAttribute(h->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
       cudaGetLastError();   // without a pool the gathers read the mesh as it is
