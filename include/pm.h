@@ -279,9 +279,9 @@ int pm_solve_fixed(pm_handle_t* h, const int64_t* rho_coarse, const int64_t* rho
  * Device memory: where 2 n >= n_fine^3 and 16 n_fine^3 bytes are at most 512 MB,
  * this call, pm_kick_drift, pm_interpolate_adjoint and the reverse steps copy
  * the fine mesh into a buffer of that size (one per call in flight, allocated
- * and freed on `stream`) and read that; where it cannot be had they read the
- * mesh, with the same result.  Up to 512 MB of it stay with the handle between
- * calls, until pm_destroy. */
+ * and freed on `stream`) and read that; where it cannot be had, or `stream` is
+ * being captured, they read the mesh, with the same result.  Up to 512 MB of
+ * it stay with the handle between calls, until pm_destroy. */
 int pm_interpolate(pm_handle_t* h, const float* x, int64_t n, const float* acc_coarse,
                    const float* acc_fine, float* a, void* stream);
 

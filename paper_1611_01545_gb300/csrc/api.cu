@@ -358,28 +358,47 @@ PCodesOut oview(const pm_codes_t& c, bool vel16) {
   return PCodesOut{reinterpret_cast<uint32_t*>(c.pos), c.vel, c.vmax, vel16};
 }
 
-// Interleaved copy of the acceleration mesh for a gather of n particles, or null
-// where it does not pay (fewer particles than half the nodes), would take more
-// than kMesh4Bytes, or cannot be had.  release_mesh4 gives it back, in stream order.
+// Interleaved copy of the acceleration mesh for a gather of n particles, given back
+// in stream order when it goes out of scope.  There is none (get() is null, the gather
+// reads the mesh as it is, with the same result) where it does not pay (fewer particles
+// than half the nodes), would take more than kMesh4Bytes, cannot be had, or where the
+// stream is being captured: an allocation in the caller's graph would hold memory of
+// its own and bar the graph from being cloned or instantiated twice.
 constexpr int64_t kMesh4Bytes = (int64_t)512 << 20;
-const float4* interleaved_mesh(pm_handle* h, const float* acc, int64_t n, cudaStream_t st) {
-  const int64_t nodes = h->gm.nfine3();
-  if (!h->pool || 2 * n < nodes || nodes * 16 > kMesh4Bytes) return nullptr;
-  void* p = nullptr;
-  if (cudaMallocFromPoolAsync(&p, (size_t)nodes * 16, h->pool, st) != cudaSuccess) {
-    cudaGetLastError();
-    return nullptr;
+class InterleavedMesh {
+ public:
+  InterleavedMesh(pm_handle* h, const float* acc, int64_t n, cudaStream_t st) : st_(st) {
+    const int64_t nodes = h->gm.nfine3();
+    if (!h->pool || 2 * n < nodes || nodes * 16 > kMesh4Bytes) return;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
+      cudaGetLastError();
+      return;
+    }
+    void* p = nullptr;
+    if (cudaMallocFromPoolAsync(&p, (size_t)nodes * 16, h->pool, st) != cudaSuccess) {
+      cudaGetLastError();
+      return;
+    }
+    mesh_ = static_cast<float4*>(p);
+    if (launch_interleave(acc, nodes, mesh_, st) != cudaSuccess) {
+      cudaGetLastError();
+      release();
+    }
   }
-  if (launch_interleave(acc, nodes, static_cast<float4*>(p), st) != cudaSuccess) {
-    cudaGetLastError();
-    cudaFreeAsync(p, st);
-    return nullptr;
+  ~InterleavedMesh() { release(); }
+  InterleavedMesh(const InterleavedMesh&) = delete;
+  InterleavedMesh& operator=(const InterleavedMesh&) = delete;
+  const float4* get() const { return mesh_; }
+
+ private:
+  void release() {
+    if (mesh_ && cudaFreeAsync(mesh_, st_) != cudaSuccess) cudaGetLastError();
+    mesh_ = nullptr;
   }
-  return static_cast<const float4*>(p);
-}
-cudaError_t release_mesh4(const float4* p, cudaStream_t st) {
-  return p ? cudaFreeAsync(const_cast<float4*>(p), st) : cudaSuccess;
-}
+  cudaStream_t st_;
+  float4* mesh_ = nullptr;
+};
 
 int check_species(pm_handle* h, int s) {
   if (s < 0 || s > 1) return fail(h, PM_ERR_ARG, "species must be 0 or 1");
@@ -863,9 +882,8 @@ int pm_interpolate(pm_handle_t* h, const float* x, int64_t n, const float* acc_c
                    void* stream) {
   if (!h || (n && (!x || !a)) || !acc_fine || (h->gm.two && !acc_coarse)) return fail(h, PM_ERR_ARG, "null argument");
   cudaStream_t st = (cudaStream_t)stream;
-  const float4* acc4 = interleaved_mesh(h, acc_fine, n, st);
-  CK(h, launch_interpolate(x, n, h->geo, acc_coarse, acc_fine, acc4, a, st));
-  CK(h, release_mesh4(acc4, st));
+  const InterleavedMesh acc4(h, acc_fine, n, st);
+  CK(h, launch_interpolate(x, n, h->geo, acc_coarse, acc_fine, acc4.get(), a, st));
   return PM_OK;
 }
 
@@ -873,9 +891,8 @@ int pm_kick_drift(pm_handle_t* h, float* x, float* v, int64_t n, const float* ac
                   double c_kick, double c_drift, void* stream) {
   if (!h || (n && (!x || !v)) || !acc_fine || (h->gm.two && !acc_coarse)) return fail(h, PM_ERR_ARG, "null argument");
   cudaStream_t st = (cudaStream_t)stream;
-  const float4* acc4 = interleaved_mesh(h, acc_fine, n, st);
-  CK(h, launch_kick_drift(x, v, n, h->geo, acc_coarse, acc_fine, acc4, (float)c_kick, (float)c_drift, st));
-  CK(h, release_mesh4(acc4, st));
+  const InterleavedMesh acc4(h, acc_fine, n, st);
+  CK(h, launch_kick_drift(x, v, n, h->geo, acc_coarse, acc_fine, acc4.get(), (float)c_kick, (float)c_drift, st));
   return PM_OK;
 }
 
@@ -1262,10 +1279,9 @@ int pm_interpolate_adjoint(pm_handle_t* h, const float* x, int64_t n, const floa
   if (!h || (n && (!x || !lam_x || !lam_v)) || !acc_fine || !lam_acc) return fail(h, PM_ERR_ARG, "null argument");
   if (h->gm.two) return fail(h, PM_ERR_CONFIG, "adjoints are implemented for the single periodic mesh");
   cudaStream_t st = (cudaStream_t)stream;
-  const float4* acc4 = interleaved_mesh(h, acc_fine, n, st);
-  CK(h, launch_adj_interp(x, n, h->gm.nf, acc_fine, acc4, (float)c_kick, (float)c_drift, lam_x, lam_v, lam_acc, false,
-                          st));
-  CK(h, release_mesh4(acc4, st));
+  const InterleavedMesh acc4(h, acc_fine, n, st);
+  CK(h, launch_adj_interp(x, n, h->gm.nf, acc_fine, acc4.get(), (float)c_kick, (float)c_drift, lam_x, lam_v, lam_acc,
+                          false, st));
   return PM_OK;
 }
 
@@ -1276,11 +1292,12 @@ static int step_adjoint_core(pm_handle_t* h, const pm_particles_t state[2], pm_p
   const size_t nf3 = (size_t)g.nfine3();
   // interleaved float4 accumulation mesh: one vector reduction per CIC corner
   CK(h, cudaMemsetAsync(h->lam_acc, 0, 4 * nf3 * 4, st));
-  const float4* acc4 = interleaved_mesh(h, acc, state[0].n + state[1].n, st);
-  for (int s = 0; s < 2; ++s)
-    CK(h, launch_adj_interp(state[s].x, state[s].n, g.nf, acc, acc4, (float)c_kick, (float)c_drift, lam[s].x, lam[s].v,
-                            h->lam_acc, true, st));
-  CK(h, release_mesh4(acc4, st));
+  {
+    const InterleavedMesh acc4(h, acc, state[0].n + state[1].n, st);
+    for (int s = 0; s < 2; ++s)
+      CK(h, launch_adj_interp(state[s].x, state[s].n, g.nf, acc, acc4.get(), (float)c_kick, (float)c_drift, lam[s].x,
+                              lam[s].v, h->lam_acc, true, st));
+  }
   CK(h, solve_adjoint_launch(h->plan_mesh, h->lam_acc, true, h->rho_f, h->adj_spec, st));   // rho_f holds lam_rho
   for (int s = 0; s < 2; ++s)
     CK(h, launch_adj_deposit(state[s].x, state[s].n, (float)h->cfg.mass[s], g.nf, h->rho_f, lam[s].x, st));
