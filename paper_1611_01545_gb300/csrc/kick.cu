@@ -812,6 +812,10 @@ size_t kick_count_smem(const Geo& g, const Blk& bk) {
          3 * ((size_t)st.comp + coarse) * sizeof(float);
 }
 
+// Shared memory per block that a shape may need to be accepted (pm_set_tuning), in
+// terms of the general kernels: offsets, and 12 bytes per window cell and species for
+// the scatter.  The scatter takes less, 8 bytes per window cell, and the row form of
+// the count pass at most 127 KB.
 size_t kick_scatter_smem(const Geo& g, const Blk& bk) {
   size_t nrow = (size_t)bk.RY * bk.RZ;
   return 2 * nrow * (bk.RX + 1) * sizeof(int64_t) + 2 * (size_t)window_cells(g, bk) * (8 + 4);

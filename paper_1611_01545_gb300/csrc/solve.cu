@@ -51,7 +51,6 @@ template <int N> struct SolveCfg {
 
 struct SolveArgs {
   const void* src;
-  int src_fixed;
   int src_n;
   int nts;
   int t, b;
@@ -91,10 +90,6 @@ __device__ __forceinline__ void async_copy4(void* smem_dst, const void* gmem_src
 }
 __device__ __forceinline__ void async_copy8(void* smem_dst, const void* gmem_src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"((unsigned)__cvta_generic_to_shared(smem_dst)),
-               "l"(gmem_src) : "memory");
-}
-__device__ __forceinline__ void async_copy16(void* smem_dst, const void* gmem_src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(smem_dst)),
                "l"(gmem_src) : "memory");
 }
 __device__ __forceinline__ void async_wait() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
@@ -231,23 +226,21 @@ __global__ void __launch_bounds__(PassB<N>::threads) k_solve_b_adj(SolveArgs a) 
   }
 }
 
-// ---- 96^3 passes staged by the tensor memory accelerator ----------------
+// ---- copies by the tensor memory accelerator ---------------------------------
 //
-// The 96^3 transforms (the buffered fine tiles, and a 96^3 periodic mesh)
-// move their shared-memory pencils with TMA bulk copies instead of
-// per-thread copies:
-//   A  the window plane arrives as 36 boxes of 16 x 16 cells (a tensor map
-//      of the source mesh; window origins are multiples of 16 cells, so no
-//      box crosses the periodic boundary), is repacked into two-row complex
-//      rows and transformed as before; the half-spectrum plane leaves as one
+// Where the shapes allow it, planes and pencils move between global and shared
+// memory as TMA bulk copies instead of per-thread copies:
+//   A  96^3 windows of float meshes on 16-cell boundaries arrive as 36 boxes of
+//      16 x 16 cells (a tensor map of the source mesh; window origins are multiples
+//      of 16 cells, so no box crosses the periodic boundary), from which the first
+//      transform step reads; at every size the half-spectrum plane leaves as one
 //      bulk store;
-//   B  the z pencils of KT = 26 kx columns arrive as one 52 x 1 x 96 box of
-//      the spectrum (columns past kx = N/2 read as zeros); the second step of
-//      the forward z transform, the three kernel products and the first step
-//      of each inverse transform run in registers per (column, k1) item; the
-//      output z range of each component leaves as one box store;
-// Spectrum rows are padded to spec_pitch(96) = 50 complex values (400
-// bytes), so rows, boxes and planes start on 16-byte boundaries.
+//   B  at 96 the z pencils of 18 kx columns arrive as one box of 36 floats x 1 x 96
+//      of the spectrum (columns past kx = N / 2 read as zeros); the output rows are
+//      written from registers;
+//   C  at every size the plane arrives as one bulk load.
+// The spectrum rows between A and B are padded to spec_pitch(96) = 50 complex values
+// (400 bytes), so rows, boxes and planes start on 16-byte boundaries.
 
 constexpr int kTmaAlign = 128;   // shared-memory alignment of every TMA destination and source
 constexpr int kBox = 16;         // edge (cells) of the pass-A window boxes
@@ -1055,7 +1048,7 @@ static cudaError_t solve_large_n(const SolvePlan& p, const void* src, bool fixed
     cudaFuncSetAttribute(k_large_cx<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::smem_cx);
     attr_done = true;
   }
-  SolveArgs a{src, fixed ? 1 : 0, N, 1, N, 0, 0, p.spec, p.spec3, p.kern, p.kern_quads, p.tw, dst, 0, amax, nullptr, 0, 1, p.status};
+  SolveArgs a{src, N, 1, N, 0, 0, p.spec, p.spec3, p.kern, p.kern_quads, p.tw, dst, 0, amax, nullptr, 0, 1, p.status};
   {
     TimedScope ts(tm, "fft_a_mesh", st);
     if (fixed) k_large_ax<N, true><<<dim3(N / L::R, N), L::threads, L::smem_ax, st>>>(a);
@@ -1166,7 +1159,7 @@ static cudaError_t solve_n(const SolvePlan& p, const void* src, bool fixed, floa
   const int nprob = p.nts * p.nts * p.nts;
   for (int p0 = 0; p0 < nprob; p0 += p.batch) {
     int nb = (nprob - p0 < p.batch) ? (nprob - p0) : p.batch;
-    SolveArgs a{src, fixed ? 1 : 0, p.src_n, p.nts, p.t, p.b, p0, p.spec, p.spec3, p.kern, p.kern_quads, p.tw, dst, 0, amax,
+    SolveArgs a{src, p.src_n, p.nts, p.t, p.b, p0, p.spec, p.spec3, p.kern, p.kern_quads, p.tw, dst, 0, amax,
                 pro ? pro->coarse : nullptr, pro ? pro->nc : 0, pro ? pro->rc : 1, p.status};
     {
       TimedScope ts(tm, N == p.src_n && p.b == 0 ? "fft_a_mesh" : "fft_a_tiles", st);
@@ -1227,7 +1220,7 @@ static cudaError_t solve_adjoint_n(const SolvePlan& p, const float* lam_acc, boo
   cudaFuncSetAttribute(ka, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassA<N>::smem);
   cudaFuncSetAttribute(k_solve_b_adj<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(float2) * (N + 2 * (size_t)N * PassB<N>::KC)));
   cudaFuncSetAttribute(k_solve_c<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PassC<N>::smem_max());
-  SolveArgs a{lam_acc, 0, p.src_n, 1, N, 0, 0, spec3comp, p.spec3, p.kern, p.kern_quads, p.tw, lam_rho, 1, nullptr, nullptr, 0, 1,
+  SolveArgs a{lam_acc, p.src_n, 1, N, 0, 0, spec3comp, p.spec3, p.kern, p.kern_quads, p.tw, lam_rho, 1, nullptr, nullptr, 0, 1,
               p.status};
   ka<<<dim3(N, 3), PassA<N>::threads, PassA<N>::smem, st>>>(a, CUtensorMap{});
   a.comp_mode = 0;
