@@ -88,12 +88,11 @@ struct Win {
   int ox, oy, oz, wx, wy, wz;
 };
 __device__ __forceinline__ Win window_of(const Geo& g, const Blk& bk, CellBlock cb) {
-  if (bk.D < 0) return Win{0, 0, 0, 0, 0, 0};
   Win w;
   const int n = g.ncmp, D = bk.D;
-  w.wx = bk.RX + 2 * D < n ? bk.RX + 2 * D : n;
-  w.wy = bk.RY + 2 * D < n ? bk.RY + 2 * D : n;
-  w.wz = bk.RZ + 2 * D < n ? bk.RZ + 2 * D : n;
+  w.wx = bk.wx;
+  w.wy = bk.wy;
+  w.wz = bk.wz;
   w.ox = w.wx == n ? 0 : cb.ix0 - D;
   w.oy = w.wy == n ? 0 : cb.iy0 - D;
   w.oz = w.wz == n ? 0 : cb.iz0 - D;
@@ -826,13 +825,18 @@ int block_brick(const Blk& bk) {
   return (B > 1 && bk.nby % B == 0 && bk.nbz % B == 0 && (int64_t)bk.nby * bk.nbz >= PM_BRICK_MIN_ROWS) ? B : 1;
 }
 
-int window_cells(const Geo& g, const Blk& bk) {
+// Edge of the window along an axis on which the block has R cells.
+static int window_edge(const Geo& g, const Blk& bk, int R) {
   if (bk.D < 0) return 0;
-  const int n = g.ncmp;
-  int wx = bk.RX + 2 * bk.D < n ? bk.RX + 2 * bk.D : n;
-  int wy = bk.RY + 2 * bk.D < n ? bk.RY + 2 * bk.D : n;
-  int wz = bk.RZ + 2 * bk.D < n ? bk.RZ + 2 * bk.D : n;
-  return wx * wy * wz;
+  return R + 2 * bk.D < g.ncmp ? R + 2 * bk.D : g.ncmp;
+}
+static void set_window(const Geo& g, Blk& bk) {
+  bk.wx = window_edge(g, bk, bk.RX);
+  bk.wy = window_edge(g, bk, bk.RY);
+  bk.wz = window_edge(g, bk, bk.RZ);
+}
+int window_cells(const Geo& g, const Blk& bk) {
+  return window_edge(g, bk, bk.RX) * window_edge(g, bk, bk.RY) * window_edge(g, bk, bk.RZ);
 }
 
 
@@ -892,6 +896,7 @@ cudaError_t launch_kick_count(const PCodes& c0, const PCodes& c1, const int64_t*
                               const float* vq0, const float* vq1, const float4* app, bool coarse, cudaStream_t st) {
   KickArgs k{c0, c1, off0, off1, g, bk, acc_c, acc_f, ck, cd, t, vmax_bits, tkey, tpv, vq0, vq1, app, coarse ? 1 : 0};
   k.t.kb = rank_bits(g, bk);
+  set_window(g, k.bk);
   return c0.vel16 ? kick_count<true>(k, c0.n + c1.n, st) : kick_count<false>(k, c0.n + c1.n, st);
 }
 
@@ -901,6 +906,7 @@ cudaError_t launch_kick_scatter(int64_t n0, int64_t n1, const int64_t* off0, con
                                 const uint4* tpv, bool coded, int* status, cudaStream_t st) {
   ScatterArgs k{n0, n1, off0, off1, g, bk, t, newoff0, newoff1, o0, o1, tkey, tpv, coded ? 1 : 0, status};
   k.t.kb = rank_bits(g, bk);
+  set_window(g, k.bk);
   const size_t smem = 2 * (size_t)window_cells(g, bk) * sizeof(int64_t);
   const auto f = o0.vel16 ? k_kick_scatter<true> : k_kick_scatter<false>;
   allow_smem(f, smem);

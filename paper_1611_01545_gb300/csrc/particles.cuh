@@ -19,6 +19,7 @@ struct Blk {
   int RX, RY, RZ;     // cells per block along x, y, z
   int nbx, nby, nbz;  // blocks along x, y, z
   int D;              // half-width (cells) of the new-cell histogram window; -1: no window
+  int wx, wy, wz;     // that window's extents (set by the recompress launchers; 0: no window)
   int brick;          // blocks are handed out in bricks of brick x brick (y, z) block rows (1: row order)
   int* work;          // persistent launch: device counter of cell blocks taken (zeroed before the launch); null: one CTA per block
 };
